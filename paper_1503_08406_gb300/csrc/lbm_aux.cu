@@ -127,37 +127,99 @@ __global__ void macros_kernel(Dev d, int layout, float* ux, float* uy, float* rh
   if (fl) fl[s] = d.fl[s];
 }
 
+// lo += what hi + v loses in FP32 (Knuth's two-sum), hi = hi + v: hi + lo stays
+// the exact sum to about 2^-48 of it
+__device__ __forceinline__ void two_sum(float& hi, float& lo, float v) {
+  const float s = hi + v, t = s - hi;
+  lo += (hi - (s - t)) + (v - t);
+  hi = s;
+}
+
 // per-block FP64 partial sums in a fixed order:
 // [0] mass, [1] enthalpy, [2] sum f_l, [3] non-wall count, [4] Nusselt sum, [5] Nusselt rows
+//
+// Bound by the FP64 pipe (two lanes a clock on an SM), conversions from FP32
+// included, not by the 68 bytes it reads per node: so each node makes eight
+// FP64 operations where a plain FP64 sum of everything makes about 35.  The
+// nine deviations add up in FP32 pairs (two_sum), rho0 is counted and
+// multiplied once, f_l = 0 and 1 are counted, phi f_l is an exact FP32 pair and
+// dT / (sigma St) multiplies the sum.  (2048^2, FP32: 336 -> 121 us.)
+//
+// The mass needs no gather: in the AA layout every slot of a lattice node is
+// read by exactly one lattice node (its own, or the neighbour the population
+// streams to), so the nodes' own slots hold the sum in both layouts.  Only flow
+// walls, whose nodes hold and read populations of lattice nodes, need it.
+template <typename S>
 __global__ void __launch_bounds__(RB) reduce_kernel(Dev d, int layout, double* partials) {
   __shared__ double sh[6][RB];
   const int tid = threadIdx.x;
-  double acc[6] = {0, 0, 0, 0, 0, 0};
-  for (long long s = blockIdx.x * (long long)RB + tid; s < d.n; s += (long long)gridDim.x * RB) {
-    const int y = (int)(s / d.nx), x = (int)(s - (long long)y * d.nx);
-    if (!is_wall(d, x, y)) {
-      float f[9];
-      gather_f(d, x, y, layout, f);
-      double m = (double)d.rho0;   // stored populations are f_i - w_i rho0
-      for (int i = 0; i < 9; ++i) m += (double)f[i];
-      const double T = (double)interior_T(d, x, y, layout);
-      const double fl = (double)d.fl[s];
-      acc[0] += m;
-      // a = phi dT / (sigma(f_l) St), Eq. (38) with Eq. (7)
-      const double sr = d.sigma_var ? (double)d.sigma / ((double)d.sigma_s +
-                                                         fl * ((double)d.sigma - d.sigma_s))
-                                    : 1.0;
-      acc[1] += T + (double)d.phi[s] * (double)d.lat * sr * fl;
-      acc[2] += fl;
-      acc[3] += 1.0;
+  const int n = (int)d.n, nx = d.nx;
+  const S* F = static_cast<const S*>(d.f);
+  const S* G = static_cast<const S*>(d.g);
+  const float r0 = std::is_same<S, float>::value ? 0.f : d.wt0 * d.g_ref;
+  const float r1 = std::is_same<S, float>::value ? 0.f : d.wt1 * d.g_ref;
+  const bool gather = layout == 1 && d.flow && d.flow_walls;
+  double mass = 0, heat = 0, latent = 0, liquid = 0;
+  int count = 0, ones = 0;   // non-wall nodes, those with f_l = 1
+  for (int s = blockIdx.x * RB + tid; s < n; s += gridDim.x * RB) {
+    const int y = s / nx, x = s - y * nx;
+    if (is_wall(d, x, y)) continue;
+    float f[9], g[5];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) f[i] = Pop<S>::ld(F + i * n + s);
+    g[0] = Pop<S>::ld(G + s) + r0;
+    if (layout == 0) {
+#pragma unroll
+      for (int i = 1; i < 5; ++i) g[i] = Pop<S>::ld(G + i * n + s) + r1;
+    } else {
+      const int xm = x == 0 ? s + nx - 1 : s - 1, xp = x == nx - 1 ? s - x : s + 1;
+      const int ym = y == 0 ? n - nx + x : s - nx, yp = y == d.ny - 1 ? x : s + nx;
+      g[1] = Pop<S>::ld(G + 3 * n + xm) + r1;
+      g[2] = Pop<S>::ld(G + 4 * n + ym) + r1;
+      g[3] = Pop<S>::ld(G + n + xp) + r1;
+      g[4] = Pop<S>::ld(G + 2 * n + yp) + r1;
     }
-    if (d.wall_l && x == 0 && d.nx >= 3 && (!d.wall_b || (y > 0 && y < d.ny - 1))) {
-      const double T0 = node_T(d, 0, y, layout), T1 = node_T(d, 1, y, layout),
-                   T2 = node_T(d, 2, y, layout);
-      acc[4] += -(-3.0 * T0 + 4.0 * T1 - T2) * 0.5 * (double)d.H_over_dT;
-      acc[5] += 1.0;
+    const float fl = d.fl[s], phi = d.phi[s];
+    if (gather) gather_f(d, x, y, layout, f);
+    float hi = f[0], lo = 0.f;
+#pragma unroll
+    for (int i = 1; i < 9; ++i) two_sum(hi, lo, f[i]);
+    if (fabsf(hi) <= 1e37f) {
+      mass += (double)hi;
+      mass += (double)lo;
+    } else {   // NaN, Inf, or out of FP32's range on the way
+      for (int i = 0; i < 9; ++i) mass += (double)f[i];
+    }
+    heat += (double)(g[0] + g[1] + g[2] + g[3] + g[4]);
+    ++count;
+    // a = phi dT / (sigma(f_l) St), Eq. (38) with Eq. (7)
+    if (d.sigma_var) {
+      const double fd = (double)fl;
+      latent += (double)phi * fd * (double)d.sigma /
+                ((double)d.sigma_s + fd * ((double)d.sigma - d.sigma_s));
+      liquid += fd;
+    } else if (fl == 1.f) {
+      latent += (double)phi;
+      ++ones;
+    } else if (fl != 0.f) {
+      const float p = phi * fl;
+      latent += (double)p;
+      latent += (double)fmaf(phi, fl, -p);
+      liquid += (double)fl;
     }
   }
+  // the left wall's rows, spread over the grid
+  double nu = 0, rows = 0;
+  if (d.wall_l && nx >= 3)
+    for (int y = blockIdx.x * RB + tid; y < d.ny; y += gridDim.x * RB) {
+      if (d.wall_b && (y == 0 || y == d.ny - 1)) continue;
+      const double T0 = node_T(d, 0, y, layout), T1 = node_T(d, 1, y, layout),
+                   T2 = node_T(d, 2, y, layout);
+      nu += -(-3.0 * T0 + 4.0 * T1 - T2) * 0.5 * (double)d.H_over_dT;
+      rows += 1.0;
+    }
+  const double acc[6] = {(double)d.rho0 * count + mass, heat + (double)d.lat * latent,
+                         liquid + (double)ones, (double)count, nu, rows};
   for (int k = 0; k < 6; ++k) sh[k][tid] = acc[k];
   __syncthreads();
   for (int w = RB / 2; w > 0; w >>= 1) {
@@ -165,8 +227,7 @@ __global__ void __launch_bounds__(RB) reduce_kernel(Dev d, int layout, double* p
       for (int k = 0; k < 6; ++k) sh[k][tid] += sh[k][tid + w];
     __syncthreads();
   }
-  if (tid == 0)
-    for (int k = 0; k < 6; ++k) partials[blockIdx.x * 6 + k] = sh[k][0];
+  if (tid < 6) partials[blockIdx.x * 6 + tid] = sh[tid][0];
 }
 
 // The left-wall Nusselt number of the current state (the rows and the
@@ -191,15 +252,28 @@ __global__ void __launch_bounds__(RB) wall_nusselt_kernel(Dev d, int layout, dou
   if (tid == 0 && d.wall_l && d.nx >= 3 && y1 > y0) acc[0] += sh[0] / (double)(y1 - y0);
 }
 
-__global__ void reduce_final_kernel(const double* partials, int nblocks, double* out) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// The partial sums of all blocks, in a fixed order: each thread its share of
+// the blocks, then a tree (one thread over 1024 blocks, a serial chain of
+// loads and FP64 adds, took 366 us; this 8 us).
+__global__ void __launch_bounds__(RB) reduce_final_kernel(const double* partials, int nblocks,
+                                                          double* out) {
+  __shared__ double sh[6][RB];
+  const int tid = threadIdx.x;
   double t[6] = {0, 0, 0, 0, 0, 0};
-  for (int b = 0; b < nblocks; ++b)
+  for (int b = tid; b < nblocks; b += RB)
     for (int k = 0; k < 6; ++k) t[k] += partials[b * 6 + k];
-  out[0] = t[0];
-  out[1] = t[1];
-  out[2] = t[3] > 0 ? t[2] / t[3] : 0.0;
-  out[3] = t[5] > 0 ? t[4] / t[5] : 0.0;
+  for (int k = 0; k < 6; ++k) sh[k][tid] = t[k];
+  __syncthreads();
+  for (int w = RB / 2; w > 0; w >>= 1) {
+    if (tid < w)
+      for (int k = 0; k < 6; ++k) sh[k][tid] += sh[k][tid + w];
+    __syncthreads();
+  }
+  if (tid != 0) return;
+  out[0] = sh[0][0];
+  out[1] = sh[1][0];
+  out[2] = sh[3][0] > 0 ? sh[2][0] / sh[3][0] : 0.0;
+  out[3] = sh[5][0] > 0 ? sh[4][0] / sh[5][0] : 0.0;
 }
 
 // f (9 planes) and g (5 planes) in the natural layout; each output is optional
@@ -347,8 +421,11 @@ int reduce_blocks(const Dev& d) {
 }
 void launch_reduce(const Dev& d, int layout, double* partials, double* out, int nblocks,
                    cudaStream_t s) {
-  reduce_kernel<<<nblocks, RB, 0, s>>>(d, layout, partials);
-  reduce_final_kernel<<<1, 32, 0, s>>>(partials, nblocks, out);
+  if (d.storage == 1) reduce_kernel<__half><<<nblocks, RB, 0, s>>>(d, layout, partials);
+  else if (d.storage == 2)
+    reduce_kernel<__nv_bfloat16><<<nblocks, RB, 0, s>>>(d, layout, partials);
+  else reduce_kernel<float><<<nblocks, RB, 0, s>>>(d, layout, partials);
+  reduce_final_kernel<<<1, RB, 0, s>>>(partials, nblocks, out);
 }
 void launch_wall_nusselt(const Dev& d, int layout, double* acc, cudaStream_t s) {
   wall_nusselt_kernel<<<1, RB, 0, s>>>(d, layout, acc);

@@ -1,0 +1,65 @@
+"""The reduction's FP32-pair sums against FP64 sums of the state, on every
+storage and layout.
+"""
+import numpy as np
+import pytest
+
+import lbm_workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def P():
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_1503_08406_gb300 as P
+    return P
+
+
+@pytest.mark.parametrize("steps", [4, 5])
+@pytest.mark.parametrize("over", [{}, {"storage": "fp16"}, {"flow_walls": 1},
+                                  {"sigma_solid": 0.5}, {"T_l": 0.1}])
+def test_reduce_equals_fp64_sums_of_the_state(P, steps, over):
+    w = W.melted_cavity(77)
+    p = {**w.params, **over}
+    lat = P.Lattice(77, 77, **p)
+    lat.set_fields(w.phi, w.K, w.T0, w.fl0)
+    lat.step(steps)
+    _check_sums(lat, w, p)
+
+
+def test_reduce_beyond_fp32_range(P):
+    """Deviations whose FP32 sum overflows, not their FP64 sum."""
+    w = W.melted_cavity(40)
+    lat = P.Lattice(40, 40, **w.params)
+    lat.set_fields(w.phi, w.K, w.T0, w.fl0)
+    f, g, fl = lat.get_state()
+    f[:, 5, 5] = 3e38
+    lat.set_state(f, g, fl)
+    _check_sums(lat, w, w.params)
+
+
+def _check_sums(lat, w, p):
+    """Against the same sums of the checkpoint in FP64 (T is the FP32 sum of its
+    populations); both add at most 1e4 terms of one sign in FP64, each within
+    2^-48 of exact: 1e-12 covers it."""
+    f, g, fl = lat.get_state()
+    got = lat.reduce()
+    inside = np.zeros_like(fl, dtype=bool)
+    inside[1:-1, 1:-1] = True
+    T = g[0]
+    for i in range(1, 5):
+        T = T + g[i]
+    fl = fl.astype(np.float64)
+    sl, ss = p["sigma"], p.get("sigma_solid") or p["sigma"]
+    a = w.phi.astype(np.float32).astype(np.float64) * np.float64(np.float32(
+        p["dT"] / (p["sigma"] * p["St"]))) * np.float32(sl) / (
+            np.float32(ss) + fl * (np.float64(np.float32(sl)) - np.float32(ss)))
+    mass = (1.0 + f.astype(np.float64).sum(0))[inside].sum()
+    heat = (T.astype(np.float64) + a * fl)[inside].sum()
+    assert abs(got["mass"] - mass) <= 1e-12 * abs(mass)
+    assert abs(got["enthalpy"] - heat) <= 1e-12 * abs(heat)
+    assert abs(got["melt_frac"] - fl[inside].mean()) <= 1e-12
