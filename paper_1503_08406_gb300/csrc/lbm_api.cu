@@ -131,7 +131,7 @@ int check_params(const lbm_params* p) {
 }
 
 struct Layout {
-  size_t f, g, fl, phi, K, wallTl, flags, list, lcount, ctr, nearmap, proc, tact, scr, stats,
+  size_t f, g, fl, phi, K, wallTl, flags, nearmap, proc, list, lcount, ctr, tact, scr, stats,
       tmp, partials, sums, bad, total;
 };
 
@@ -149,12 +149,12 @@ Layout layout_of(const lbm_params* p, int nred) {
   L.phi = o; o += up(n * sizeof(float));
   L.K = o; o += up(n * sizeof(float));
   L.wallTl = o; o += up((size_t)p->ny * sizeof(float));
-  L.flags = o; o += up(2 * tiles * sizeof(int));
+  L.flags = o; o += 2 * tiles * sizeof(int);   // these three cleared together
+  L.nearmap = o; o += 2 * tiles * sizeof(int);
+  L.proc = o; o += up(o + tiles * sizeof(int)) - o;
   L.list = o; o += up(2 * tiles * sizeof(int));
   L.lcount = o; o += up(2 * sizeof(int));
   L.ctr = o; o += up(2 * sizeof(int));
-  L.nearmap = o; o += up(2 * tiles * sizeof(int));
-  L.proc = o; o += up(tiles * sizeof(int));
   L.tact = o; o += up(tiles);
   L.scr = o; o += up(n * sizeof(float2));
   L.stats = o; o += up(8 * sizeof(int));
@@ -381,11 +381,12 @@ int lbm_derived(const lbm_ctx* c, double out[8]) {
 
 int64_t lbm_steps_done(const lbm_ctx* c) { return c ? c->steps : -1; }
 
-// empty work lists and tile flags; tile status words keep old stamps, which
-// never equal a later step's stamp
+// empty work lists, and no stamps in the tile flags and status words: after a
+// reset the stamps go on from the last one of the other parity, so that a step
+// may take the stamp of one before the reset
 static int reset_lists(lbm_ctx* c) {
   const Dev& d = c->d;
-  LBM_CUDA(cudaMemsetAsync(d.flags, 0, 2 * sizeof(int) * d.ntiles, c->stream));
+  LBM_CUDA(cudaMemsetAsync(d.flags, 0, 5 * sizeof(int) * d.ntiles, c->stream));   // to proc's end
   LBM_CUDA(cudaMemsetAsync(d.lcount, 0, 2 * sizeof(int), c->stream));
   LBM_CUDA(cudaMemsetAsync(d.stats + 5, 0, sizeof(int), c->stream));
   lbm::launch_tile_activity(d, c->stream);   // f_l was just loaded
@@ -1772,7 +1773,7 @@ int lbm_adjoint_coupled(lbm_ctx* c, int objective, int64_t nsteps, int32_t check
       lbm::launch_set_state(c->d, SS, SS + 9 * n, sm);
       cudaMemcpyAsync(c->d.fl, SS + 14 * n, n * sizeof(float), cudaMemcpyDeviceToDevice, sm);
       lbm::launch_tile_activity(c->d, sm);
-      cudaMemsetAsync(c->d.flags, 0, 2 * sizeof(int) * c->d.ntiles, sm);
+      cudaMemsetAsync(c->d.flags, 0, 5 * sizeof(int) * c->d.ntiles, sm);   // to proc's end
       cudaMemsetAsync(c->d.lcount, 0, 2 * sizeof(int), sm);
       if (sm == c->cap) {
         // in a capture: the step sequence of lbm_step's graphs (the next step's

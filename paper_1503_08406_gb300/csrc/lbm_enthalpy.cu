@@ -9,14 +9,16 @@
 // enthalpy relation f_l = clamp((h - T_s)/(T_l - T_s + a), 0, 1) is solved for
 // f_l(n+1) as a fixed point.
 //
-// Work list.  The fused kernel appends every 32x32 tile that may hold a phase
-// change this step to list[parity] (a tile flag de-duplicates).  Both kernels
-// below run a fixed grid of CTAs that walk that list, so steps with no front
-// cost almost nothing.  Per-tile status words carry a step stamp (a counter the
-// fused kernel advances), so nothing needs clearing between steps.
+// Work list.  The fused kernel stamps every 32x32 tile that may hold a phase
+// change this step with the step's number (a counter it advances); tiles
+// numerous enough to make walking the stamps slow are also put on a list.  Both
+// kernels below run a fixed grid of CTAs that take the listed tiles in turn, so
+// steps with no front cost almost nothing.  Stamps and the per-tile status
+// words need no clearing between steps.
 //
 // enthalpy_solve: per listed tile, load T*, f_l(n) and a on the tile plus an
-// 8-node halo into shared memory and run red-black Gauss-Seidel sweeps; each
+// 8-node halo, list the nodes that are not clamped whatever happens around
+// them, and run red-black Gauss-Seidel sweeps over those; each
 // node update solves its own term exactly,
 //   f(x) = clamp((T*(x) + w~_0 a f_l(n) - T_s - w~_1 sum_{i>0} q(x - e_i)) / (T_l - T_s + w~_0 a), 0, 1),
 //   q = a (f - f_l(n)),
@@ -87,300 +89,357 @@ __device__ __forceinline__ bool sub_sync_or(int threads, bool v) {
   return r != 0;
 }
 
-// CTA bid of nblk (the whole grid of a single lattice's launch, a range of a
-// batched one) takes listed tiles bid, bid + nblk, ...
-template <int PAR, typename S, int EB>
-__device__ __forceinline__ void enthalpy_solve_body(const Dev& d, int bid, int nblk) {
-  const long long tr0 = trace_start(d);
-  constexpr int LAYOUT = 1 - PAR;
-  extern __shared__ float smem[];
-  float* sbase = smem;               // T* + w~0 a f_l(n) - T_s
-  float* sinv = sbase + RE * RE;     // 1 / (T_l - T_s + w~0 a); 0 on fixed nodes
-  float* sa = sinv + RE * RE;        // a; 0 on walls and outside
-  float* sfn = sa + RE * RE;         // f_l(n)
-  float* sq = sfn + RE * RE;         // a (f - f_l(n))
-  float* sf = sq + RE * RE;          // current iterate
-  __shared__ int sbox[4];            // box of the nodes the sweeps update: x0, x1, y0, y1
-  const int tid = threadIdx.x;
-  const int cnt = d.lcount[PAR];
-  const int stamp = stamp_of(d, PAR);
-  const float w0 = d.wt0, w1 = d.wt1, Ts = d.T_s, dTt = d.dTt;
-  for (int li = bid; li < cnt; li += nblk) {
-    const int tile = d.list[PAR * d.ntiles + li];
-    const int X0 = (tile % d.etx) * TE, Y0 = (tile / d.etx) * TE;
-    // a region (tile and halo) inside the wall ring needs no wrapping and holds
-    // no wall node: its loads go straight to their addresses
-    const bool inner = X0 - RH >= 1 && X0 + TE + RH <= d.nx - 1 && Y0 - RH >= 1 &&
-                       Y0 + TE + RH <= d.ny - 1;
-    if (inner) {
-      // every thread's nodes loaded in one go (all loads in flight together)
-      constexpr int NK = (RE * RE + EB - 1) / EB;
-      float fnv[NK], phv[NK], Tv[NK];
+// ---- the solve's shared-memory layout ----------------------------------------
+// A region (tile and halo) of RE x RE nodes inside a ring of one, split by
+// colour: node (lx, ly) of colour c = (lx + ly) & 1 sits at
+// c CN + (ly + 1) CW + (lx + 1) / 2.  A warp's nodes of one colour, and each of
+// their four neighbours (all of the other colour), are then consecutive words
+// (no bank conflicts), and the ring (a = q = 0) needs no boundary tests.
+constexpr int CW = (RE + 2) / 2;        // 25 words a row of one colour
+constexpr int CN = CW * (RE + 2);       // nodes of one colour, ring included
+constexpr int CHALF = RE * RE / 2;      // nodes of one colour in the region
+struct SolveSmem {
+  float2 bi[2 * CN];             // T* + w~0 a f_l(n) - T_s, and 1 / (T_l - T_s + w~0 a)
+  float2 af[2 * CN];             // a and f_l(n); a = 0 on walls, outside and on the ring
+  float q[2 * CN];               // a (f - f_l(n))
+  float f[2 * CN];               // current iterate
+  unsigned short nodes[2][CHALF];   // the nodes the sweeps update, by colour: place | lx odd << 15
+  int cnt[2];                    // how many
+  int bits;                      // what changed in the tile
+  int mine;                      // listed tiles of this CTA
+  unsigned short tile[COUNT_TILES];
+  int wsum[32];
+};
+
+// The tiles the step listed, counted from their stamps by every CTA for itself
+// (at most COUNT_TILES of them): CTA bid takes those of rank bid, bid + nblk,
+// ...  Returns their number; the CTA's own are in sm.tile[0 .. sm.mine).  They
+// are also put on the step's list, for the commit kernel.
+template <int PAR>
+__device__ __forceinline__ int count_tiles(const Dev& d, SolveSmem& sm, int stamp, int bid,
+                                           int nblk) {
+  constexpr int J = (COUNT_TILES + EB - 1) / EB;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int* fl = d.flags + PAR * d.ntiles;
+  int got[J];
 #pragma unroll
-      for (int j = 0; j < NK; ++j) {
-        const int k = tid + j * EB;
-        if (k < RE * RE) {
-          const int ly = k / RE, lx = k - ly * RE;
-          const int gx = X0 - RH + lx, gy = Y0 - RH + ly;
-          const int s = gy * d.nx + gx;
-          fnv[j] = d.fl[s];
-          phv[j] = d.phi[s];
-          Tv[j] = tstar_t<S>(d, s, gx - 1, gx + 1, gy - 1, gy + 1, gx, gy, LAYOUT);
-        }
-      }
+  for (int j = 0; j < J; ++j) got[j] = j * EB + tid < d.ntiles ? fl[j * EB + tid] : 0;
+  unsigned vote[J];
+  int total = 0;
 #pragma unroll
-      for (int j = 0; j < NK; ++j) {
-        const int k = tid + j * EB;
-        if (k < RE * RE) {
-          const float fn = fnv[j];
-          const float a = phv[j] * d.lat * sigma_ratio(d, fn);   // phi dT / (sigma(f_l(n)) St)
-          sbase[k] = Tv[j] + w0 * a * fn - Ts;
-          sinv[k] = 1.f / (dTt + w0 * a);
-          sa[k] = a;
-          sfn[k] = fn;
-          sq[k] = 0.f;
-          sf[k] = fn;
-        }
-      }
-    } else {
-#pragma unroll 3
-      for (int k = tid; k < RE * RE; k += EB) {
-        const int ly = k / RE, lx = k - ly * RE;
-        const int gx = wrapx(d, X0 - RH + lx), gy = wrapy(d, Y0 - RH + ly);
-        float base = 0.f, inv = 0.f, a = 0.f, fn = 0.f;
-        if (gx >= 0 && gy >= 0) {
-          const int s = gy * d.nx + gx;
-          fn = d.fl[s];
-          if (!is_wall(d, gx, gy)) {
-            a = d.phi[s] * d.lat * sigma_ratio(d, fn);   // phi dT / (sigma(f_l(n)) St)
-            const int xm = (gx == 0) ? d.nx - 1 : gx - 1, xp = (gx == d.nx - 1) ? 0 : gx + 1;
-            const int ym = (gy == 0) ? d.ny - 1 : gy - 1, yp = (gy == d.ny - 1) ? 0 : gy + 1;
-            base = tstar_t<S>(d, s, xm, xp, ym, yp, gx, gy, LAYOUT) + w0 * a * fn - Ts;
-            inv = 1.f / (dTt + w0 * a);
-          }
-        }
-        sbase[k] = base;
-        sinv[k] = inv;
-        sa[k] = a;
-        sfn[k] = fn;
-        sq[k] = 0.f;
-        sf[k] = fn;
-      }
-    }
-    __syncthreads();
-    // Nodes whose update is clamped whatever their neighbours do are fixed now
-    // and left out of the sweeps: with q_j in [-a_j f_l(n)_j, a_j (1 - f_l(n)_j)],
-    // the unclamped value (b - w~_1 sum_j q_j) inv stays <= 0 (or >= 1) when it
-    // does so at the extreme sum.  The sweeps then cover only the bounding box of
-    // the nodes left (a band along the front); the fixed point is unchanged.
-    if (tid == 0) {
-      sbox[0] = RE;
-      sbox[1] = -1;
-      sbox[2] = RE;
-      sbox[3] = -1;
-    }
-    __syncthreads();
-    {
-      int bx0 = RE, bx1 = -1, by0 = RE, by1 = -1;
-      for (int k = tid; k < RE * RE; k += EB) {
-        const float inv = sinv[k];
-        if (inv == 0.f) continue;
-        const int ly = k / RE, lx = k - ly * RE;
-        float nlo = 0.f, nhi = 0.f;   // extreme neighbour sums of q
-        auto acc = [&](int j) {
-          nlo -= sa[j] * sfn[j];
-          nhi += sa[j] * (1.f - sfn[j]);
-        };
-        if (lx > 0) acc(k - 1);
-        if (lx < RE - 1) acc(k + 1);
-        if (ly > 0) acc(k - RE);
-        if (ly < RE - 1) acc(k + RE);
-        const float b = sbase[k];
-        const float hi_raw = (b - w1 * nlo) * inv, lo_raw = (b - w1 * nhi) * inv;
-        float v = -1.f;
-        if (hi_raw < -1e-6f) v = 0.f;            // clamped to 0 for any neighbour values
-        else if (lo_raw > 1.f + 1e-6f) v = 1.f;  // clamped to 1
-        if (v >= 0.f) {
-          sf[k] = v;
-          sq[k] = sa[k] * (v - sfn[k]);
-          sinv[k] = 0.f;
-        } else {
-          bx0 = min(bx0, lx);
-          bx1 = max(bx1, lx);
-          by0 = min(by0, ly);
-          by1 = max(by1, ly);
-        }
-      }
-      bx0 = __reduce_min_sync(0xffffffffu, bx0);
-      bx1 = __reduce_max_sync(0xffffffffu, bx1);
-      by0 = __reduce_min_sync(0xffffffffu, by0);
-      by1 = __reduce_max_sync(0xffffffffu, by1);
-      if ((tid & 31) == 0 && bx1 >= 0) {
-        atomicMin(&sbox[0], bx0);
-        atomicMax(&sbox[1], bx1);
-        atomicMin(&sbox[2], by0);
-        atomicMax(&sbox[3], by1);
-      }
-    }
-    __syncthreads();
-    const int lx0 = sbox[0], ly0 = sbox[2];
-    const int ncol = sbox[1] >= lx0 ? (sbox[1] - lx0 + 2) >> 1 : 0;   // per colour and row
-    const int nbox = ncol * (sbox[3] - ly0 + 1);
-    const float inv_ncol = ncol ? 1.f / (float)ncol : 0.f;
-    // the sweeps run on as many whole warps as one colour of the box needs;
-    // the other warps wait at the barrier after them
-    const int sw = min(EB, (nbox + 31) & ~31);
-    int it = 0;
-    bool more = sw > 0;   // (nothing left to sweep: solved by the fixing pass)
-    int polish = more ? 2 : 0;   // extra sweeps after the stop test passes
-    if (nbox <= EB) {
-      // One node per colour and thread: each sweeping thread keeps its two
-      // nodes' place (packed with which neighbours lie in the region),
-      // coefficients and current value in registers, so that a sweep only
-      // exchanges q through shared memory.
-      int kk[2];
-      float cb[2], cinv[2], ca[2], cfn[2], cf[2];
-#pragma unroll
-      for (int color = 0; color < 2; ++color) {
-        int k = -1;
-        if (tid < nbox) {
-          // (row, column pair) of the box; exact for j < 2^16 and ncol <= 24
-          const int r = (int)(((float)tid + 0.5f) * inv_ncol);
-          const int ly = ly0 + r;
-          const int lx = lx0 + ((lx0 + ly + color) & 1) + 2 * (tid - r * ncol);
-          if (lx < RE) {
-            k = ly * RE + lx;
-            if (sinv[k] == 0.f) k = -1;   // wall, outside, or fixed above
-            else
-              k |= ((lx > 0) | ((lx < RE - 1) << 1) | ((ly > 0) << 2) | ((ly < RE - 1) << 3)) << 16;
-          }
-        }
-        const int q = k & 0xffff;
-        const float inv = k >= 0 ? sinv[q] : 0.f;
-        kk[color] = k;
-        cb[color] = k >= 0 ? sbase[q] : 0.f;
-        cinv[color] = inv;
-        ca[color] = k >= 0 ? sa[q] : 0.f;
-        cfn[color] = k >= 0 ? sfn[q] : 0.f;
-        cf[color] = k >= 0 ? sf[q] : 0.f;
-      }
-      if (tid < sw)
-        for (; it < d.max_inner && (more || polish > 0); ++it) {
-          if (!more) --polish;
-          // over-relaxed for the first sweeps, then plain Gauss-Seidel: at the last
-          // few ulps over-relaxation can cycle instead of meeting the stop test
-          const float om = (more && it < SOR_SWEEPS) ? SOR_OMEGA : 1.f;
-          bool changed = false;
-#pragma unroll
-          for (int color = 0; color < 2; ++color) {
-            const int k = kk[color];
-            if (k >= 0) {
-              const int q = k & 0xffff;
-              const int m = k >> 16;
-              float nb = 0.f;
-              if (m & 1) nb += sq[q - 1];
-              if (m & 2) nb += sq[q + 1];
-              if (m & 4) nb += sq[q - RE];
-              if (m & 8) nb += sq[q + RE];
-              const float fo = cf[color];
-              const float raw = (cb[color] - w1 * nb) * cinv[color];
-              float v = (om == 1.f) ? raw : fo + om * (raw - fo);
-              v = fminf(fmaxf(v, 0.f), 1.f);
-              // converged at about four ulps of v and of the terms that make it
-              const float tol =
-                  4.8e-7f * (v + (fabsf(cb[color]) + w1 * fabsf(nb)) * cinv[color]);
-              if (fabsf(v - fo) > tol) changed = true;
-              cf[color] = v;
-              // (a (v - f_l(n)) is exactly 0 on a node that does not move: a
-              // spurious source there would cost a rounding of its neighbours'
-              // 16-bit populations in the commit)
-              sq[q] = ca[color] * (v - cfn[color]);
-            }
-            // the second colour's barrier also collects the convergence vote
-            if (color == 0) sub_sync(sw);
-          }
-          const bool c = sub_sync_or(sw, changed);
-          if (more) more = c;
-        }
-#pragma unroll
-      for (int color = 0; color < 2; ++color)
-        if (kk[color] >= 0) sf[kk[color] & 0xffff] = cf[color];
-    } else if (tid < sw) {
-      for (; it < d.max_inner && (more || polish > 0); ++it) {
-        if (!more) --polish;
-        const float om = (more && it < SOR_SWEEPS) ? SOR_OMEGA : 1.f;
-        bool changed = false;
-#pragma unroll
-        for (int color = 0; color < 2; ++color) {
-          for (int j = tid; j < nbox; j += EB) {
-            const int r = (int)(((float)j + 0.5f) * inv_ncol);
-            const int ly = ly0 + r;
-            const int lx = lx0 + ((lx0 + ly + color) & 1) + 2 * (j - r * ncol);
-            if (lx >= RE) continue;
-            const int k = ly * RE + lx;
-            const float inv = sinv[k];
-            if (inv == 0.f) continue;   // wall, outside, or fixed above
-            const float a = sa[k];
-            float nb = 0.f;
-            if (lx > 0) nb += sq[k - 1];
-            if (lx < RE - 1) nb += sq[k + 1];
-            if (ly > 0) nb += sq[k - RE];
-            if (ly < RE - 1) nb += sq[k + RE];
-            const float b = sbase[k];
-            const float fo = sf[k];
-            const float raw = (b - w1 * nb) * inv;
-            float v = (om == 1.f) ? raw : fo + om * (raw - fo);
-            v = fminf(fmaxf(v, 0.f), 1.f);
-            const float tol = 4.8e-7f * (v + (fabsf(b) + w1 * fabsf(nb)) * inv);
-            if (fabsf(v - fo) > tol) changed = true;
-            sf[k] = v;
-            sq[k] = a * (v - sfn[k]);
-          }
-          if (color == 0) sub_sync(sw);
-        }
-        const bool c = sub_sync_or(sw, changed);
-        if (more) more = c;
-      }
-    }
-    __syncthreads();
-    bool fchg = false, achg = false;
-    for (int k = tid; k < TE * TE; k += EB) {
-      const int ly = k / TE, lx = k - ly * TE;
-      const int gx = X0 + lx, gy = Y0 + ly;
-      if (gx >= d.nx || gy >= d.ny) continue;
-      const int r = (ly + RH) * RE + (lx + RH);
-      const float fo = sfn[r], fnw = sf[r];
-      d.scr[gy * d.nx + gx] = make_float2(fo, fnw);
-      if (fnw != fo) {
-        fchg = true;
-        if ((fo >= d.f_act) != (fnw >= d.f_act)) achg = true;
-      }
-    }
-    const int bits = 1 | (__syncthreads_or(fchg) ? 2 : 0) | (__syncthreads_or(achg) ? 4 : 0);
-    if (tid == 0) {
-      if (more) {
-        atomicExch(&d.stats[0], 1);
-        d.stats[3] = tile;
-      }
-      atomicAdd(&d.stats[1], 1);
-      atomicMax(&d.stats[2], it);
-      d.proc[tile] = (stamp << 3) | bits;
-    }
-    __syncthreads();
+  for (int j = 0; j < J; ++j) {
+    vote[j] = __ballot_sync(0xffffffffu, j * EB + tid < d.ntiles && got[j] == stamp);
+    total += __popc(vote[j]);
   }
-  if (threadIdx.x == 0 && d.trace) trace_end(d, 100 * PAR + 20, d.ctr[PAR], tr0);
+  if (lane == 0) sm.wsum[warp] = total;
+  if (tid == 0) sm.mine = 0;
+  __syncthreads();
+  int before = 0, all = 0;
+#pragma unroll
+  for (int w = 0; w < EB / 32; ++w) {
+    const int v = sm.wsum[w];
+    before += w < warp ? v : 0;
+    all += v;
+  }
+#pragma unroll
+  for (int j = 0; j < J; ++j) {
+    if ((vote[j] >> lane) & 1u) {
+      const int rank = before + __popc(vote[j] & ((1u << lane) - 1u));
+      if (rank % nblk == bid) {
+        sm.tile[atomicAdd(&sm.mine, 1)] = (unsigned short)(j * EB + tid);
+        d.list[PAR * d.ntiles + rank] = j * EB + tid;
+      }
+    }
+    before += __popc(vote[j]);
+  }
+  __syncthreads();
+  return all;
 }
 
-template <int PAR, typename S, int EB>
-__global__ void __launch_bounds__(EB) enthalpy_solve_kernel(Dev d) {
-  enthalpy_solve_body<PAR, S, EB>(d, (int)blockIdx.x, (int)gridDim.x);
+// One listed tile.  EB threads in rows of RE: a thread's nodes lie one above
+// the other, an even number of rows apart, so they share a column and a colour
+// and every index follows from the first by a constant.  During the sweeps a
+// thread holds up to NC nodes of either colour in registers.
+template <int PAR, typename S>
+__device__ __forceinline__ void solve_tile(const Dev& d, SolveSmem& sm, int tile, int stamp) {
+  constexpr int LAYOUT = 1 - PAR;
+  constexpr int RT = EB / RE;                      // rows the CTA covers at once
+  constexpr int NK = RE / RT;                      // nodes of a thread
+  constexpr int NC = (CHALF + EB - 1) / EB;
+  static_assert(EB % RE == 0 && RE % RT == 0 && RT % 2 == 0 && EB % 32 == 0, "block size");
+  constexpr unsigned FULL = 0xffffffffu;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const float w0 = d.wt0, w1 = d.wt1, Ts = d.T_s, dTt = d.dTt;
+  const int X0 = (tile % d.etx) * TE, Y0 = (tile / d.etx) * TE;
+  const int ly0 = tid / RE, lx = tid - ly0 * RE;
+  const bool odd = (lx + ly0) & 1;                 // colour of the thread's nodes
+  const int r0 = (ly0 + 1) * CW + ((lx + 1) >> 1);   // place in the colour; + RT CW a node
+  const int p0 = (odd ? CN : 0) + r0;
+  if (tid < 2) sm.cnt[tid] = 0;
+  if (tid == 2) sm.bits = 0;
+  float fnv[NK], av[NK], Tv[NK];
+  unsigned off = 0u;   // bit j: this thread's node j is a wall node or outside
+  // a region inside the wall ring needs no wrapping and holds no wall node: its
+  // loads go straight to their addresses, all of a thread's in flight together
+  if (X0 - RH >= 1 && X0 + TE + RH <= d.nx - 1 && Y0 - RH >= 1 && Y0 + TE + RH <= d.ny - 1) {
+    const int gx = X0 - RH + lx;
+#pragma unroll
+    for (int j = 0; j < NK; ++j) {
+      const int gy = Y0 - RH + ly0 + j * RT, s = gy * d.nx + gx;
+      fnv[j] = d.fl[s];
+      av[j] = d.phi[s];
+      Tv[j] = tstar_t<S>(d, s, gx - 1, gx + 1, gy - 1, gy + 1, gx, gy, LAYOUT);
+    }
+  } else {
+    const int gx = wrapx(d, X0 - RH + lx);
+    const int xm = (gx == 0) ? d.nx - 1 : gx - 1, xp = (gx == d.nx - 1) ? 0 : gx + 1;
+#pragma unroll
+    for (int j = 0; j < NK; ++j) {
+      fnv[j] = av[j] = Tv[j] = 0.f;
+      const int gy = wrapy(d, Y0 - RH + ly0 + j * RT);
+      bool out = true;
+      if (gx >= 0 && gy >= 0) {
+        const int s = gy * d.nx + gx;
+        fnv[j] = d.fl[s];
+        out = is_wall(d, gx, gy);
+        if (!out) {
+          const int ym = (gy == 0) ? d.ny - 1 : gy - 1, yp = (gy == d.ny - 1) ? 0 : gy + 1;
+          av[j] = d.phi[s];
+          Tv[j] = tstar_t<S>(d, s, xm, xp, ym, yp, gx, gy, LAYOUT);
+        }
+      }
+      if (out) off |= 1u << j;
+    }
+  }
+  float bv[NK], iv[NK];
+#pragma unroll
+  for (int j = 0; j < NK; ++j) {
+    const bool out = (off >> j) & 1u;
+    const float fn = fnv[j];
+    const float a = out ? 0.f : av[j] * d.lat * sigma_ratio(d, fn);   // phi dT / (sigma(f_l(n)) St)
+    // (explicit roundings: every instance of the kernel computes the same bits)
+    const float wa = __fmul_rn(w0, a);
+    av[j] = a;
+    bv[j] = out ? 0.f : __fmaf_rn(wa, fn, Tv[j]) - Ts;
+    iv[j] = out ? 0.f : 1.f / __fadd_rn(dTt, wa);
+    const int p = p0 + j * RT * CW;
+    sm.af[p] = make_float2(a, fn);
+    sm.bi[p] = make_float2(bv[j], iv[j]);
+    sm.q[p] = 0.f;
+    sm.f[p] = fn;
+  }
+  __syncthreads();
+  // Nodes whose update is clamped whatever their neighbours do are fixed now
+  // and left out of the sweeps: with q_j in [-a_j f_l(n)_j, a_j (1 - f_l(n)_j)],
+  // the unclamped value (b - w~_1 sum_j q_j) inv stays <= 0 (or >= 1) when it
+  // does so at the extreme sum (by a margin that covers rounding; none is
+  // needed where f_l(n) = 0 at the node and around it and b <= 0, the untouched
+  // solid at T_s: no q there is negative).  The nodes left, a band along the
+  // front, are listed by colour; the fixed point is unchanged.
+  unsigned keep = 0u;
+  const int o0 = (odd ? 0 : CN) + r0, wst = o0 - (lx & 1);   // other colour; west neighbour
+#pragma unroll
+  for (int j = 0; j < NK; ++j) {
+    const int r = j * RT * CW;
+    const float2 nb[4] = {sm.af[wst + r], sm.af[wst + r + 1], sm.af[o0 + r - CW],
+                          sm.af[o0 + r + CW]};
+    float nlo = 0.f, nhi = 0.f;   // extreme neighbour sums of q
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      nlo -= nb[i].x * nb[i].y;
+      nhi += nb[i].x * (1.f - nb[i].y);
+    }
+    const float fn = fnv[j];
+    const float hi_raw = (bv[j] - w1 * nlo) * iv[j], lo_raw = (bv[j] - w1 * nhi) * iv[j];
+    float v = -1.f;
+    if (hi_raw < -1e-6f || (bv[j] <= 0.f && fn == 0.f && nlo == 0.f)) v = 0.f;
+    else if (lo_raw > 1.f + 1e-6f) v = 1.f;
+    if ((off >> j) & 1u) continue;
+    if (v >= 0.f) {
+      sm.f[p0 + r] = v;
+      sm.q[p0 + r] = av[j] * (v - fn);
+    } else {
+      keep |= 1u << j;
+    }
+  }
+  // list them: one place per warp and colour, then each lane's nodes in turn
+  {
+    const unsigned of_odd = __ballot_sync(FULL, odd);
+    const unsigned own = odd ? of_odd : ~of_odd;
+    unsigned vote[NK];
+    int n0 = 0, n1 = 0;
+#pragma unroll
+    for (int j = 0; j < NK; ++j) {
+      vote[j] = __ballot_sync(FULL, (keep >> j) & 1u);
+      n0 += __popc(vote[j] & ~of_odd);
+      n1 += __popc(vote[j] & of_odd);
+    }
+    int at0 = 0, at1 = 0;
+    if (lane == 0) {
+      if (n0) at0 = atomicAdd(&sm.cnt[0], n0);
+      if (n1) at1 = atomicAdd(&sm.cnt[1], n1);
+    }
+    at0 = __shfl_sync(FULL, at0, 0);
+    at1 = __shfl_sync(FULL, at1, 0);
+    int at = odd ? at1 : at0;
+    const unsigned below = (1u << lane) - 1u;
+#pragma unroll
+    for (int j = 0; j < NK; ++j) {
+      const unsigned u = vote[j] & own;
+      if ((keep >> j) & 1u)
+        sm.nodes[odd][at + __popc(u & below)] =
+            (unsigned short)((r0 + j * RT * CW) | ((lx & 1) << 15));
+      at += __popc(u);
+    }
+  }
+  __syncthreads();
+  const int c0 = sm.cnt[0], c1 = sm.cnt[1], most = max(c0, c1);
+  // the sweeps run on as many whole warps as the larger colour needs; the
+  // other warps wait at the barrier after them
+  const int sw = min(EB, (most + 31) & ~31);
+  int it = 0;
+  bool more = sw > 0;   // (nothing left to sweep: solved by the fixing pass)
+  int polish = more ? 2 : 0;   // extra sweeps after the stop test passes
+  if (tid < sw) {
+    // each sweeping thread keeps its nodes' coefficients and current values in
+    // registers, so that a sweep only exchanges q through shared memory
+    int kk[2][NC];
+    float cb[2][NC], cinv[2][NC], ca[2][NC], cfn[2][NC], cf[2][NC];
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+      for (int m = 0; m < NC; ++m) {
+        const int j = tid + m * EB;
+        const bool on = j < (c ? c1 : c0);
+        const int v = on ? sm.nodes[c][j] : 0;
+        const int p = c * CN + (v & 0x7fff);
+        const float2 bi = sm.bi[p], af = sm.af[p];
+        kk[c][m] = on ? (p | (v & 0x8000)) : -1;   // (2 CN < 2^15)
+        cb[c][m] = bi.x;
+        cinv[c][m] = bi.y;
+        ca[c][m] = af.x;
+        cfn[c][m] = af.y;
+        cf[c][m] = sm.f[p];
+      }
+    for (; it < d.max_inner && (more || polish > 0); ++it) {
+      if (!more) --polish;
+      // over-relaxed for the first sweeps, then plain Gauss-Seidel: at the last
+      // few ulps over-relaxation can cycle instead of meeting the stop test
+      const float om = (more && it < SOR_SWEEPS) ? SOR_OMEGA : 1.f;
+      bool changed = false;
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+#pragma unroll
+        for (int m = 0; m < NC; ++m) {
+          if (m > 0 && m * EB >= most) break;   // (the same in every thread)
+          const int k = kk[c][m];
+          if (k >= 0) {
+            const int p = k & 0x7fff;
+            const int o = c ? p - CN : p + CN, w = o - (k >> 15);
+            const float nb = ((sm.q[w] + sm.q[w + 1]) + sm.q[o - CW]) + sm.q[o + CW];
+            const float fo = cf[c][m];
+            const float raw = (cb[c][m] - w1 * nb) * cinv[c][m];
+            float v = (om == 1.f) ? raw : fo + om * (raw - fo);
+            v = fminf(fmaxf(v, 0.f), 1.f);
+            // converged at about four ulps of v and of the terms that make it
+            const float tol =
+                4.8e-7f * (v + (fabsf(cb[c][m]) + w1 * fabsf(nb)) * cinv[c][m]);
+            if (fabsf(v - fo) > tol) changed = true;
+            cf[c][m] = v;
+            // (a (v - f_l(n)) is exactly 0 on a node that does not move: a
+            // spurious source there would cost a rounding of its neighbours'
+            // 16-bit populations in the commit)
+            sm.q[p] = ca[c][m] * (v - cfn[c][m]);
+          }
+        }
+        // the second colour's barrier also collects the convergence vote
+        if (c == 0) sub_sync(sw);
+      }
+      const bool c = sub_sync_or(sw, changed);
+      if (more) more = c;
+    }
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+      for (int m = 0; m < NC; ++m)
+        if (kk[c][m] >= 0) sm.f[kk[c][m] & 0x7fff] = cf[c][m];
+  }
+  __syncthreads();
+  unsigned ch = 0u;
+  for (int k = tid; k < TE * TE; k += EB) {
+    const int ly = k / TE, lt = k - ly * TE;
+    const int gx = X0 + lt, gy = Y0 + ly;
+    if (gx >= d.nx || gy >= d.ny) continue;
+    const int r = ((lt + ly) & 1) * CN + (ly + RH + 1) * CW + ((lt + RH + 1) >> 1);
+    const float fo = sm.af[r].y, fnw = sm.f[r];
+    d.scr[gy * d.nx + gx] = make_float2(fo, fnw);
+    if (fnw != fo) ch |= (fo >= d.f_act) != (fnw >= d.f_act) ? 6u : 2u;
+  }
+  ch = __reduce_or_sync(FULL, ch);
+  if (lane == 0 && ch) atomicOr(&sm.bits, (int)ch);
+  __syncthreads();
+  if (tid == 0) {
+    if (more) {
+      atomicExch(&d.stats[0], 1);
+      d.stats[3] = tile;
+    }
+    atomicAdd(&d.stats[1], 1);
+    atomicMax(&d.stats[2], it);
+    d.proc[tile] = (stamp << 3) | 1 | sm.bits;
+  }
+  __syncthreads();
+}
+
+// CTA bid of nblk (the whole grid of a single lattice's launch, a range of a
+// batched one) takes listed tiles bid, bid + nblk, ...
+//
+// Bound by latency: one tile's chain of the stamps, the loads, the fixing pass
+// and some thirteen sweeps, on one SM (10 us of the 20 us step at 256^2).  It
+// took 23 us there (40 us beside the far tiles at 2048^2) when the sweeps ran
+// over the bounding box of the nodes left: solid at exactly T_s is not clamped
+// by the margin test, so the box was half the region, three nodes a thread, and
+// each sweep worked out every node's place again.
+template <int PAR, typename S>
+__device__ __forceinline__ void enthalpy_solve_body(const Dev& d, int bid, int nblk) {
+  const long long tr0 = trace_start(d);
+  extern __shared__ __align__(16) unsigned char solve_smem[];
+  SolveSmem& sm = *reinterpret_cast<SolveSmem*>(solve_smem);
+  const int tid = threadIdx.x;
+  const int ctr = d.ctr[PAR];
+  const int stamp = ctr & 0x0FFFFFFF;
+  // the ring: no node there, a = q = 0
+  for (int k = tid; k < 4 * (RE + 2); k += EB) {
+    const int e = k / (RE + 2), i = k - e * (RE + 2);
+    const int px = e == 0 ? 0 : e == 1 ? RE + 1 : i, py = e == 2 ? 0 : e == 3 ? RE + 1 : i;
+    const int p = ((px + py) & 1) * CN + py * CW + (px >> 1);
+    sm.af[p] = make_float2(0.f, 0.f);
+    sm.q[p] = 0.f;
+  }
+  if (d.ntiles > COUNT_TILES) {   // the stream-collide pass kept a list
+    int tile = bid < d.ntiles ? d.list[PAR * d.ntiles + bid] : 0;
+    const int cnt = d.lcount[PAR];
+    for (int li = bid; li < cnt; li += nblk) {
+      if (li != bid) tile = d.list[PAR * d.ntiles + li];
+      solve_tile<PAR, S>(d, sm, tile, stamp);
+    }
+  } else {
+    const int rank = count_tiles<PAR>(d, sm, ctr, bid, nblk);
+    for (int i = 0; i < sm.mine; ++i) solve_tile<PAR, S>(d, sm, sm.tile[i], stamp);
+    if (tid == 0 && bid == 0) d.lcount[PAR] = rank;
+  }
+  if (tid == 0 && d.trace) trace_end(d, 100 * PAR + 20, ctr, tr0);
+}
+
+template <int PAR, typename S>
+__global__ void __launch_bounds__(EB, 1) enthalpy_solve_kernel(Dev d) {
+  enthalpy_solve_body<PAR, S>(d, (int)blockIdx.x, (int)gridDim.x);
 }
 
 // (three CTAs a SM: a batch lists many small tiles at once)
-template <int PAR, typename S, int EB>
-__global__ void __launch_bounds__(EB, 3) enthalpy_solve_batch_kernel(const __grid_constant__ BatchPlan P) {
+template <int PAR, typename S>
+__global__ void __launch_bounds__(EB, 2) enthalpy_solve_batch_kernel(const __grid_constant__ BatchPlan P) {
   const int c = plan_lattice(P, (int)blockIdx.x);
-  enthalpy_solve_body<PAR, S, EB>(P.d[c], (int)blockIdx.x - P.start[c], P.start[c + 1] - P.start[c]);
+  enthalpy_solve_body<PAR, S>(P.d[c], (int)blockIdx.x - P.start[c], P.start[c + 1] - P.start[c]);
 }
 
 // x changed flow activity and is the inward node of a flow wall w next to it:
@@ -421,40 +480,44 @@ __device__ __forceinline__ void enthalpy_commit_body(const Dev& d, int bid, int 
   constexpr int RW = TE + 2;              // tile plus a one-node ring
   __shared__ float2 sp[RW * RW];          // (f_l(n), f_l(n+1)); (-1,-1) on walls / outside
   __shared__ unsigned char ssolved[RW * RW];
-  __shared__ int links;
+  static_assert(CB == TE * TE, "one thread per node of a tile");
   const int tid = threadIdx.x;
+  // (the first tile's number is read beside the count; a CTA without a tile
+  // reads a place of the list that is not in use)
+  int tile = bid < d.ntiles ? d.list[PAR * d.ntiles + bid] : 0;
   const int cnt = d.lcount[PAR];
   const int stamp = stamp_of(d, PAR);
   const int n = (int)d.n;
   for (int li = bid; li < cnt; li += nblk) {
-    const int tile = d.list[PAR * d.ntiles + li];
+    if (li != bid) tile = d.list[PAR * d.ntiles + li];
     const int tx0 = tile % d.etx, ty0 = tile / d.etx;
     const int X0 = tx0 * TE, Y0 = ty0 * TE;
-    const int pb = d.proc[tile] & 7;
-    if (tid == 0) {
-      d.flags[PAR * d.ntiles + tile] = 0;   // this step's fused pass is done with it
-      // flow links need attention only around tiles where a node's activity changed
-      int l = 0;
-      if (d.flow && LAYOUT == 1) {
-        for (int dy = -1; dy <= 1; ++dy)
-          for (int dx = -1; dx <= 1; ++dx) {
-            int tx = tx0 + dx, ty = ty0 + dy;
-            if (tx < 0 || tx >= d.etx) {
-              if (!d.per_x) continue;
-              tx = (tx + d.etx) % d.etx;
-            }
-            if (ty < 0 || ty >= d.ety) {
-              if (!d.per_y) continue;
-              ty = (ty + d.ety) % d.ety;
-            }
-            const int t = ty * d.etx + tx;
-            if (solved(d, t, stamp) && (d.proc[t] & 4)) l = 1;
-          }
-      }
-      links = l;
+    // this thread's node, read beside the tile's status word
+    const int x = X0 + tid % TE, y = Y0 + tid / TE, s = y * d.nx + x;
+    const bool node = x < d.nx && y < d.ny && !is_wall(d, x, y);
+    float2 p = make_float2(0.f, 0.f);
+    float ph = 0.f;
+    if (node) {
+      p = d.scr[s];
+      ph = d.phi[s];
     }
-    __syncthreads();
-    const bool lk = links != 0;
+    const int pb = d.proc[tile] & 7;
+    // flow links need attention only around tiles where a node's activity
+    // changed (nine threads look at the tile and those around it)
+    bool lk = false;
+    if (LAYOUT == 1 && d.flow) {
+      bool l = false;
+      if (tid < 9) {
+        int tx = tx0 + tid % 3 - 1, ty = ty0 + tid / 3 - 1;
+        if (d.per_x) tx = tx < 0 ? d.etx - 1 : tx >= d.etx ? 0 : tx;
+        if (d.per_y) ty = ty < 0 ? d.ety - 1 : ty >= d.ety ? 0 : ty;
+        if (tx >= 0 && tx < d.etx && ty >= 0 && ty < d.ety) {
+          const int v = d.proc[ty * d.etx + tx];
+          l = (v >> 3) == stamp && (v & 4);
+        }
+      }
+      lk = __syncthreads_or(l);
+    }
     if ((pb & 2) || lk) {
       if (lk) {
         // old/new liquid fraction of the tile and its ring: scratch in tiles
@@ -488,29 +551,31 @@ __device__ __forceinline__ void enthalpy_commit_body(const Dev& d, int bid, int 
         __syncthreads();
       }
       int flows = 0;   // a node of the tile carries flow after the step
-#pragma unroll 4
-      for (int k = tid; k < TE * TE; k += CB) {
-        const int ly = k / TE, lx = k - ly * TE;
-        const int x = X0 + lx, y = Y0 + ly;
-        if (x >= d.nx || y >= d.ny || is_wall(d, x, y)) continue;
-        const int s = y * d.nx + x;
-        const float2 p = d.scr[s];
+      if (node) {
+        const int ly = tid / TE, lx = tid % TE;
         const float fn = p.x, fnew = p.y;
-        flows |= fnew >= d.f_act;
+        flows = fnew >= d.f_act;
         if (fnew != fn) {
           d.fl[s] = fnew;
-          const float S0 = -d.phi[s] * d.lat * sigma_ratio(d, fn) * (fnew - fn);
+          const float S0 = -ph * d.lat * sigma_ratio(d, fn) * (fnew - fn);
           // N^-1 S~ = S0 w~, streamed: population i of node x + e_i gains w~_i S0
+          int slot[5];
+          float old[5];
 #pragma unroll
           for (int i = 0; i < 5; ++i) {
             const int rx = wrapx(d, x + ex9(i)), ry = wrapy(d, y + ey9(i));
-            if (rx < 0 || ry < 0 || is_wall(d, rx, ry)) continue;
+            const bool to = rx >= 0 && ry >= 0 && !is_wall(d, rx, ry);
+            slot[i] = !to ? -1 : (LAYOUT == 1) ? opp5(i) * n + s : i * n + ry * d.nx + rx;
+            old[i] = to ? ld_pop(d, d.g, slot[i]) : 0.f;
+          }
+#pragma unroll
+          for (int i = 0; i < 5; ++i) {
+            if (slot[i] < 0) continue;
             const float w = (i == 0) ? d.wt0 : d.wt1;
-            const int slot = (LAYOUT == 1) ? opp5(i) * n + s : i * n + ry * d.nx + rx;
             // (16-bit storage: rounded stochastically, or every small source
             // would be lost to rounding in the same direction)
-            st_pop_round(d, d.g, slot, ld_pop(d, d.g, slot) + w * S0,
-                         mix32((unsigned)slot ^ mix32((unsigned)stamp)));
+            st_pop_round(d, d.g, slot[i], old[i] + w * S0,
+                         mix32((unsigned)slot[i] ^ mix32((unsigned)stamp)));
           }
         }
         if (lk) {
@@ -581,18 +646,14 @@ __global__ void __launch_bounds__(CB, 2) enthalpy_commit_batch_kernel(const __gr
   enthalpy_commit_body<PAR, false>(P.d[c], (int)blockIdx.x - P.start[c], P.start[c + 1] - P.start[c]);
 }
 
-size_t enthalpy_solve_smem() { return 6 * RE * RE * sizeof(float); }
+size_t enthalpy_solve_smem() { return sizeof(SolveSmem); }
 
 template <typename S>
 static void solve_setup_t(int bytes) {
-  cudaFuncSetAttribute(enthalpy_solve_kernel<0, S, EB_WIDE>,
-                       cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  cudaFuncSetAttribute(enthalpy_solve_kernel<1, S, EB_WIDE>,
-                       cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  cudaFuncSetAttribute(enthalpy_solve_kernel<0, S, EB_NARROW>,
-                       cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  cudaFuncSetAttribute(enthalpy_solve_kernel<1, S, EB_NARROW>,
-                       cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  cudaFuncSetAttribute(enthalpy_solve_kernel<0, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       bytes);
+  cudaFuncSetAttribute(enthalpy_solve_kernel<1, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       bytes);
 }
 
 void enthalpy_setup() {
@@ -602,20 +663,11 @@ void enthalpy_setup() {
   solve_setup_t<__nv_bfloat16>(bytes);
 }
 
-// A large lattice's solve runs beside a long far-tile pass, whose SMs it shares:
-// narrow CTAs (fewer registers held) cost that pass less.  On a small lattice
-// the far-tile pass hides under the solve, whose latency is then the step
-// time: wide CTAs finish sooner.
 template <typename S>
 static void launch_solve_t(const Dev& d, int parity, cudaStream_t s) {
   const size_t sm = enthalpy_solve_smem();
-  if (d.ntiles >= SOLVE_NARROW_TILES) {
-    if (parity == 0) enthalpy_solve_kernel<0, S, EB_NARROW><<<d.egrid, EB_NARROW, sm, s>>>(d);
-    else enthalpy_solve_kernel<1, S, EB_NARROW><<<d.egrid, EB_NARROW, sm, s>>>(d);
-  } else {
-    if (parity == 0) enthalpy_solve_kernel<0, S, EB_WIDE><<<d.egrid, EB_WIDE, sm, s>>>(d);
-    else enthalpy_solve_kernel<1, S, EB_WIDE><<<d.egrid, EB_WIDE, sm, s>>>(d);
-  }
+  if (parity == 0) enthalpy_solve_kernel<0, S><<<d.egrid, EB, sm, s>>>(d);
+  else enthalpy_solve_kernel<1, S><<<d.egrid, EB, sm, s>>>(d);
 }
 
 void launch_enthalpy_solve(const Dev& d, int parity, cudaStream_t s) {
@@ -629,19 +681,18 @@ void fused_batch_setup();   // lbm_fused_f32.cu
 void batch_setup() {
   fused_batch_setup();
   const int bytes = (int)enthalpy_solve_smem();
-  cudaFuncSetAttribute(enthalpy_solve_batch_kernel<0, float, EB_WIDE>,
+  cudaFuncSetAttribute(enthalpy_solve_batch_kernel<0, float>,
                        cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  cudaFuncSetAttribute(enthalpy_solve_batch_kernel<1, float, EB_WIDE>,
+  cudaFuncSetAttribute(enthalpy_solve_batch_kernel<1, float>,
                        cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
 
-// the lattices of a batch are small: the wide CTAs, which finish a tile sooner
 void launch_enthalpy_solve_batch(const BatchPlan& P, int parity, cudaStream_t s) {
   const size_t sm = enthalpy_solve_smem();
   const int grid = P.start[P.count];
   if (grid <= 0) return;
-  if (parity == 0) enthalpy_solve_batch_kernel<0, float, EB_WIDE><<<grid, EB_WIDE, sm, s>>>(P);
-  else enthalpy_solve_batch_kernel<1, float, EB_WIDE><<<grid, EB_WIDE, sm, s>>>(P);
+  if (parity == 0) enthalpy_solve_batch_kernel<0, float><<<grid, EB, sm, s>>>(P);
+  else enthalpy_solve_batch_kernel<1, float><<<grid, EB, sm, s>>>(P);
 }
 
 void launch_enthalpy_commit_batch(const BatchPlan& P, int parity, cudaStream_t s) {

@@ -67,29 +67,26 @@ __device__ __forceinline__ void fstore(S* p, float v, unsigned& rnd) {
   else st_round(p, v, next_rand(rnd));
 }
 
-// put enthalpy tile t on this step's work list (once), and stamp the tiles
-// within one tile of it in this parity's near map
-__device__ __forceinline__ void mark_tile(const Dev& d, int t, int par) {
-  int* fl = d.flags + par * d.ntiles;
-  if (fl[t] == 0 && atomicExch(&fl[t], 1) == 0) {
-    const int i = atomicAdd(&d.lcount[par], 1);
-    d.list[par * d.ntiles + i] = t;
-    const int stamp = d.ctr[1 - par] + 1;   // this step's stamp
-    const int tx = t % d.etx, ty = t / d.etx;
-    for (int dy = -1; dy <= 1; ++dy) {
-      int yy = ty + dy;
-      if (yy < 0 || yy >= d.ety) {
-        if (!d.per_y) continue;
-        yy = (yy + d.ety) % d.ety;
-      }
-      for (int dx = -1; dx <= 1; ++dx) {
-        int xx = tx + dx;
-        if (xx < 0 || xx >= d.etx) {
-          if (!d.per_x) continue;
-          xx = (xx + d.etx) % d.etx;
-        }
+// List enthalpy tile t in the step with this stamp.  On a lattice of up to
+// COUNT_TILES tiles that is one store that nothing waits for: the solve kernel
+// counts the stamped tiles itself (an append to a list, a chain of three
+// memory round trips, ends a small lattice's pass 2 us later).  A larger one
+// appends to the step's list, and stamps the tiles within one tile of it in the
+// near map, which costs its long pass nothing and spares every CTA of the solve
+// a walk over all the flags.
+__device__ __forceinline__ void mark_tile(const Dev& d, int t, int par, int stamp) {
+  int* fl = d.flags + par * d.ntiles + t;
+  if (d.ntiles <= COUNT_TILES) {
+    *fl = stamp;
+  } else if (*fl != stamp && atomicExch(fl, stamp) != stamp) {
+    d.list[par * d.ntiles + atomicAdd(&d.lcount[par], 1)] = t;
+    const int ty = t / d.etx, tx = t - ty * d.etx;
+    for (int k = 0; k < 9; ++k) {
+      int xx = tx + k % 3 - 1, yy = ty + k / 3 - 1;
+      if (d.per_x) xx = xx < 0 ? d.etx - 1 : xx >= d.etx ? 0 : xx;
+      if (d.per_y) yy = yy < 0 ? d.ety - 1 : yy >= d.ety ? 0 : yy;
+      if (xx >= 0 && xx < d.etx && yy >= 0 && yy < d.ety)
         d.nearmap[par * d.ntiles + yy * d.etx + xx] = stamp;
-      }
     }
   }
 }
@@ -255,13 +252,14 @@ static __device__ __noinline__ void extrapolated_post(const Dev& d, const float 
 // populations reflected at each link, used where the neighbour carries no
 // flow.  wact (flow walls only): bit i set when neighbour i is a wall node that
 // carries flow (its inward node does), so that the link streams instead of
-// reflecting.  Writes the post-collision populations to their AA slots and
+// reflecting.  stamp: where the step's stamp is kept (read when the node lists
+// a tile).  Writes the post-collision populations to their AA slots and
 // returns whether the node fails the phase-change screen.
 template <typename S, int PAR, int FLOW, bool EDGE = true>
 __device__ __forceinline__ bool node_update(const Dev& d, int x, int y, const Geo& q,
                                             const float fln[9], const float gin[5], float f[9],
                                             const float fb[9], float phi, float K,
-                                            unsigned wact = 0u, unsigned seed = 0u) {
+                                            unsigned wact, unsigned seed, const int* stamp) {
   const int nx = d.nx, ny = d.ny;
   const int n = (int)d.n;
   const int s = q.s;
@@ -407,7 +405,7 @@ __device__ __forceinline__ bool node_update(const Dev& d, int x, int y, const Ge
     for (int j = 0; j < 3; ++j)
 #pragma unroll
       for (int i = 0; i < 3; ++i)
-        if (txs[i] != cx || tys[j] != cy) mark_tile(d, tys[j] * d.etx + txs[i], PAR);
+        if (txs[i] != cx || tys[j] != cy) mark_tile(d, tys[j] * d.etx + txs[i], PAR, *stamp);
   }
   return unsafe;
 }
@@ -439,13 +437,12 @@ __device__ __forceinline__ void step_prologue(const Dev& d) {
 }
 
 // Split steps: does this launch (MODE 1 far tiles, MODE 2 near tiles) take the
-// tile whose enthalpy tile is et?  The previous step's near map carries its
-// stamp on the tiles within one tile of its listed tiles.
+// tile whose enthalpy tile is et?  Near: within one tile of a tile the previous
+// step (its stamp: prev) listed.
 template <int PAR, int MODE>
-__device__ __forceinline__ bool takes_tile(const Dev& d, int et) {
+__device__ __forceinline__ bool takes_tile(const Dev& d, int et, int prev) {
   if (MODE == 0) return true;
-  const bool nr = d.nearmap[(1 - PAR) * d.ntiles + et] == d.ctr[1 - PAR];
-  return (MODE == 2) == nr;
+  return (MODE == 2) == near_listed(d, et, 1 - PAR, prev);
 }
 
 // ---- flow walls (Sec. 4, non-equilibrium extrapolation) ---------------------
@@ -491,7 +488,8 @@ __global__ void __launch_bounds__(256) flow_wall_kernel(Dev d) {
     const int sf = iy * nx + ix;
     const float flf = d.fl[sf];
     if (flf < d.f_act) continue;   // the inward node carries no flow: the wall reflects
-    if (MODE != 0 && !takes_tile<PAR, MODE>(d, (iy / TE) * d.etx + ix / TE)) continue;
+    if (MODE != 0 && !takes_tile<PAR, MODE>(d, (iy / TE) * d.etx + ix / TE, d.ctr[1 - PAR]))
+      continue;
     // x_f's populations before the step's collision, as its own update reads them
     float f[9], g[5];
     if (PAR == 0) {
@@ -580,9 +578,16 @@ template <typename S, int PAR, int FLOW, int MODE>
 __global__ void __launch_bounds__(TX* TY, 4) fused_step_kernel(Dev d) {
   constexpr unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x;
+  const int prev = d.ctr[1 - PAR], stamp = prev + 1;   // (no launch of this step changes it)
   if (MODE != 1 && blockIdx.x == 0 && blockIdx.y == 0 && lane == 0 && threadIdx.y == 0)
     step_prologue<PAR>(d);
-  if (!takes_tile<PAR, MODE>(d, ((blockIdx.y * TY) / TE) * d.etx + (blockIdx.x * TX) / TE)) return;
+  if (MODE != 0) {   // (one tile per CTA: a warp's first nine lanes look at its surroundings)
+    const int et = ((blockIdx.y * TY) / TE) * d.etx + (blockIdx.x * TX) / TE;
+    const bool hit = d.ntiles > COUNT_TILES
+                         ? lane == 0 && d.nearmap[(1 - PAR) * d.ntiles + et] == prev
+                         : lane < 9 && listed_at(d, et, lane, 1 - PAR, prev);
+    if ((MODE == 2) != __any_sync(FULL, hit)) return;
+  }
   const int x = blockIdx.x * TX + lane, y = blockIdx.y * TY + threadIdx.y;
   const int nx = d.nx, ny = d.ny;
   if (y >= ny) return;  // whole warp: one warp is one row segment
@@ -635,11 +640,11 @@ __global__ void __launch_bounds__(TX* TY, 4) fused_step_kernel(Dev d) {
       wact = wall_activity(d, x, y, q, [&](int dx, int dy) {
         return d.fl[(long long)wrapy(d, y + dy) * nx + wrapx(d, x + dx)];
       });
-    const unsigned seed = std::is_same<S, float>::value ? 0u : mix32((unsigned)d.ctr[1 - PAR]);
-    unsafe = node_update<S, PAR, FLOW>(d, x, y, q, fln, g, f, fb, phi, K, wact, seed);
+    const unsigned seed = std::is_same<S, float>::value ? 0u : mix32((unsigned)prev);
+    unsafe = node_update<S, PAR, FLOW>(d, x, y, q, fln, g, f, fb, phi, K, wact, seed, &stamp);
   }
   if (__any_sync(FULL, unsafe) && lane == 0)
-    mark_tile(d, (y / TE) * d.etx + (blockIdx.x * TX) / TE, PAR);
+    mark_tile(d, (y / TE) * d.etx + (blockIdx.x * TX) / TE, PAR, stamp);
 }
 
 // ---- TMA-staged kernel ----------------------------------------------
@@ -755,7 +760,7 @@ __device__ __forceinline__ void tma_issue(const TmaMaps& m, unsigned buf, unsign
 // EDGE = false: the tile has no wall node and no neighbour of a wall node.
 template <typename S, int PAR, int FLOW, bool EDGE>
 __device__ __forceinline__ bool tma_node(const Dev& d, const unsigned char* sb, int x0, int y0,
-                                         int lane, int ty, unsigned seed) {
+                                         int lane, int ty, unsigned seed, const int* stamp) {
   using L = TmaLayout<PAR, S>;
   const int nx = d.nx, ny = d.ny;
   const int x = x0 + lane, y = y0 + ty;
@@ -810,7 +815,7 @@ __device__ __forceinline__ bool tma_node(const Dev& d, const unsigned char* sb, 
       unsigned wact = 0u;
       if (FLOW && EDGE && d.flow_walls)
         wact = wall_activity(d, x, y, q, [&](int dx, int dy) { return sFL[c + dy * WX + dx]; });
-      unsafe = node_update<S, PAR, FLOW, EDGE>(d, x, y, q, fln, g, f, fb, phi, K, wact, seed);
+      unsafe = node_update<S, PAR, FLOW, EDGE>(d, x, y, q, fln, g, f, fb, phi, K, wact, seed, stamp);
   }
   return unsafe;
 }
@@ -824,6 +829,7 @@ __device__ __forceinline__ void fused_tma_body(const Dev& d, const TmaMaps& m, i
   constexpr unsigned FULL = 0xffffffffu;
   extern __shared__ __align__(128) unsigned char smem[];
   unsigned* s_mask = reinterpret_cast<unsigned*>(smem + L::IDX_OFF);
+  int* s_stamp = reinterpret_cast<int*>(s_mask + 1);   // this step's stamp
   const int lane = threadIdx.x, ty = threadIdx.y;
   const int tid = ty * TX + lane;
   const int nx = d.nx, ny = d.ny;
@@ -836,9 +842,9 @@ __device__ __forceinline__ void fused_tma_body(const Dev& d, const TmaMaps& m, i
   const int t0 = bid, dt = nblk;
   const int cnt = (ntile - t0 + dt - 1) / dt;
   const long long tr0 = trace_start(d);
-  // 16-bit storage: the step's part of every node's rounding seed (this
-  // launch does not change ctr[1 - PAR])
-  const unsigned seed = std::is_same<S, float>::value ? 0u : mix32((unsigned)d.ctr[1 - PAR]);
+  const int prev = d.ctr[1 - PAR];   // the previous step's stamp (no launch of this step changes it)
+  // 16-bit storage: the step's part of every node's rounding seed
+  const unsigned seed = std::is_same<S, float>::value ? 0u : mix32((unsigned)prev);
   if (MODE != 1 && bid == 0 && tid == 0) step_prologue<PAR>(d);
   constexpr int NB = L::NBUF;
   const unsigned buf0 = smem_u32(smem);
@@ -861,11 +867,12 @@ __device__ __forceinline__ void fused_tma_body(const Dev& d, const TmaMaps& m, i
     const int t = t0 + lane * dt;
     const int et = ((t / tiles_x) * TY / TE) * d.etx + (t % tiles_x) * TX / TE;
     bool take = lane < cnt;
-    if (take && MODE != 0) take = takes_tile<PAR, MODE>(d, et);
+    if (take && MODE != 0) take = takes_tile<PAR, MODE>(d, et, prev);
     fmask = !FLOW ? 0u : d.tskip ? __ballot_sync(FULL, take && d.tact[et]) : ~0u;
     const unsigned mask = __ballot_sync(FULL, take);
     if (lane == 0) {
       *s_mask = mask;
+      *s_stamp = prev + 1;
       if (mask) {
         for (int j = 0; j < NB; ++j)
           asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar0 + 8 * j) : "memory");
@@ -907,10 +914,10 @@ __device__ __forceinline__ void fused_tma_body(const Dev& d, const TmaMaps& m, i
     // interior tiles (no wall node and no wall neighbour in them) take a copy
     // of the update with the wall logic compiled out
     const bool edge = x0 < 2 || x0 + TX > nx - 2 || y0 < 2 || y0 + TY > ny - 2;
-    const bool unsafe = edge ? tma_node<S, PAR, FLOW, true>(d, sb, x0, y0, lane, ty, seed)
-                             : tma_node<S, PAR, FLOW, false>(d, sb, x0, y0, lane, ty, seed);
+    const bool unsafe = edge ? tma_node<S, PAR, FLOW, true>(d, sb, x0, y0, lane, ty, seed, s_stamp)
+                             : tma_node<S, PAR, FLOW, false>(d, sb, x0, y0, lane, ty, seed, s_stamp);
     if (__any_sync(FULL, unsafe) && lane == 0)
-      mark_tile(d, ((unsigned)y / TE) * d.etx + (unsigned)x0 / TE, PAR);
+      mark_tile(d, ((unsigned)y / TE) * d.etx + (unsigned)x0 / TE, PAR, *s_stamp);
     // every thread is done with buffer b before it is refilled with the tile
     // NB places further on
     __syncthreads();
@@ -934,8 +941,7 @@ __device__ __forceinline__ void fused_tma_body(const Dev& d, const TmaMaps& m, i
       mbar_wait(bar0 + 8 * bj, (phases >> bj) & 1u);
     }
   }
-  // (ctr[1 - PAR] + 1: the step this launch computes; no launch of the step changes it)
-  if (tid == 0 && d.trace) trace_end(d, 100 * PAR + 10 + MODE, d.ctr[1 - PAR] + 1, tr0);
+  if (tid == 0 && d.trace) trace_end(d, 100 * PAR + 10 + MODE, *s_stamp, tr0);
 }
 
 template <typename S, int PAR, int FLOW, int MODE>

@@ -34,11 +34,8 @@ constexpr int TY = 8;        // fused kernel tile (threads y)
 constexpr int TE = 32;       // enthalpy tile edge
 constexpr int RH = 8;        // enthalpy halo width
 constexpr int RE = TE + 2 * RH;
-// enthalpy solve block sizes: narrow CTAs on large lattices (they share SMs with
-// the far-tile pass), wide ones on small lattices (the solve's latency is the step)
-constexpr int EB_NARROW = 256;
-constexpr int EB_WIDE = 512;
-constexpr int SOLVE_NARROW_TILES = 1024;   // enthalpy tiles from which the narrow form runs
+constexpr int EB = 576;      // enthalpy solve block size: 12 rows of a region (solve_tile)
+constexpr int COUNT_TILES = 1152;   // up to this many tiles the solve counts the listed ones itself
 constexpr int CB = 1024;     // enthalpy commit block size (one thread per node of a tile:
                              // narrower CTAs measured slower beside the far-tile pass)
 constexpr int RB = 256;      // reduction block size
@@ -91,12 +88,12 @@ struct Dev {
   const float* phi;
   const float* K;
   const float* wallTl;
-  int* flags;                // [2][ntiles]: 1 once listed in that parity's step (cleared by the solve)
-  int* list;                 // [2][ntiles]: tiles to solve, one list per step parity
+  int* flags;                // [2][ntiles]: per parity, the stamp of the last step that listed the tile
+  int* list;                 // [2][ntiles]: the step's listed tiles, as the solve counted them
   int* lcount;               // [2]: entries in each list
   int* ctr;                  // [2]: step stamp per parity (the fused pass sets ctr[p] = ctr[1-p] + 1)
-  int* nearmap;              // [2][ntiles]: per parity, the stamp of the step that listed a tile
-                             // within one tile of this one
+  int* nearmap;              // [2][ntiles], lattices of more than COUNT_TILES tiles: per parity,
+                             // the stamp of the step that listed a tile within one of this one
   int* proc;                 // per enthalpy tile: (stamp << 3) | bits, bit 0 solved, bit 1
                              // some f_l changed, bit 2 some node's flow activity changed
   float2* scr;               // per node of solved tiles: (f_l(n), f_l(n+1))
@@ -326,6 +323,26 @@ __device__ __forceinline__ int wrapy(const Dev& d, int y) {
 __device__ __forceinline__ bool is_wall(const Dev& d, int x, int y) {
   return (d.wall_l && x == 0) || (d.wall_r && x == d.nx - 1) || (d.wall_b && y == 0) ||
          (d.wall_t && y == d.ny - 1);
+}
+// Near map.  Up to COUNT_TILES tiles: was neighbour k (0..8, row by row; 4 is t
+// itself) of tile t listed in the step of parity par with this stamp?
+__device__ __forceinline__ bool listed_at(const Dev& d, int t, int k, int par, int stamp) {
+  const int ty = t / d.etx, tx = t - ty * d.etx;
+  int xx = tx + k % 3 - 1, yy = ty + k / 3 - 1;
+  if (d.per_x) xx = xx < 0 ? d.etx - 1 : xx >= d.etx ? 0 : xx;
+  if (d.per_y) yy = yy < 0 ? d.ety - 1 : yy >= d.ety ? 0 : yy;
+  if (xx < 0 || xx >= d.etx || yy < 0 || yy >= d.ety) return false;
+  return d.flags[par * d.ntiles + yy * d.etx + xx] == stamp;
+}
+// Was a tile within one tile of tile t listed?  Nine independent loads on a
+// small lattice, where they wait once; one on a large one, whose CTAs are many
+// (2048^2: nine took 3% of the step) and whose marks keep a map of it.
+__device__ __forceinline__ bool near_listed(const Dev& d, int t, int par, int stamp) {
+  if (d.ntiles > COUNT_TILES) return d.nearmap[par * d.ntiles + t] == stamp;
+  bool hit = false;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) hit |= listed_at(d, t, k, par, stamp);
+  return hit;
 }
 // inward neighbour of wall node (x, y): one node into the lattice from each wall
 // it lies on (the diagonal neighbour at a corner)

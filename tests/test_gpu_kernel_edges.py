@@ -1,5 +1,7 @@
-"""The reduction's FP32-pair sums against FP64 sums of the state, on every
-storage and layout.
+"""Kernel forms at the sizes where they change: the count of listed enthalpy
+tiles (by the solve kernel up to 1152 tiles, by a list above), the stamps of a
+context whose fields are loaded again after an odd number of steps, and the
+reduction's FP32-pair sums.
 """
 import numpy as np
 import pytest
@@ -17,6 +19,44 @@ def P():
     __graft_entry__.build()
     import paper_1503_08406_gb300 as P
     return P
+
+
+def _f32(w):
+    for k in ("phi", "K", "T0", "fl0"):
+        setattr(w, k, getattr(w, k).astype(np.float32).astype(np.float64))
+    return w
+
+
+# one row of tiles, 1 to 1153 of them; many listed (a noisy temperature field)
+@pytest.mark.parametrize("nx", [32, 33, 36864, 36865, 36896])
+def test_listed_tiles_counted_or_listed(P, oracle_mod, nx):
+    w = _f32(W.periodic_box(nx, ny=12))
+    lat = P.Lattice(w.nx, w.ny, **w.params)
+    lat.set_fields(w.phi, w.K, w.T0, w.fl0)
+    lat.step(5)
+    assert lat.status() == 0
+    o = oracle_mod.Oracle(w.nx, w.ny, **w.params)
+    o.set_fields(w.phi, w.K, w.T0, w.fl0)
+    o.step(5)
+    got, exp = lat.macros(), o.macros()
+    for k in ("ux", "uy", "T", "fl"):   # the short-run bar of the parity tests
+        assert np.abs(got[k] - exp[k]).max() < 2e-5 * np.abs(exp[k]).max(), k
+
+
+@pytest.mark.parametrize("lead", [1, 2, 3])
+def test_fields_loaded_again_leave_no_stamps(P, lead):
+    """A context stepped, then loaded with fields whose front lies elsewhere,
+    continues as a new one does."""
+    a, b = W.melted_cavity(96, melted_cols=70), W.melted_cavity(96, melted_cols=20)
+    used, new = (P.Lattice(96, 96, **b.params) for _ in range(2))
+    used.set_fields(a.phi, a.K, a.T0, a.fl0)
+    for _ in range(lead):
+        used.step(1)
+    for lat in (used, new):
+        lat.set_fields(b.phi, b.K, b.T0, b.fl0)
+        lat.step(7)
+    for x, y in zip(used.get_state(), new.get_state()):
+        assert np.array_equal(x.view(np.uint32), y.view(np.uint32))
 
 
 @pytest.mark.parametrize("steps", [4, 5])
