@@ -51,7 +51,6 @@ namespace lbm {
 constexpr float SOR_OMEGA = 1.15f;
 constexpr int SOR_SWEEPS = 8;   // over-relaxed sweeps before plain Gauss-Seidel
 
-__device__ __forceinline__ int stamp_of(const Dev& d, int par) { return d.ctr[par] & 0x0FFFFFFF; }
 __device__ __forceinline__ bool solved(const Dev& d, int tile, int stamp) {
   return (d.proc[tile] >> 3) == stamp;
 }
@@ -156,16 +155,110 @@ __device__ __forceinline__ int count_tiles(const Dev& d, SolveSmem& sm, int stam
   return all;
 }
 
+// The sweeps over the listed nodes (c0 and c1 of the two colours), on the first
+// sw threads of the CTA (whole warps), M nodes of a colour a thread (M sw holds
+// them all).  A thread keeps its nodes' coefficients and current values in
+// registers, so that a sweep only exchanges q through shared memory; a thread
+// without a node works on a corner of the ring, which no node reads, so that
+// nothing branches (half a sweep 0.19 -> 0.13 us).  One node a thread and more
+// warps beat two, three or four nodes a thread and fewer (256 x 4 slab: 14.9
+// against 15.1 us a step with two, 17.5 and 18.1 with branches and three, four).
+template <int M>
+__device__ __forceinline__ void sweep_nodes(const Dev& d, SolveSmem& sm, int c0, int c1, int sw,
+                                            int& sweeps, bool& unfinished) {
+  const int tid = threadIdx.x;
+  const float w1 = d.wt1;
+  int pp[2][M], oo[2][M], ww[2][M];   // the node's place, its place in the other colour, its west
+  float cb[2][M], cinv[2][M], ca[2][M], cfn[2][M], cf[2][M];
+#pragma unroll
+  for (int c = 0; c < 2; ++c)
+#pragma unroll
+    for (int m = 0; m < M; ++m) {
+      const int j = tid + m * sw;
+      const bool on = j < (c ? c1 : c0);
+      const int v = on ? sm.nodes[c][j] : CW;   // (CW: row 1 of the ring's west side)
+      const int r = v & 0x7fff;
+      const int p = c * CN + r;
+      const float2 bi = sm.bi[p], af = sm.af[p];
+      pp[c][m] = on ? p : 0;                    // 0: a corner of the ring
+      oo[c][m] = (1 - c) * CN + r;
+      ww[c][m] = oo[c][m] - (v >> 15);
+      cb[c][m] = on ? bi.x : 0.f;
+      cinv[c][m] = on ? bi.y : 0.f;
+      ca[c][m] = on ? af.x : 0.f;
+      cfn[c][m] = on ? af.y : 0.f;
+      cf[c][m] = on ? sm.f[p] : 0.f;
+    }
+  int it = 0, polish = 2;   // extra sweeps after the stop test passes
+  bool more = true;
+  for (; it < d.max_inner && (more || polish > 0); ++it) {
+    if (!more) --polish;
+    // over-relaxed for the first sweeps, then plain Gauss-Seidel: at the last
+    // few ulps over-relaxation can cycle instead of meeting the stop test
+    const float om = (more && it < SOR_SWEEPS) ? SOR_OMEGA : 1.f;
+    bool changed = false;
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      float nb[M];
+#pragma unroll
+      for (int m = 0; m < M; ++m) {
+        const float* q = sm.q + ww[c][m];
+        const float* o = sm.q + oo[c][m];
+        nb[m] = ((q[0] + q[1]) + o[-CW]) + o[CW];
+      }
+#pragma unroll
+      for (int m = 0; m < M; ++m) {
+        const float fo = cf[c][m];
+        const float raw = (cb[c][m] - w1 * nb[m]) * cinv[c][m];
+        float v = (om == 1.f) ? raw : fo + om * (raw - fo);
+        v = fminf(fmaxf(v, 0.f), 1.f);
+        // converged at about four ulps of v and of the terms that make it
+        const float tol =
+            4.8e-7f * (v + (fabsf(cb[c][m]) + w1 * fabsf(nb[m])) * cinv[c][m]);
+        changed |= fabsf(v - fo) > tol;
+        cf[c][m] = v;
+        // (a (v - f_l(n)) is exactly 0 on a node that does not move: a
+        // spurious source there would cost a rounding of its neighbours'
+        // 16-bit populations in the commit)
+        sm.q[pp[c][m]] = ca[c][m] * (v - cfn[c][m]);
+      }
+      if (c == 0) {
+        if (sw == 32) __syncwarp();
+        else sub_sync(sw);
+      }
+    }
+    // the second colour's barrier also collects the convergence vote
+    bool any;
+    if (sw == 32) {
+      any = __any_sync(0xffffffffu, changed);
+      __syncwarp();
+    } else {
+      any = sub_sync_or(sw, changed);
+    }
+    if (more) more = any;
+  }
+#pragma unroll
+  for (int c = 0; c < 2; ++c)
+#pragma unroll
+    for (int m = 0; m < M; ++m)
+      if (pp[c][m] != 0) sm.f[pp[c][m]] = cf[c][m];
+  sweeps = it;
+  unfinished = more;
+}
+
 // One listed tile.  EB threads in rows of RE: a thread's nodes lie one above
 // the other, an even number of rows apart, so they share a column and a colour
-// and every index follows from the first by a constant.  During the sweeps a
-// thread holds up to NC nodes of either colour in registers.
+// and every index follows from the first by a constant.
+//
+// listed: null for a tile known to be listed; else where its stamp is, read
+// beside the tile's nodes (which a tile not listed then reads for nothing).
 template <int PAR, typename S>
-__device__ __forceinline__ void solve_tile(const Dev& d, SolveSmem& sm, int tile, int stamp) {
+__device__ __forceinline__ void solve_tile(const Dev& d, SolveSmem& sm, int tile, int ctr,
+                                           const int* listed) {
   constexpr int LAYOUT = 1 - PAR;
   constexpr int RT = EB / RE;                      // rows the CTA covers at once
   constexpr int NK = RE / RT;                      // nodes of a thread
-  constexpr int NC = (CHALF + EB - 1) / EB;
+  static_assert(2 * EB >= CHALF, "room for every node");
   static_assert(EB % RE == 0 && RE % RT == 0 && RT % 2 == 0 && EB % 32 == 0, "block size");
   constexpr unsigned FULL = 0xffffffffu;
   const int tid = threadIdx.x, lane = tid & 31;
@@ -210,6 +303,13 @@ __device__ __forceinline__ void solve_tile(const Dev& d, SolveSmem& sm, int tile
       }
       if (out) off |= 1u << j;
     }
+  }
+  if (listed) {
+    const int at = *listed;
+    // (the values are wanted here: the loads stay above the branch)
+#pragma unroll
+    for (int j = 0; j < NK; ++j) asm volatile("" ::"f"(fnv[j]), "f"(av[j]), "f"(Tv[j]));
+    if (at != ctr) return;
   }
   float bv[NK], iv[NK];
 #pragma unroll
@@ -294,75 +394,14 @@ __device__ __forceinline__ void solve_tile(const Dev& d, SolveSmem& sm, int tile
   }
   __syncthreads();
   const int c0 = sm.cnt[0], c1 = sm.cnt[1], most = max(c0, c1);
-  // the sweeps run on as many whole warps as the larger colour needs; the
-  // other warps wait at the barrier after them
-  const int sw = min(EB, (most + 31) & ~31);
   int it = 0;
-  bool more = sw > 0;   // (nothing left to sweep: solved by the fixing pass)
-  int polish = more ? 2 : 0;   // extra sweeps after the stop test passes
-  if (tid < sw) {
-    // each sweeping thread keeps its nodes' coefficients and current values in
-    // registers, so that a sweep only exchanges q through shared memory
-    int kk[2][NC];
-    float cb[2][NC], cinv[2][NC], ca[2][NC], cfn[2][NC], cf[2][NC];
-#pragma unroll
-    for (int c = 0; c < 2; ++c)
-#pragma unroll
-      for (int m = 0; m < NC; ++m) {
-        const int j = tid + m * EB;
-        const bool on = j < (c ? c1 : c0);
-        const int v = on ? sm.nodes[c][j] : 0;
-        const int p = c * CN + (v & 0x7fff);
-        const float2 bi = sm.bi[p], af = sm.af[p];
-        kk[c][m] = on ? (p | (v & 0x8000)) : -1;   // (2 CN < 2^15)
-        cb[c][m] = bi.x;
-        cinv[c][m] = bi.y;
-        ca[c][m] = af.x;
-        cfn[c][m] = af.y;
-        cf[c][m] = sm.f[p];
-      }
-    for (; it < d.max_inner && (more || polish > 0); ++it) {
-      if (!more) --polish;
-      // over-relaxed for the first sweeps, then plain Gauss-Seidel: at the last
-      // few ulps over-relaxation can cycle instead of meeting the stop test
-      const float om = (more && it < SOR_SWEEPS) ? SOR_OMEGA : 1.f;
-      bool changed = false;
-#pragma unroll
-      for (int c = 0; c < 2; ++c) {
-#pragma unroll
-        for (int m = 0; m < NC; ++m) {
-          if (m > 0 && m * EB >= most) break;   // (the same in every thread)
-          const int k = kk[c][m];
-          if (k >= 0) {
-            const int p = k & 0x7fff;
-            const int o = c ? p - CN : p + CN, w = o - (k >> 15);
-            const float nb = ((sm.q[w] + sm.q[w + 1]) + sm.q[o - CW]) + sm.q[o + CW];
-            const float fo = cf[c][m];
-            const float raw = (cb[c][m] - w1 * nb) * cinv[c][m];
-            float v = (om == 1.f) ? raw : fo + om * (raw - fo);
-            v = fminf(fmaxf(v, 0.f), 1.f);
-            // converged at about four ulps of v and of the terms that make it
-            const float tol =
-                4.8e-7f * (v + (fabsf(cb[c][m]) + w1 * fabsf(nb)) * cinv[c][m]);
-            if (fabsf(v - fo) > tol) changed = true;
-            cf[c][m] = v;
-            // (a (v - f_l(n)) is exactly 0 on a node that does not move: a
-            // spurious source there would cost a rounding of its neighbours'
-            // 16-bit populations in the commit)
-            sm.q[p] = ca[c][m] * (v - cfn[c][m]);
-          }
-        }
-        // the second colour's barrier also collects the convergence vote
-        if (c == 0) sub_sync(sw);
-      }
-      const bool c = sub_sync_or(sw, changed);
-      if (more) more = c;
-    }
-#pragma unroll
-    for (int c = 0; c < 2; ++c)
-#pragma unroll
-      for (int m = 0; m < NC; ++m)
-        if (kk[c][m] >= 0) sm.f[kk[c][m] & 0x7fff] = cf[c][m];
+  bool more = most > 0;   // (nothing left to sweep: solved by the fixing pass)
+  if (most <= EB) {
+    const int sw = min(EB, (most + 31) & ~31);
+    if (tid < sw) sweep_nodes<1>(d, sm, c0, c1, sw, it, more);
+  } else {
+    const int sw = min(EB, 32 * ((most + 63) / 64));
+    if (tid < sw) sweep_nodes<2>(d, sm, c0, c1, sw, it, more);
   }
   __syncthreads();
   unsigned ch = 0u;
@@ -385,7 +424,7 @@ __device__ __forceinline__ void solve_tile(const Dev& d, SolveSmem& sm, int tile
     }
     atomicAdd(&d.stats[1], 1);
     atomicMax(&d.stats[2], it);
-    d.proc[tile] = (stamp << 3) | 1 | sm.bits;
+    d.proc[tile] = ((ctr & 0x0FFFFFFF) << 3) | 1 | sm.bits;
   }
   __syncthreads();
 }
@@ -406,7 +445,6 @@ __device__ __forceinline__ void enthalpy_solve_body(const Dev& d, int bid, int n
   SolveSmem& sm = *reinterpret_cast<SolveSmem*>(solve_smem);
   const int tid = threadIdx.x;
   const int ctr = d.ctr[PAR];
-  const int stamp = ctr & 0x0FFFFFFF;
   // the ring: no node there, a = q = 0
   for (int k = tid; k < 4 * (RE + 2); k += EB) {
     const int e = k / (RE + 2), i = k - e * (RE + 2);
@@ -415,16 +453,18 @@ __device__ __forceinline__ void enthalpy_solve_body(const Dev& d, int bid, int n
     sm.af[p] = make_float2(0.f, 0.f);
     sm.q[p] = 0.f;
   }
-  if (d.ntiles > COUNT_TILES) {   // the stream-collide pass kept a list
+  if (d.ntiles <= nblk) {   // a CTA for every tile: whose it is needs no count
+    if (bid < d.ntiles) solve_tile<PAR, S>(d, sm, bid, ctr, d.flags + PAR * d.ntiles + bid);
+  } else if (d.ntiles > COUNT_TILES) {   // the stream-collide pass kept a list
     int tile = bid < d.ntiles ? d.list[PAR * d.ntiles + bid] : 0;
     const int cnt = d.lcount[PAR];
     for (int li = bid; li < cnt; li += nblk) {
       if (li != bid) tile = d.list[PAR * d.ntiles + li];
-      solve_tile<PAR, S>(d, sm, tile, stamp);
+      solve_tile<PAR, S>(d, sm, tile, ctr, nullptr);
     }
   } else {
     const int rank = count_tiles<PAR>(d, sm, ctr, bid, nblk);
-    for (int i = 0; i < sm.mine; ++i) solve_tile<PAR, S>(d, sm, sm.tile[i], stamp);
+    for (int i = 0; i < sm.mine; ++i) solve_tile<PAR, S>(d, sm, sm.tile[i], ctr, nullptr);
     if (tid == 0 && bid == 0) d.lcount[PAR] = rank;
   }
   if (tid == 0 && d.trace) trace_end(d, 100 * PAR + 20, ctr, tr0);
@@ -482,12 +522,15 @@ __device__ __forceinline__ void enthalpy_commit_body(const Dev& d, int bid, int 
   __shared__ unsigned char ssolved[RW * RW];
   static_assert(CB == TE * TE, "one thread per node of a tile");
   const int tid = threadIdx.x;
-  // (the first tile's number is read beside the count; a CTA without a tile
-  // reads a place of the list that is not in use)
-  int tile = bid < d.ntiles ? d.list[PAR * d.ntiles + bid] : 0;
-  const int cnt = d.lcount[PAR];
-  const int stamp = stamp_of(d, PAR);
+  // as in the solve: a CTA for every tile (tile bid, if it is listed), or the
+  // step's list, whose first entry is read beside the count (a CTA without a
+  // tile reads a place of the list that is not in use)
+  const bool direct = d.ntiles <= nblk;
+  const int at = bid < d.ntiles ? (direct ? d.flags : d.list)[PAR * d.ntiles + bid] : 0;
+  const int ctr = d.ctr[PAR], stamp = ctr & 0x0FFFFFFF;
+  const int cnt = direct ? d.ntiles : d.lcount[PAR];
   const int n = (int)d.n;
+  int tile = direct ? bid : at;
   for (int li = bid; li < cnt; li += nblk) {
     if (li != bid) tile = d.list[PAR * d.ntiles + li];
     const int tx0 = tile % d.etx, ty0 = tile / d.etx;
@@ -504,20 +547,19 @@ __device__ __forceinline__ void enthalpy_commit_body(const Dev& d, int bid, int 
     const int pb = d.proc[tile] & 7;
     // flow links need attention only around tiles where a node's activity
     // changed (nine threads look at the tile and those around it)
-    bool lk = false;
-    if (LAYOUT == 1 && d.flow) {
-      bool l = false;
-      if (tid < 9) {
-        int tx = tx0 + tid % 3 - 1, ty = ty0 + tid / 3 - 1;
-        if (d.per_x) tx = tx < 0 ? d.etx - 1 : tx >= d.etx ? 0 : tx;
-        if (d.per_y) ty = ty < 0 ? d.ety - 1 : ty >= d.ety ? 0 : ty;
-        if (tx >= 0 && tx < d.etx && ty >= 0 && ty < d.ety) {
-          const int v = d.proc[ty * d.etx + tx];
-          l = (v >> 3) == stamp && (v & 4);
-        }
-      }
-      lk = __syncthreads_or(l);
+    int around = 0;
+    if (LAYOUT == 1 && d.flow && tid < 9) {
+      int tx = tx0 + tid % 3 - 1, ty = ty0 + tid / 3 - 1;
+      if (d.per_x) tx = tx < 0 ? d.etx - 1 : tx >= d.etx ? 0 : tx;
+      if (d.per_y) ty = ty < 0 ? d.ety - 1 : ty >= d.ety ? 0 : ty;
+      if (tx >= 0 && tx < d.etx && ty >= 0 && ty < d.ety) around = d.proc[ty * d.etx + tx];
     }
+    if (direct) {   // (the reads above stay above the branch)
+      asm volatile("" ::"f"(p.x), "f"(ph), "r"(pb), "r"(around));
+      if (at != ctr) break;
+    }
+    bool lk = false;
+    if (LAYOUT == 1 && d.flow) lk = __syncthreads_or((around >> 3) == stamp && (around & 4));
     if ((pb & 2) || lk) {
       if (lk) {
         // old/new liquid fraction of the tile and its ring: scratch in tiles
