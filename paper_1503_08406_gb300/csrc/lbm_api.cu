@@ -512,21 +512,16 @@ static int capture_body(lbm_ctx* c, int steps, int start = 0, const Hooks* hooks
   int nl = 0;
   for (int k = 0; k < steps; ++k) {
     const int par = (start + k) & 1;
-    const int fw = c->d.flow && c->d.flow_walls ? 1 : 0;   // a flow-wall pass before each pass
     if (k == 0) {
-      lbm::launch_flow_walls(c->d, par, 0, c->cap);
       lbm::launch_fused(c->d, c->tma(), par, 0, c->cap);
     } else {
-      lbm::launch_flow_walls(c->d, par, 2, c->cap);
       lbm::launch_fused(c->d, c->tma(), par, 2, c->cap);       // near tiles, after the last commit
       cudaStreamWaitEvent(c->cap, c->ev_join, 0);    // and the far tiles
     }
-    nl += 1 + fw;
+    nl += 1;
     if (k + 1 < steps) {
       cudaEventRecord(c->ev_fork, c->cap);
       cudaStreamWaitEvent(c->cap2, c->ev_fork, 0);
-      lbm::launch_flow_walls(c->d, 1 - par, 1, c->cap2);
-      nl += fw;
       lbm::launch_fused(c->d, c->tma(), 1 - par, 1, c->cap2);  // next step, far tiles
       cudaEventRecord(c->ev_join, c->cap2);
       nl += 1;
@@ -605,7 +600,6 @@ static int step_direct(lbm_ctx* c) {
     }
     cudaEventRecord(e[0], c->stream);
   }
-  lbm::launch_flow_walls(c->d, c->parity, 0, c->stream);
   lbm::launch_fused(c->d, c->tma(), c->parity, 0, c->stream);
   if (c->timing) {
     cudaEventRecord(e[1], c->stream);
@@ -617,7 +611,7 @@ static int step_direct(lbm_ctx* c) {
   if (c->timing) cudaEventRecord(e[4], c->stream);
   c->parity ^= 1;
   c->steps++;
-  c->launches += 3 + (c->d.flow && c->d.flow_walls ? 1 : 0);
+  c->launches += 3;
   return LBM_OK;
 }
 
@@ -1787,7 +1781,6 @@ int lbm_adjoint_coupled(lbm_ctx* c, int objective, int64_t nsteps, int32_t check
       } else {
         int par = 0;
         for (int64_t m = 1; m <= len; ++m) {
-          lbm::launch_flow_walls(c->d, par, 0, sm);
           lbm::launch_fused(c->d, c->tma(), par, 0, sm);
           lbm::launch_enthalpy_solve(c->d, par, sm);
           lbm::launch_enthalpy_commit(c->d, par, sm);

@@ -246,6 +246,56 @@ static __device__ __noinline__ void extrapolated_post(const Dev& d, const float 
   flow_collide(d, fb, T, fl, phi, K, fe, ub, vb);
 }
 
+// Flow walls (Sec. 4, non-equilibrium extrapolation).  A wall node x_b whose
+// inward node x_f carries flow takes, before collision, f^eq(rho_f, 0) + f(x_f) -
+// f^eq(rho_f, u_f), collides with x_f's T, f_l, phi and K, and streams like a flow
+// node; the links from its neighbours into it stream instead of reflecting.  The
+// node that x_f's update belongs to does it from what it has in registers (a
+// launch of its own before each pass read x_f's populations again and added
+// 6 us to each step's chain at 200^2): x_b only writes slots that nobody else
+// reads or writes in the step, and every neighbour of x_b lies within one node
+// of x_f.  fe: the collided populations; walls: which neighbours of (x, y) are
+// wall nodes; active: which neighbours carry flow (bit 0 the node itself).
+template <typename S, int PAR>
+static __device__ __noinline__ void store_flow_walls(const Dev& d, int x, int y, int xm, int xp,
+                                                     int ym, int yp, const float fe[9],
+                                                     unsigned walls, unsigned active,
+                                                     unsigned seed) {
+  S* F = static_cast<S*>(d.f);
+  const int n = (int)d.n, nx = d.nx;
+  for (int k = 1; k < 9; ++k) {
+    if (!((walls >> k) & 1u)) continue;
+    const int kx = ex9(k), ky = ey9(k);
+    const int wx = kx == 0 ? x : kx > 0 ? xp : xm, wy = ky == 0 ? y : ky > 0 ? yp : ym;
+    int ix, iy;
+    inward_of(d, wx, wy, ix, iy);
+    if (ix != x || iy != y) continue;   // another node's wall
+    const int sb = wy * nx + wx;
+    unsigned rnd = 0u;
+    if constexpr (!std::is_same<S, float>::value) rnd = mix32((unsigned)sb ^ seed);
+    if (PAR == 0) {
+#pragma unroll
+      for (int i = 0; i < 9; ++i) fstore(&F[opp9(i) * n + sb], fe[i], rnd);
+    } else {
+      fstore(&F[sb], fe[0], rnd);
+#pragma unroll
+      for (int i = 1; i < 9; ++i) {
+        // does the receiving node carry flow?  (Two nodes away: beyond the wall.)
+        const int ox = kx + ex9(i), oy = ky + ey9(i);
+        bool a = false;
+        int z = sb;
+        if (ox >= -1 && ox <= 1 && oy >= -1 && oy <= 1) {
+          const int j = ox == 0 ? (oy == 0 ? 0 : oy > 0 ? 2 : 4)
+                        : ox > 0 ? (oy == 0 ? 1 : oy > 0 ? 5 : 8) : (oy == 0 ? 3 : oy > 0 ? 6 : 7);
+          a = (active >> j) & 1u;
+          z = (oy == 0 ? y : oy > 0 ? yp : ym) * nx + (ox == 0 ? x : ox > 0 ? xp : xm);
+        }
+        fstore(&F[a ? i * n + z : opp9(i) * n + sb], fe[i], rnd);
+      }
+    }
+  }
+}
+
 // The update of one non-wall node from its gathered inputs: fln = f_l of the
 // 3x3 neighbourhood (-1 on walls), gin = its five thermal populations, f = its
 // nine flow populations as streamed from the neighbours, fb = (odd steps) the
@@ -294,16 +344,21 @@ __device__ __forceinline__ bool node_update(const Dev& d, int x, int y, const Ge
       // links into non-flow lattice nodes (the front; walls keep their own
       // rule): what arrives from the solid node is its extrapolated population
       // in place of our reflected one, in the same slot
-      unsigned fm = 0u;
+      unsigned fm = 0u, am = 1u, wm = 0u;   // such links; active neighbours; walls this node feeds
 #pragma unroll
-      for (int i = 1; i < 9; ++i)
-        if (!act[i] && !(EDGE && q.wl[i])) fm |= 1u << i;
-      if (fm) {
+      for (int i = 1; i < 9; ++i) {
+        const bool wall = EDGE && q.wl[i];
+        if (act[i]) am |= 1u << i;
+        else if (d.flow_front && !wall) fm |= 1u << i;
+        if (wall && d.flow_walls) wm |= 1u << i;
+      }
+      if (fm || wm) {
         float fe[9];
         extrapolated_post(d, f, T, flc, phi, K, ux, uy, fe);
 #pragma unroll
         for (int i = 1; i < 9; ++i)
           if ((fm >> i) & 1u) fp[i] = fe[opp9(i)];
+        if (EDGE && wm) store_flow_walls<S, PAR>(d, x, y, q.xm, q.xp, q.ym, q.yp, fe, wm, am, seed);
       }
     }
     if (PAR == 0) {
@@ -445,133 +500,6 @@ __device__ __forceinline__ bool takes_tile(const Dev& d, int et, int prev) {
   return (MODE == 2) == near_listed(d, et, 1 - PAR, prev);
 }
 
-// ---- flow walls (Sec. 4, non-equilibrium extrapolation) ---------------------
-//
-// With flow walls on, a wall node x_b whose inward node x_f carries flow takes,
-// before collision, f^eq(rho_f, 0) + f(x_f) - f^eq(rho_f, u_f) (rho, u and
-// varphi of x_f; the u-terms of Eq. (29) only, since f^eq's rho-term cancels),
-// collides with x_f's T, f_l, phi and K, and streams like a flow node; the
-// links from its neighbours into it stream instead of reflecting.  This kernel
-// does that for the wall nodes, one thread each, before the step's
-// stream-collide pass overwrites x_f's populations (in the AA pattern a node
-// reads and writes the same slots, and x_b only writes slots that nobody else
-// reads or writes in the step).  MODE 1 / 2 take the wall nodes whose x_f lies
-// in a far / near enthalpy tile, as the split stream-collide passes do.
-template <typename S, int PAR, int MODE>
-__global__ void __launch_bounds__(256) flow_wall_kernel(Dev d) {
-  const int nx = d.nx, ny = d.ny, n = (int)d.n;
-  const int nbot = d.wall_b ? nx : 0, ntop = d.wall_t ? nx : 0;
-  const int ylo = d.wall_b ? 1 : 0, yhi = d.wall_t ? ny - 1 : ny;
-  const int nleft = d.wall_l ? yhi - ylo : 0, nright = d.wall_r ? yhi - ylo : 0;
-  const int total = nbot + ntop + nleft + nright;
-  S* F = static_cast<S*>(d.f);
-  const S* G = static_cast<const S*>(d.g);
-  const float r0 = d.wt0 * d.g_ref, r1 = d.wt1 * d.g_ref;
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < total; k += gridDim.x * blockDim.x) {
-    int x, y, kk = k;
-    if (kk < nbot) {
-      x = kk;
-      y = 0;
-    } else if ((kk -= nbot) < ntop) {
-      x = kk;
-      y = ny - 1;
-    } else if ((kk -= ntop) < nleft) {
-      x = 0;
-      y = ylo + kk;
-    } else {
-      x = nx - 1;
-      y = ylo + kk - nleft;
-    }
-    int ix, iy;
-    inward_of(d, x, y, ix, iy);
-    if (is_wall(d, ix, iy)) continue;   // a lattice too narrow to have an inward node
-    const int sf = iy * nx + ix;
-    const float flf = d.fl[sf];
-    if (flf < d.f_act) continue;   // the inward node carries no flow: the wall reflects
-    if (MODE != 0 && !takes_tile<PAR, MODE>(d, (iy / TE) * d.etx + ix / TE, d.ctr[1 - PAR]))
-      continue;
-    // x_f's populations before the step's collision, as its own update reads them
-    float f[9], g[5];
-    if (PAR == 0) {
-#pragma unroll
-      for (int i = 0; i < 9; ++i) f[i] = Pop<S>::ld(&F[i * n + sf]);
-#pragma unroll
-      for (int i = 0; i < 5; ++i) g[i] = gload(&G[i * n + sf], i ? r1 : r0);
-    } else {
-      f[0] = Pop<S>::ld(&F[sf]);
-#pragma unroll
-      for (int i = 1; i < 9; ++i) {
-        const int sx = wrapx(d, ix - ex9(i)), sy = wrapy(d, iy - ey9(i));
-        bool a;   // does the source node carry flow?
-        if (is_wall(d, sx, sy)) {
-          int jx, jy;
-          inward_of(d, sx, sy, jx, jy);
-          a = d.fl[jy * nx + jx] >= d.f_act;
-        } else {
-          a = d.fl[sy * nx + sx] >= d.f_act;
-        }
-        f[i] = a ? Pop<S>::ld(&F[opp9(i) * n + sy * nx + sx]) : Pop<S>::ld(&F[i * n + sf]);
-      }
-      g[0] = gload(&G[sf], r0);
-#pragma unroll
-      for (int i = 1; i < 5; ++i) {
-        const int sx = wrapx(d, ix - ex9(i)), sy = wrapy(d, iy - ey9(i));
-        g[i] = gload(&G[opp5(i) * n + sy * nx + sx], r1);
-      }
-    }
-    const float T = g[0] + g[1] + g[2] + g[3] + g[4];
-    const float phi = d.phi[sf], K = d.K[sf];
-    const float jx = f[1] - f[3] + f[5] - f[6] - f[7] + f[8];
-    const float jy = f[2] - f[4] + f[5] + f[6] - f[7] - f[8];
-    float ux, uy, Fx, Fy;
-    velocity(jx, jy, T, flf, phi, K, d, ux, uy, Fx, Fy);
-    float fp[9];
-    extrapolated_post(d, f, T, flf, phi, K, ux, uy, fp);
-    const int sb = y * nx + x;
-    unsigned rnd = 0u;
-    if constexpr (!std::is_same<S, float>::value)
-      rnd = mix32((unsigned)sb ^ mix32((unsigned)d.ctr[1 - PAR]));
-    if (PAR == 0) {
-#pragma unroll
-      for (int i = 0; i < 9; ++i) fstore(&F[opp9(i) * n + sb], fp[i], rnd);
-    } else {
-      fstore(&F[sb], fp[0], rnd);
-#pragma unroll
-      for (int i = 1; i < 9; ++i) {
-        const int zx = wrapx(d, x + ex9(i)), zy = wrapy(d, y + ey9(i));
-        bool a = false;   // does the receiving node carry flow?
-        if (zx >= 0 && zy >= 0) {
-          if (is_wall(d, zx, zy)) {
-            int jx2, jy2;
-            inward_of(d, zx, zy, jx2, jy2);
-            a = d.fl[jy2 * nx + jx2] >= d.f_act;
-          } else {
-            a = d.fl[zy * nx + zx] >= d.f_act;
-          }
-        }
-        fstore(&F[a ? i * n + zy * nx + zx : opp9(i) * n + sb], fp[i], rnd);
-      }
-    }
-  }
-}
-
-template <typename S>
-static void launch_flow_walls_t(const Dev& d, int parity, int mode, cudaStream_t s) {
-  const int total = 2 * (d.nx + d.ny);
-  const int grid = (total + 255) / 256;
-#define LBM_FW(P, M) flow_wall_kernel<S, P, M><<<grid, 256, 0, s>>>(d)
-  if (parity == 0) {
-    if (mode == 0) LBM_FW(0, 0);
-    else if (mode == 1) LBM_FW(0, 1);
-    else LBM_FW(0, 2);
-  } else {
-    if (mode == 0) LBM_FW(1, 0);
-    else if (mode == 1) LBM_FW(1, 1);
-    else LBM_FW(1, 2);
-  }
-#undef LBM_FW
-}
-
 // ---- ordinary-load kernel ----------------------------------------------------
 
 template <typename S, int PAR, int FLOW, int MODE>
@@ -636,7 +564,7 @@ __global__ void __launch_bounds__(TX* TY, 4) fused_step_kernel(Dev d) {
       }
     }
     unsigned wact = 0u;
-    if (FLOW && d.flow_walls)
+    if (FLOW == 2 && d.flow_walls)
       wact = wall_activity(d, x, y, q, [&](int dx, int dy) {
         return d.fl[(long long)wrapy(d, y + dy) * nx + wrapx(d, x + dx)];
       });
@@ -813,7 +741,7 @@ __device__ __forceinline__ bool tma_node(const Dev& d, const unsigned char* sb, 
         }
       }
       unsigned wact = 0u;
-      if (FLOW && EDGE && d.flow_walls)
+      if (FLOW == 2 && EDGE && d.flow_walls)
         wact = wall_activity(d, x, y, q, [&](int dx, int dy) { return sFL[c + dy * WX + dx]; });
       unsafe = node_update<S, PAR, FLOW, EDGE>(d, x, y, q, fln, g, f, fb, phi, K, wact, seed, stamp);
   }
@@ -963,10 +891,11 @@ __global__ void __launch_bounds__(TX* TY, TMA_MIN_CTAS)
 
 // ---- launches ------------------------------------------------------------------
 
-// FLOW: 0 no flow lattice, 1 flow, 2 flow with the front extrapolation
+// FLOW: 0 no flow lattice, 1 flow, 2 flow with extrapolated walls or front (a
+// variant of its own, which leaves the common one's registers alone)
 template <typename S, int MODE>
 static void launch_mode(const Dev& d, int parity, dim3 grid, dim3 block, cudaStream_t s) {
-  if (d.flow && d.flow_front) {
+  if (d.flow && (d.flow_front || d.flow_walls)) {
     if (parity == 0) fused_step_kernel<S, 0, 2, MODE><<<grid, block, 0, s>>>(d);
     else fused_step_kernel<S, 1, 2, MODE><<<grid, block, 0, s>>>(d);
   } else if (d.flow) {
@@ -986,7 +915,7 @@ static void launch_tma_one(const Dev& d, const TmaMaps& m, cudaStream_t s) {
 
 template <typename S, int MODE>
 static void launch_tma_mode(const Dev& d, const TmaMaps& m, int parity, cudaStream_t s) {
-  if (d.flow && d.flow_front) {
+  if (d.flow && (d.flow_front || d.flow_walls)) {
     if (parity == 0) launch_tma_one<S, 0, 2, MODE>(d, m, s);
     else launch_tma_one<S, 1, 2, MODE>(d, m, s);
   } else if (d.flow) {

@@ -432,10 +432,6 @@ void launch_nonfinite(const Dev& d, int nblocks, cudaStream_t s);
 // one CTA waiting, with a limit of limit_ns, on an mbarrier nothing completes
 // (sets stats[4] when the wait gives up, as a timed-out bulk copy does)
 void launch_wait_probe(const Dev& d, long long limit_ns, cudaStream_t s);
-// the wall nodes' flow update when flow walls are on (mode as for launch_fused,
-// by the enthalpy tile of each wall node's inward node); runs before the
-// stream-collide pass of the same step and mode
-void launch_flow_walls(const Dev& d, int parity, int mode, cudaStream_t s);
 void launch_validate(const Dev& d, const float* phi, const float* K, const float* T0,
                      const float* fl0, int* bad, cudaStream_t s);
 
