@@ -444,6 +444,7 @@ __device__ __forceinline__ void enthalpy_solve_body(const Dev& d, int bid, int n
   extern __shared__ __align__(16) unsigned char solve_smem[];
   SolveSmem& sm = *reinterpret_cast<SolveSmem*>(solve_smem);
   const int tid = threadIdx.x;
+  if (d.ntiles <= nblk) allow_dependents();
   const int ctr = d.ctr[PAR];
   // the ring: no node there, a = q = 0
   for (int k = tid; k < 4 * (RE + 2); k += EB) {
@@ -526,9 +527,19 @@ __device__ __forceinline__ void enthalpy_commit_body(const Dev& d, int bid, int 
   // step's list, whose first entry is read beside the count (a CTA without a
   // tile reads a place of the list that is not in use)
   const bool direct = d.ntiles <= nblk;
-  const int at = bid < d.ntiles ? (direct ? d.flags : d.list)[PAR * d.ntiles + bid] : 0;
   const int ctr = d.ctr[PAR], stamp = ctr & 0x0FFFFFFF;
-  const int cnt = direct ? d.ntiles : d.lcount[PAR];
+  int at = 0, cnt = d.ntiles;
+  if (direct) {
+    allow_dependents();
+    // the pass before the solve stamped the tiles: a CTA without one is done
+    if (bid < d.ntiles) at = d.flags[PAR * d.ntiles + bid];
+    if (bid != 0 && at != ctr) cnt = 0;
+    else wait_for_previous();
+    if (at != ctr) cnt = 0;
+  } else {
+    if (bid < d.ntiles) at = d.list[PAR * d.ntiles + bid];
+    cnt = d.lcount[PAR];
+  }
   const int n = (int)d.n;
   int tile = direct ? bid : at;
   for (int li = bid; li < cnt; li += nblk) {
@@ -553,10 +564,6 @@ __device__ __forceinline__ void enthalpy_commit_body(const Dev& d, int bid, int 
       if (d.per_x) tx = tx < 0 ? d.etx - 1 : tx >= d.etx ? 0 : tx;
       if (d.per_y) ty = ty < 0 ? d.ety - 1 : ty >= d.ety ? 0 : ty;
       if (tx >= 0 && tx < d.etx && ty >= 0 && ty < d.ety) around = d.proc[ty * d.etx + tx];
-    }
-    if (direct) {   // (the reads above stay above the branch)
-      asm volatile("" ::"f"(p.x), "f"(ph), "r"(pb), "r"(around));
-      if (at != ctr) break;
     }
     bool lk = false;
     if (LAYOUT == 1 && d.flow) lk = __syncthreads_or((around >> 3) == stamp && (around & 4));
@@ -744,15 +751,22 @@ void launch_enthalpy_commit_batch(const BatchPlan& P, int parity, cudaStream_t s
   else enthalpy_commit_batch_kernel<1><<<grid, CB, 0, s>>>(P);
 }
 
+template <int PAR, bool WALLS>
+static void launch_commit_one(const Dev& d, cudaStream_t s) {
+  if (early_launches(d))
+    launch_early(enthalpy_commit_kernel<PAR, WALLS>, dim3(d.cgrid), dim3(CB), 0, s, d);
+  else enthalpy_commit_kernel<PAR, WALLS><<<d.cgrid, CB, 0, s>>>(d);
+}
+
 void launch_enthalpy_commit(const Dev& d, int parity, cudaStream_t s) {
   // flow walls add their links to the re-pairing (a variant of its own, which
   // leaves the common one's registers alone)
   if (d.flow && d.flow_walls) {
-    if (parity == 0) enthalpy_commit_kernel<0, true><<<d.cgrid, CB, 0, s>>>(d);
-    else enthalpy_commit_kernel<1, true><<<d.cgrid, CB, 0, s>>>(d);
+    if (parity == 0) launch_commit_one<0, true>(d, s);
+    else launch_commit_one<1, true>(d, s);
   } else {
-    if (parity == 0) enthalpy_commit_kernel<0, false><<<d.cgrid, CB, 0, s>>>(d);
-    else enthalpy_commit_kernel<1, false><<<d.cgrid, CB, 0, s>>>(d);
+    if (parity == 0) launch_commit_one<0, false>(d, s);
+    else launch_commit_one<1, false>(d, s);
   }
 }
 

@@ -507,14 +507,18 @@ __global__ void __launch_bounds__(TX* TY, 4) fused_step_kernel(Dev d) {
   constexpr unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x;
   const int prev = d.ctr[1 - PAR], stamp = prev + 1;   // (no launch of this step changes it)
-  if (MODE != 1 && blockIdx.x == 0 && blockIdx.y == 0 && lane == 0 && threadIdx.y == 0)
-    step_prologue<PAR>(d);
+  const bool first = blockIdx.x == 0 && blockIdx.y == 0;
+  if (MODE != 1 && first) {
+    if (MODE == 2) wait_for_previous();
+    if (lane == 0 && threadIdx.y == 0) step_prologue<PAR>(d);
+  }
   if (MODE != 0) {   // (one tile per CTA: a warp's first nine lanes look at its surroundings)
     const int et = ((blockIdx.y * TY) / TE) * d.etx + (blockIdx.x * TX) / TE;
     const bool hit = d.ntiles > COUNT_TILES
                          ? lane == 0 && d.nearmap[(1 - PAR) * d.ntiles + et] == prev
                          : lane < 9 && listed_at(d, et, lane, 1 - PAR, prev);
     if ((MODE == 2) != __any_sync(FULL, hit)) return;
+    if (MODE == 2) wait_for_previous();
   }
   const int x = blockIdx.x * TX + lane, y = blockIdx.y * TY + threadIdx.y;
   const int nx = d.nx, ny = d.ny;
@@ -773,7 +777,6 @@ __device__ __forceinline__ void fused_tma_body(const Dev& d, const TmaMaps& m, i
   const int prev = d.ctr[1 - PAR];   // the previous step's stamp (no launch of this step changes it)
   // 16-bit storage: the step's part of every node's rounding seed
   const unsigned seed = std::is_same<S, float>::value ? 0u : mix32((unsigned)prev);
-  if (MODE != 1 && bid == 0 && tid == 0) step_prologue<PAR>(d);
   constexpr int NB = L::NBUF;
   const unsigned buf0 = smem_u32(smem);
   const unsigned bar0 = buf0 + L::BAR_OFF;   // mbarrier of buffer j: bar0 + 8 j
@@ -796,6 +799,9 @@ __device__ __forceinline__ void fused_tma_body(const Dev& d, const TmaMaps& m, i
     const int et = ((t / tiles_x) * TY / TE) * d.etx + (t % tiles_x) * TX / TE;
     bool take = lane < cnt;
     if (take && MODE != 0) take = takes_tile<PAR, MODE>(d, et, prev);
+    // (the near map is older than the kernel before this one, the state is not)
+    if (MODE == 2 && (bid == 0 || __any_sync(FULL, take))) wait_for_previous();
+    if (MODE != 1 && bid == 0 && lane == 0) step_prologue<PAR>(d);
     fmask = !FLOW ? 0u : d.tskip ? __ballot_sync(FULL, take && d.tact[et]) : ~0u;
     const unsigned mask = __ballot_sync(FULL, take);
     if (lane == 0) {
@@ -893,24 +899,34 @@ __global__ void __launch_bounds__(TX* TY, TMA_MIN_CTAS)
 
 // FLOW: 0 no flow lattice, 1 flow, 2 flow with extrapolated walls or front (a
 // variant of its own, which leaves the common one's registers alone)
+template <typename S, int PAR, int FLOW, int MODE>
+static void launch_step_one(const Dev& d, cudaStream_t s) {
+  const dim3 block(TX, TY), grid((d.nx + TX - 1) / TX, (d.ny + TY - 1) / TY);
+  if (MODE == 2 && early_launches(d))
+    launch_early(fused_step_kernel<S, PAR, FLOW, MODE>, grid, block, 0, s, d);
+  else fused_step_kernel<S, PAR, FLOW, MODE><<<grid, block, 0, s>>>(d);
+}
+
 template <typename S, int MODE>
-static void launch_mode(const Dev& d, int parity, dim3 grid, dim3 block, cudaStream_t s) {
+static void launch_mode(const Dev& d, int parity, cudaStream_t s) {
   if (d.flow && (d.flow_front || d.flow_walls)) {
-    if (parity == 0) fused_step_kernel<S, 0, 2, MODE><<<grid, block, 0, s>>>(d);
-    else fused_step_kernel<S, 1, 2, MODE><<<grid, block, 0, s>>>(d);
+    if (parity == 0) launch_step_one<S, 0, 2, MODE>(d, s);
+    else launch_step_one<S, 1, 2, MODE>(d, s);
   } else if (d.flow) {
-    if (parity == 0) fused_step_kernel<S, 0, 1, MODE><<<grid, block, 0, s>>>(d);
-    else fused_step_kernel<S, 1, 1, MODE><<<grid, block, 0, s>>>(d);
+    if (parity == 0) launch_step_one<S, 0, 1, MODE>(d, s);
+    else launch_step_one<S, 1, 1, MODE>(d, s);
   } else {
-    if (parity == 0) fused_step_kernel<S, 0, 0, MODE><<<grid, block, 0, s>>>(d);
-    else fused_step_kernel<S, 1, 0, MODE><<<grid, block, 0, s>>>(d);
+    if (parity == 0) launch_step_one<S, 0, 0, MODE>(d, s);
+    else launch_step_one<S, 1, 0, MODE>(d, s);
   }
 }
 
 template <typename S, int PAR, int FLOW, int MODE>
 static void launch_tma_one(const Dev& d, const TmaMaps& m, cudaStream_t s) {
   const size_t sm = TmaLayout<PAR, S>::SMEM;
-  fused_tma_kernel<S, PAR, FLOW, MODE><<<d.tgrid, dim3(TX, TY), sm, s>>>(d, m);
+  if (MODE == 2 && early_launches(d))
+    launch_early(fused_tma_kernel<S, PAR, FLOW, MODE>, dim3(d.tgrid), dim3(TX, TY), sm, s, d, m);
+  else fused_tma_kernel<S, PAR, FLOW, MODE><<<d.tgrid, dim3(TX, TY), sm, s>>>(d, m);
 }
 
 template <typename S, int MODE>
@@ -936,10 +952,9 @@ static void launch_fused_t(const Dev& d, const TmaMaps* m, int parity, int mode,
     else launch_tma_mode<S, 2>(d, *m, parity, s);
     return;
   }
-  dim3 block(TX, TY), grid((d.nx + TX - 1) / TX, (d.ny + TY - 1) / TY);
-  if (mode == 0) launch_mode<S, 0>(d, parity, grid, block, s);
-  else if (mode == 1) launch_mode<S, 1>(d, parity, grid, block, s);
-  else launch_mode<S, 2>(d, parity, grid, block, s);
+  if (mode == 0) launch_mode<S, 0>(d, parity, s);
+  else if (mode == 1) launch_mode<S, 1>(d, parity, s);
+  else launch_mode<S, 2>(d, parity, s);
 }
 
 // encode one tiled tensor map over a [planes][ny][nx] array of esize-byte elements
