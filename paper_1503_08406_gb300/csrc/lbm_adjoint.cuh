@@ -30,8 +30,10 @@ struct NuSrc {
   float g1, g2, tw;
 };
 // the left-wall Nusselt number of the current state (lbm_reduce's out[3]),
-// added to acc[0] (lbm_aux.cu)
-void launch_wall_nusselt(const Dev& d, int layout, double* acc, cudaStream_t s);
+// added to acc[0] (lbm_aux.cu); mode and par as for launch_keep_state: mode 1
+// leaves the terms of its rows in rows[ny], where mode 2 finds them
+void launch_wall_nusselt(const Dev& d, int layout, int mode, int par, double* rows, double* acc,
+                         cudaStream_t s);
 // a = phi dT / (sigma St); lam_g = the Nusselt terms of the last state; lam_f
 // = 1 / (non-wall nodes) on non-wall nodes for the melted fraction (melt),
 // else 0

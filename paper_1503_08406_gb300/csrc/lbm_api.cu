@@ -34,7 +34,7 @@ struct lbm_ctx {
   // CUDA graphs of 2..GRAPH_MAX steps from either step parity, captured on a
   // private stream when first needed and replayed on the context stream
   cudaStream_t cap, cap2;         // capture streams (the second one runs the far-tile fused pass)
-  cudaEvent_t ev_fork, ev_join;
+  cudaEvent_t ev_fork, ev_join, ev_read, ev_commit;
   cudaGraphExec_t gx[2][65];       // [start parity][steps], GRAPH_MAX = 64
   int gnl[2][65];                  // kernels in each graph
   bool graphs_off;
@@ -367,6 +367,8 @@ void lbm_destroy(lbm_ctx* c) {
   if (c->cap2) cudaStreamDestroy(c->cap2);
   if (c->ev_fork) cudaEventDestroy(c->ev_fork);
   if (c->ev_join) cudaEventDestroy(c->ev_join);
+  if (c->ev_read) cudaEventDestroy(c->ev_read);
+  if (c->ev_commit) cudaEventDestroy(c->ev_commit);
   for (cudaEvent_t e : c->ev) cudaEventDestroy(e);
   if (c->own_ws && c->ws) cudaFree(c->ws);
   if (c->trace_buf) cudaFree(c->trace_buf);
@@ -462,12 +464,47 @@ static bool capture_streams(lbm_ctx* c) {
     c->cap2 = nullptr;
     return false;
   }
-  if ((!c->ev_fork && cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess) ||
-      (!c->ev_join && cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) != cudaSuccess)) {
-    cudaGetLastError();
-    return false;
-  }
+  for (cudaEvent_t* e : {&c->ev_fork, &c->ev_join, &c->ev_read, &c->ev_commit})
+    if (!*e && cudaEventCreateWithFlags(e, cudaEventDisableTiming) != cudaSuccess) {
+      cudaGetLastError();
+      *e = nullptr;
+      return false;
+    }
   return true;
+}
+
+// Work an adjoint's forward run adds after every step (all optional): f_l
+// into fl_base + fl_ctr[0] n, the whole state into st_base + st_ctr[0] 15 n
+// (each counter then advances, so a graph serves every replay), and the
+// left-wall Nusselt number added to nu_acc[0] (nu_rows: ny doubles of scratch).
+struct Hooks {
+  float* fl_base = nullptr;
+  unsigned* fl_ctr = nullptr;
+  float* st_base = nullptr;
+  unsigned* st_ctr = nullptr;
+  double* nu_acc = nullptr;
+  double* nu_rows = nullptr;
+  bool state() const { return st_base || nu_acc; }   // reads populations
+};
+
+// the hooks that read populations (mode and par as for launch_keep_state)
+static int launch_state_hooks(lbm_ctx* c, const Hooks* h, int layout, int mode, int par,
+                              cudaStream_t s) {
+  int nl = 0;
+  if (h && h->st_base) {
+    lbm::launch_keep_state(c->d, layout, h->st_base, h->st_ctr, s, mode, par);
+    ++nl;
+  }
+  if (h && h->nu_acc) {
+    lbm::launch_wall_nusselt(c->d, layout, mode, par, h->nu_rows, h->nu_acc, s);
+    ++nl;
+  }
+  return nl;
+}
+static int launch_fl_hook(lbm_ctx* c, const Hooks* h, cudaStream_t s) {
+  if (!h || !h->fl_base) return 0;
+  lbm::adj_save(c->d, h->fl_base, h->fl_ctr, s);
+  return 1;
 }
 
 // Record `steps` steps starting at parity `start` on c->cap, which is being
@@ -477,37 +514,8 @@ static bool capture_streams(lbm_ctx* c) {
 // k's enthalpy solve and commit (which touch only nodes within eight nodes of a
 // listed tile); the tiles near the front run after the commit.  Everything
 // forked onto the second stream joins back before the last kernel.
-// Work an adjoint's forward run adds after every step (all optional): f_l
-// into fl_base + fl_ctr[0] n, the whole state into st_base + st_ctr[0] 15 n
-// (each counter then advances, so a graph serves every replay), and the
-// left-wall Nusselt number added to nu_acc[0].
-struct Hooks {
-  float* fl_base = nullptr;
-  unsigned* fl_ctr = nullptr;
-  float* st_base = nullptr;
-  unsigned* st_ctr = nullptr;
-  double* nu_acc = nullptr;
-  bool any() const { return fl_base || st_base || nu_acc; }
-};
-
-static int launch_hooks(lbm_ctx* c, const Hooks* h, int layout, cudaStream_t s) {
-  if (!h) return 0;
-  int nl = 0;
-  if (h->fl_base) {
-    lbm::adj_save(c->d, h->fl_base, h->fl_ctr, s);   // f_l after the step
-    ++nl;
-  }
-  if (h->st_base) {
-    lbm::launch_keep_state(c->d, layout, h->st_base, h->st_ctr, s);   // the state after it
-    ++nl;
-  }
-  if (h->nu_acc) {
-    lbm::launch_wall_nusselt(c->d, layout, h->nu_acc, s);   // Nu after the step
-    ++nl;
-  }
-  return nl;
-}
-
+// Hooks that read populations read the far tiles' before that pass and the
+// others' after the commit.
 static int capture_body(lbm_ctx* c, int steps, int start = 0, const Hooks* hooks = nullptr) {
   int nl = 0;
   for (int k = 0; k < steps; ++k) {
@@ -519,17 +527,39 @@ static int capture_body(lbm_ctx* c, int steps, int start = 0, const Hooks* hooks
       cudaStreamWaitEvent(c->cap, c->ev_join, 0);    // and the far tiles
     }
     nl += 1;
-    if (k + 1 < steps) {
+    const bool more = k + 1 < steps;
+    const bool split = more && hooks && hooks->state();
+    if (more) {
       cudaEventRecord(c->ev_fork, c->cap);
       cudaStreamWaitEvent(c->cap2, c->ev_fork, 0);
+      if (split) {
+        // the far tiles' state is final here, and their next pass overwrites it
+        nl += launch_state_hooks(c, hooks, 1 - par, 1, par, c->cap2);
+        cudaEventRecord(c->ev_read, c->cap2);
+      }
       lbm::launch_fused(c->d, c->tma(), 1 - par, 1, c->cap2);  // next step, far tiles
-      cudaEventRecord(c->ev_join, c->cap2);
       nl += 1;
     }
     lbm::launch_enthalpy_solve(c->d, par, c->cap);
     lbm::launch_enthalpy_commit(c->d, par, c->cap);
     nl += 2;
-    nl += launch_hooks(c, hooks, 1 - par, c->cap);
+    if (split) {
+      cudaStreamWaitEvent(c->cap, c->ev_read, 0);
+      nl += launch_state_hooks(c, hooks, 1 - par, 2, par, c->cap);
+    } else {
+      nl += launch_state_hooks(c, hooks, 1 - par, 0, par, c->cap);
+    }
+    if (more) {
+      // f_l is copied beside the next step's near-tile pass, before its solve
+      if (hooks && hooks->fl_base) {
+        cudaEventRecord(c->ev_commit, c->cap);
+        cudaStreamWaitEvent(c->cap2, c->ev_commit, 0);
+        nl += launch_fl_hook(c, hooks, c->cap2);
+      }
+      cudaEventRecord(c->ev_join, c->cap2);
+    } else {
+      nl += launch_fl_hook(c, hooks, c->cap);
+    }
   }
   return nl;
 }
@@ -1297,7 +1327,8 @@ struct HookGraphs {
 static int step_hooked(lbm_ctx* c, int64_t steps, const Hooks& h, HookGraphs& cache) {
   auto direct = [&]() -> int {
     LBM_TRY(step_direct(c));
-    launch_hooks(c, &h, c->parity, c->stream);
+    launch_state_hooks(c, &h, c->parity, 0, 0, c->stream);
+    launch_fl_hook(c, &h, c->stream);
     --steps;
     return LBM_OK;
   };
@@ -1377,10 +1408,11 @@ int lbm_adjoint(lbm_ctx* c, int objective, int64_t nsteps, int32_t checkpoint_ev
   int* counts = reinterpret_cast<int*>(mem.get(2));
   unsigned* ctr = reinterpret_cast<unsigned*>(mem.get(2));
   double* nu_acc = reinterpret_cast<double*>(mem.get(2));
+  double* nu_rows = reinterpret_cast<double*>(mem.get(2 * (size_t)c->d.ny));
   double* dJ = reinterpret_cast<double*>(mem.get(2 * 129));
   if (!flS || (!keep_all && (!cps || !fin)) || !b.a || !b.lamg || !b.lamf || !b.rhs ||
       !b.mu0 || !b.mu1 || !b.lamgpre || !b.lama || !b.lamtw || !b.pos || !lists[0] ||
-      !lists[1] || !counts || !ctr || !nu_acc || !dJ)
+      !lists[1] || !counts || !ctr || !nu_acc || !nu_rows || !dJ)
     return LBM_ERR_OOM;
   // transposed collision matrix with u = 0: g+ = A g,
   // A = N^-1 [(I - Theta) N + Theta e 1^T], e = (1, 0, 0, varpi, 0), Eq. (32)-(37)
@@ -1431,12 +1463,14 @@ int lbm_adjoint(lbm_ctx* c, int objective, int64_t nsteps, int32_t checkpoint_ev
     h.fl_base = flS;
     h.fl_ctr = ctr;
     h.nu_acc = acc;
+    h.nu_rows = nu_rows;
     LBM_TRY(step_hooked(c, nsteps, h, fwd_graphs));
   } else {
     // forward, keeping the whole state every K steps
     LBM_TRY(save(cps));
     Hooks h;
     h.nu_acc = acc;
+    h.nu_rows = nu_rows;
     for (int64_t j = 1; j < ncp; ++j) {
       LBM_TRY(step_hooked(c, K, h, fwd_graphs));
       LBM_TRY(save(cps + (size_t)j * st));
@@ -1603,10 +1637,11 @@ int lbm_adjoint_coupled(lbm_ctx* c, int objective, int64_t nsteps, int32_t check
   int* lists[2] = {reinterpret_cast<int*>(mem.get(n)), reinterpret_cast<int*>(mem.get(n))};
   int* counts = reinterpret_cast<int*>(mem.get(2));
   double* nu_acc = reinterpret_cast<double*>(mem.get(2));
+  double* nu_rows = reinterpret_cast<double*>(mem.get(2 * (size_t)d.ny));
   unsigned* ctr = reinterpret_cast<unsigned*>(mem.get(4));   // two counter pairs
   if (!S || (!keep_all && (!cps || !fin || !S2)) || !lf[0] || !lf[1] || !lg[0] || !lg[1] || !b.a ||
       !b.lamf || !b.rhs || !b.mu0 || !b.mu1 || !b.lama || !b.lamtw || !b.pos || !lK ||
-      !lists[0] || !lists[1] || !counts || !nu_acc || !ctr)
+      !lists[0] || !lists[1] || !counts || !nu_acc || !nu_rows || !ctr)
     return LBM_ERR_OOM;
   // rows of the Nusselt number (lbm_reduce's): all but horizontal wall rows
   const int y0 = d.wall_b ? 1 : 0, y1 = d.wall_t ? d.ny - 1 : d.ny;
@@ -1615,6 +1650,7 @@ int lbm_adjoint_coupled(lbm_ctx* c, int objective, int64_t nsteps, int32_t check
   HookGraphs fwd_graphs;
   Hooks h;
   h.nu_acc = melt ? nullptr : nu_acc;
+  h.nu_rows = nu_rows;
   PhaseEvents ph(c);
   ph.mark(0);
   LBM_CUDA(cudaMemsetAsync(nu_acc, 0, sizeof(double), c->stream));

@@ -270,19 +270,35 @@ __global__ void __launch_bounds__(RB) reduce_kernel(Dev d, int layout, double* p
   if (tid < 6) partials[blockIdx.x * 6 + tid] = sh[tid][0];
 }
 
+// Does this part of a split read-out (mode 0 all, 1 tiles away from the front,
+// 2 tiles near it, by the step of parity par just taken) take tile t?
+__device__ __forceinline__ bool takes_part(const Dev& d, int mode, int par, int t) {
+  return mode == 0 || (mode == 2) == near_listed(d, t, par, d.ctr[par]);
+}
+
 // The left-wall Nusselt number of the current state (the rows and the
 // formula of reduce_kernel), added to acc[0]; one block, fixed summation order.
-__global__ void __launch_bounds__(RB) wall_nusselt_kernel(Dev d, int layout, double* acc) {
+// Mode 1 leaves its rows' terms in rows[], where mode 2 finds them.
+__global__ void __launch_bounds__(RB) wall_nusselt_kernel(Dev d, int layout, int mode, int par,
+                                                          double* rows, double* acc) {
   __shared__ double sh[RB];
   const int tid = threadIdx.x;
   const int y0 = d.wall_b ? 1 : 0, y1 = d.wall_t ? d.ny - 1 : d.ny;
   double v = 0.0;
   if (d.wall_l && d.nx >= 3)
     for (int y = y0 + tid; y < y1; y += RB) {
-      const double T0 = node_T(d, 0, y, layout), T1 = node_T(d, 1, y, layout),
-                   T2 = node_T(d, 2, y, layout);
-      v += -(-3.0 * T0 + 4.0 * T1 - T2) * 0.5 * (double)d.H_over_dT;
+      double r;
+      if (takes_part(d, mode, par, (y / TE) * d.etx)) {
+        const double T0 = node_T(d, 0, y, layout), T1 = node_T(d, 1, y, layout),
+                     T2 = node_T(d, 2, y, layout);
+        r = -(-3.0 * T0 + 4.0 * T1 - T2) * 0.5 * (double)d.H_over_dT;
+        if (mode == 1) rows[y] = r;
+      } else {
+        r = mode == 2 ? rows[y] : 0.0;
+      }
+      v += r;
     }
+  if (mode == 1) return;
   sh[tid] = v;
   __syncthreads();
   for (int w = RB / 2; w > 0; w >>= 1) {
@@ -361,16 +377,24 @@ __global__ void validate_kernel(Dev d, const float* phi, const float* K, const f
   if (!ok) atomicExch(bad, 1);
 }
 
-// The whole state in natural layout (f as deviations, 9 planes; g, 5 planes;
-// f_l) into dst, 15 n floats; with ctr non-null into base + ctr[0] 15 n, after
-// which ctr[0] advances (ctr[1]: 0, scratch), so one captured launch serves
-// every replay of a graph.
-__global__ void keep_state_kernel(Dev d, int layout, float* base, unsigned* ctr) {
-  const long long n = d.n;
+// The whole state of an FP32 lattice in natural layout (f as deviations, 9
+// planes; g, 5 planes; f_l) into dst, 15 n floats; with ctr non-null into base +
+// ctr[0] 15 n, after which (not in mode 1) ctr[0] advances (ctr[1]: 0, scratch),
+// so one captured launch serves every replay of a graph.  mode and par as in
+// takes_part: the next step's stream-collide pass over the far tiles may start
+// once mode 1 is done with them.
+__global__ void __launch_bounds__(256) keep_state_kernel(Dev d, int layout, int mode, int par,
+                                                         float* base, unsigned* ctr) {
+  const int n = (int)d.n, nx = d.nx;
+  const float* F = static_cast<const float*>(d.f);
+  const float* G = static_cast<const float*>(d.g);
   float* dst = base + (ctr ? (long long)ctr[0] * 15 * n : 0LL);
-  for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < n;
-       s += (long long)gridDim.x * blockDim.x) {
-    const int y = (int)(s / d.nx), x = (int)(s - (long long)y * d.nx);
+  const int x = blockIdx.x * 32 + threadIdx.x;
+  for (int yb = blockIdx.y * 8; yb < d.ny; yb += gridDim.y * 8) {
+    if (mode != 0 && !takes_part(d, mode, par, (yb / TE) * d.etx + (int)blockIdx.x)) continue;
+    const int y = yb + threadIdx.y;
+    if (x >= nx || y >= d.ny) continue;
+    const int s = y * nx + x;
     const bool wall = is_wall(d, x, y);
     const float fls = d.fl[s];
     // every load is issued before any value is chosen (gather_f / gather_g
@@ -378,35 +402,36 @@ __global__ void keep_state_kernel(Dev d, int layout, float* base, unsigned* ctr)
     float own[9], str[9], gown[5], gstr[5];
     bool act[9];
 #pragma unroll
-    for (int i = 0; i < 9; ++i) own[i] = ld_f(d, i, s);
+    for (int i = 0; i < 9; ++i) own[i] = F[i * n + s];
 #pragma unroll
-    for (int i = 0; i < 5; ++i) gown[i] = ld_g(d, i, s);
+    for (int i = 0; i < 5; ++i) gown[i] = G[i * n + s];
     const bool swapped = layout == 1 && !wall;
     if (swapped) {
 #pragma unroll
       for (int i = 1; i < 9; ++i) {
         const int sx = wrapx(d, x - ex9(i)), sy = wrapy(d, y - ey9(i));
-        const long long t = (long long)sy * d.nx + sx;
+        const int t = sy * nx + sx;
         act[i] = flow_active(d, sx, sy);
-        str[i] = ld_f(d, opp9(i), t);
-        if (i < 5) gstr[i] = ld_g(d, opp5(i), t);
+        str[i] = F[opp9(i) * n + t];
+        if (i < 5) gstr[i] = G[opp5(i) * n + t];
       }
     }
     const bool self = !wall && fls >= d.f_act;
+    const long long nn = n;
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
       const float v = (swapped && self && i > 0 && act[i]) ? str[i] : own[i];
-      dst[i * n + s] = v;
+      dst[i * nn + s] = v;
     }
 #pragma unroll
-    for (int i = 0; i < 5; ++i) dst[(9 + i) * n + s] = (swapped && i > 0) ? gstr[i] : gown[i];
-    dst[14 * n + s] = fls;
+    for (int i = 0; i < 5; ++i) dst[(9 + i) * nn + s] = (swapped && i > 0) ? gstr[i] : gown[i];
+    dst[14 * nn + s] = fls;
   }
-  if (ctr) {
+  if (ctr && mode != 1) {
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == 0 && threadIdx.y == 0) {
       __threadfence();
-      if (atomicAdd(ctr + 1, 1u) == gridDim.x - 1) {
+      if (atomicAdd(ctr + 1, 1u) == gridDim.x * gridDim.y - 1) {
         ctr[1] = 0;
         ctr[0] = ctr[0] + 1;
       }
@@ -471,8 +496,9 @@ void launch_reduce(const Dev& d, int layout, double* partials, double* out, int 
   else reduce_kernel<float><<<nblocks, RB, 0, s>>>(d, layout, partials);
   reduce_final_kernel<<<1, RB, 0, s>>>(partials, nblocks, out);
 }
-void launch_wall_nusselt(const Dev& d, int layout, double* acc, cudaStream_t s) {
-  wall_nusselt_kernel<<<1, RB, 0, s>>>(d, layout, acc);
+void launch_wall_nusselt(const Dev& d, int layout, int mode, int par, double* rows, double* acc,
+                         cudaStream_t s) {
+  wall_nusselt_kernel<<<1, RB, 0, s>>>(d, layout, mode, par, rows, acc);
 }
 void launch_get_state(const Dev& d, int layout, float* f, float* g, cudaStream_t s) {
   get_state_kernel<<<grid1(d.n, 256), 256, 0, s>>>(d, layout, f, g);
@@ -480,10 +506,11 @@ void launch_get_state(const Dev& d, int layout, float* f, float* g, cudaStream_t
 void launch_set_state(const Dev& d, const float* f, const float* g, cudaStream_t s) {
   set_state_kernel<<<grid1(d.n, 256), 256, 0, s>>>(d, f, g);
 }
-void launch_keep_state(const Dev& d, int layout, float* base, unsigned* ctr, cudaStream_t s) {
-  long long nb = (d.n + 255) / 256;
-  if (nb > 8 * 152) nb = 8 * 152;
-  keep_state_kernel<<<(unsigned)nb, 256, 0, s>>>(d, layout, base, ctr);
+void launch_keep_state(const Dev& d, int layout, float* base, unsigned* ctr, cudaStream_t s,
+                       int mode, int par) {
+  const int nby = (d.ny + 7) / 8, most = 2432 / d.etx;   // about two waves of blocks
+  const dim3 grid(d.etx, nby < most ? nby : most > 1 ? most : 1);
+  keep_state_kernel<<<grid, dim3(32, 8), 0, s>>>(d, layout, mode, par, base, ctr);
 }
 void launch_nonfinite(const Dev& d, int nblocks, cudaStream_t s) {
   nonfinite_kernel<<<nblocks, 256, 0, s>>>(d);

@@ -398,9 +398,9 @@ __device__ __forceinline__ void velocity(float jx, float jy, float T, float fl, 
 // commit and the near-tile pass are launched as programmatic dependents.  Their
 // CTAs start while the kernel before them runs (it allows that at once), read
 // what was final before that kernel, and wait for its end before anything
-// else (256 x 4 slab 14.9 -> 14.0 us a step, 256^2 18.5 -> 17.9).  CTA 0 always waits, so that a kernel's end still implies
-// the end of all before it.  On larger lattices waiting CTAs would hold SMs that
-// the far-tile pass needs.  Under the kernel trace every launch is an ordinary
+// else (256 x 4 slab 14.9 -> 14.0 us a step, 256^2 18.5 -> 17.9).  CTA 0 always
+// waits, so that a kernel's end still implies the end of all before it.  On larger
+// lattices waiting CTAs would hold SMs that the far-tile pass needs.  Under the kernel trace every launch is an ordinary
 // one, so that a record's start is the start of the CTA's work.
 inline bool early_launches(const Dev& d) { return d.ntiles <= d.egrid && !d.trace; }
 __device__ __forceinline__ void allow_dependents() {
@@ -459,7 +459,10 @@ void launch_get_state(const Dev& d, int parity, float* f, float* g, cudaStream_t
 void launch_set_state(const Dev& d, const float* f, const float* g, cudaStream_t s);
 // the whole state (f, g, f_l: 15 n floats, natural layout) into base, or into
 // base + ctr[0] 15 n and then ctr[0]++ when ctr is non-null (ctr[1] must be 0)
-void launch_keep_state(const Dev& d, int layout, float* base, unsigned* ctr, cudaStream_t s);
+// (FP32 storage).  mode 1: only the enthalpy tiles away from those the step of
+// parity par, just taken, listed (ctr does not advance); 2: only the others
+void launch_keep_state(const Dev& d, int layout, float* base, unsigned* ctr, cudaStream_t s,
+                       int mode = 0, int par = 0);
 // d.tact from d.fl, every tile (after f_l is loaded from outside the step)
 void launch_tile_activity(const Dev& d, cudaStream_t s);
 // NaN/Inf sentinel over the whole state (sets stats[5])

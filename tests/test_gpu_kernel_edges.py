@@ -1,7 +1,8 @@
 """Kernel forms at the sizes where they change: the count of listed enthalpy
 tiles (by the solve kernel up to 1152 tiles, by a list above), the stamps of a
-context whose fields are loaded again after an odd number of steps, and the
-reduction's FP32-pair sums.
+context whose fields are loaded again after an odd number of steps, the
+reduction's FP32-pair sums, and what the adjoints' forward runs read of tiles
+that the next step's pass may already take.
 """
 import numpy as np
 import pytest
@@ -103,3 +104,35 @@ def _check_sums(lat, w, p):
     assert abs(got["mass"] - mass) <= 1e-12 * abs(mass)
     assert abs(got["enthalpy"] - heat) <= 1e-12 * abs(heat)
     assert abs(got["melt_frac"] - fl[inside].mean()) <= 1e-12
+
+
+def _cavity_with_far_walls(flow):
+    """The front 140 nodes from the hot wall, so that the wall's tiles and most
+    of the liquid are away from it."""
+    w = W.adjoint_cavity(256, source_n=256, melted=0.55) if flow else W.adjoint_slab(512, 64)
+    if not flow:
+        x = np.arange(w.nx)[None, :]
+        w.T0[:, :] = np.where(x < 140, 1.0 - x / 140.0, -1.0)
+        w.fl0[:, :] = np.where(w.T0 > 0.3, 1.0, np.where(w.T0 < -0.3, 0.0, 0.5))
+    return w
+
+
+@pytest.mark.parametrize("flow", [0, 1])
+def test_nusselt_objective_reads_every_step(P, flow):
+    """J is the mean of the hot-wall Nusselt number after each step (the same
+    FP64 sum in another order: 1e-11), whichever schedule the forward run has."""
+    w = _cavity_with_far_walls(flow)
+    lat = P.Lattice(w.nx, w.ny, **w.params)
+    lat.set_fields(w.phi, w.K, w.T0, w.fl0, w.wall_T_left)
+    nus = []
+    for _ in range(20):
+        lat.step(1)
+        nus.append(lat.reduce()["nu_hot"])
+    runs = []
+    for every in (0, 5):
+        lat.set_fields(w.phi, w.K, w.T0, w.fl0, w.wall_T_left)
+        run = lat.adjoint_coupled if flow else lat.adjoint
+        runs.append(run(20, "nusselt", checkpoint_every=every))
+        assert abs(runs[-1][0] - np.mean(nus)) <= 1e-11 * abs(np.mean(nus))
+    for a, b in zip(runs[0][1:], runs[1][1:]):   # same states, same bits
+        assert np.array_equal(a, b)
