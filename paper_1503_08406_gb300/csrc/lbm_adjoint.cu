@@ -47,10 +47,9 @@ __device__ __forceinline__ int adj_nb(const Dev& d, int x, int y, int dx, int dy
 
 __device__ __forceinline__ float wt(const Dev& d, int i) { return i == 0 ? d.wt0 : d.wt1; }
 
-// Each reversed step is two kernels.  adj_band_kernel (one CTA) solves the
-// fixed point's adjoint on the unclamped nodes, a band along the front, and
-// adds nu = c mu there to lam_g' (nu is 0 elsewhere).  adj_full_kernel passes
-// over the whole lattice once: with lam_g+_i(x) = lam_g'_i(x + e_i) + nu(x + e_i) and
+// Each reversed step is two kernels.  adj_band_kernel solves the fixed point's
+// adjoint on the unclamped nodes, a band along the front, and leaves nu = c mu
+// there (0 elsewhere).  adj_full_kernel passes over the whole lattice once: with lam_g+_i(x) = lam_g'_i(x + e_i) + nu(x + e_i) and
 // S(y) = sum_i w~_i lam_g+_i(y) (the source adjoint of step F, the fixed
 // point's share included),
 //   lam_gpre = A^T lam_g+ per node
@@ -74,11 +73,11 @@ __device__ __forceinline__ bool band_node(const Dev& d, const float* f, int t) {
   return !is_wall(d, x, y) && adj_mushy(v);
 }
 
-// the band of the state with liquid fraction f, appended at list[*count]
-__global__ void adj_list_kernel(Dev d, const float* f, int* list, int* count) {
+// the band of the state with liquid fraction f
+__global__ void adj_list_kernel(Dev d, const float* f, int* list, int* count, int* pos) {
   const int s = blockIdx.x * AB + threadIdx.x;
   if (s >= (int)d.n) return;
-  if (band_node(d, f, s)) list[atomicAdd(count, 1)] = s;
+  if (band_node(d, f, s)) band_append(list, count, pos, (int)d.n, s, (s / d.nx + s % d.nx) & 1);
 }
 
 // The fixed point's adjoint on the band: right-hand side
@@ -87,10 +86,16 @@ __global__ void adj_list_kernel(Dev d, const float* f, int* list, int* count) {
 // neighbours have the other colour, so each colour updates in place, in any
 // order), over-relaxed by MU_OMEGA for the first MU_SOR sweeps, until no node
 // changes by more than MU_RTOL of its value or after max_sweeps.  The result
-// does not depend on the list's order.  Up to BAND_CAP band nodes sweep in
-// shared memory (each node's coefficients and its neighbours' places in the
-// list staged once); a wider band sweeps in global memory.  Empties the
-// previous band's list (old_count) for the full pass to refill.
+// does not depend on the list's order.
+//
+// Every CTA takes a share of the band's nodes and gathers their coefficients
+// into arrays in the band's order; the last CTA to finish does the sweeps, from
+// shared memory up to BAND_CAP nodes, and writes nu by node, which the full pass
+// adds to lam_g' as it reads it.  The gathers are scattered (some twenty sectors
+// a node) and bound the kernel when one SM makes them all, as does a
+// read-modify-write of nu into the five planes of lam_g' (2048 x 512, some 1500
+// nodes: 27 us with one CTA doing it all, 13 so; the full pass pays 3 us for nu).
+// Also clears the previous band's nu (old_list) and empties its list.
 constexpr float MU_RTOL = 4e-7f;
 // The Jacobi map's spectral radius is at most 2/3 here, so red-black SOR
 // converges fastest near omega = 2 / (1 + sqrt(1 - 4/9)) = 1.146
@@ -98,64 +103,78 @@ constexpr float MU_OMEGA = 1.15f;
 constexpr int MU_SOR = 6;
 constexpr int BAND_CAP = 4096;
 constexpr int BAND_THREADS = 1024;
-constexpr int BAND_SMEM = BAND_CAP * (int)(sizeof(float4) + sizeof(ushort4) + 4 * sizeof(float) + 1);
+constexpr int BAND_CTAS = 64;
+constexpr int BAND_SMEM = BAND_CAP * (int)(sizeof(float4) + sizeof(ushort4) + 3 * sizeof(float));
 
-// right-hand side of mu's equation at band node s
-__device__ __forceinline__ float band_rhs(const Dev& d, const AdjBuffers& b, int s) {
-  const int y = s / d.nx, x = s - y * d.nx;
-  const int n = (int)d.n;
-  float L = 0.f;
-#pragma unroll
-  for (int i = 0; i < 5; ++i) {
-    const int t = adj_nb(d, x, y, ex9(i), ey9(i));
-    L += wt(d, i) * ((t >= 0) ? b.lamg[i * n + t] : 0.f);
-  }
-  return b.lamf[s] - b.a[s] * L;
-}
-
-// nu = c mu at band node s joins every lam_g'_i there (lam_g+_i(x) takes
-// lam_g'_i + nu at x + e_i; nothing else reads lam_g' after this kernel)
-__device__ __forceinline__ void add_nu(const Dev& d, const AdjBuffers& b, int s, float v) {
-#pragma unroll
-  for (int i = 0; i < 5; ++i) b.lamg[i * (long long)d.n + s] += v;
-}
-
-__global__ void __launch_bounds__(BAND_THREADS) adj_band_kernel(Dev d, AdjBuffers b,
+__global__ void __launch_bounds__(BAND_THREADS, 1) adj_band_kernel(Dev d, AdjBuffers b,
                                                                 const float* f1, const int* list,
-                                                                const int* count, int* old_count,
-                                                                int max_sweeps) {
+                                                                const int* count,
+                                                                const int* old_list,
+                                                                int* old_count, int max_sweeps) {
   extern __shared__ float4 band_smem[];
-  const int cnt = *count;
-  if (cnt <= BAND_CAP) {
-    float4* ct = band_smem;                                    // c of the 4 neighbours
-    ushort4* ix = reinterpret_cast<ushort4*>(ct + BAND_CAP);   // their places in the list
-    float* rhs = reinterpret_cast<float*>(ix + BAND_CAP);      // divided by dd
-    float* kk = rhs + BAND_CAP;                                // a w~_1, divided by dd
-    float* dd = kk + BAND_CAP;                                 // 1 - a (1 - w~_0) c
-    float* mu = dd + BAND_CAP;
-    unsigned char* col = reinterpret_cast<unsigned char*>(mu + BAND_CAP);   // x + y parity
-    for (int j = threadIdx.x; j < cnt; j += blockDim.x) b.pos[list[j]] = j;
-    __syncthreads();
-    for (int j = threadIdx.x; j < cnt; j += blockDim.x) {
-      const int s = list[j];
-      const int y = s / d.nx, x = s - y * d.nx;
-      float c4[4];
-      unsigned short i4[4];
+  __shared__ int last;
+  const int n = (int)d.n;
+  // thread t of CTA k takes every BAND_CTAS-th node, so that a short band
+  // spreads over all CTAs
+  const int first = threadIdx.x * gridDim.x + blockIdx.x, step = gridDim.x * BAND_THREADS;
+  const int n0 = count[0], cnt = n0 + count[1];
+  const int o0 = old_count[0], ocnt = o0 + old_count[1];
+  for (int j = first; j < ocnt; j += step) b.nu[old_list[j < o0 ? j : n - 1 - (j - o0)]] = 0.f;
+  for (int j = first; j < cnt; j += step) {
+    const int s = list[j < n0 ? j : n - 1 - (j - n0)];
+    const int y = s / d.nx, x = s - y * d.nx;
+    float lg[5], f4[4], a4[4];
+    int p4[4];
+    lg[0] = b.lamg[s];
 #pragma unroll
-      for (int i = 1; i < 5; ++i) {
-        const int t = adj_nb(d, x, y, ex9(i), ey9(i));
-        const bool on = band_node(d, f1, t);
-        c4[i - 1] = on ? 1.f / (d.dTt + b.a[t]) : 0.f;
-        i4[i - 1] = (unsigned short)(on ? b.pos[t] : j);
-      }
-      ct[j] = make_float4(c4[0], c4[1], c4[2], c4[3]);
-      ix[j] = make_ushort4(i4[0], i4[1], i4[2], i4[3]);
-      const float as = b.a[s];
-      const float den = 1.f - as * (1.f - d.wt0) / (d.dTt + as);
-      rhs[j] = band_rhs(d, b, s) / den;
-      kk[j] = as * d.wt1 / den;
+    for (int i = 1; i < 5; ++i) {
+      const int t = adj_nb(d, x, y, ex9(i), ey9(i));
+      lg[i] = t >= 0 ? b.lamg[i * n + t] : 0.f;
+      // (a wall node's f_l counts as clamped)
+      int tx = x + ex9(i), ty = y + ey9(i);
+      tx = tx < 0 ? tx + d.nx : tx >= d.nx ? tx - d.nx : tx;
+      ty = ty < 0 ? ty + d.ny : ty >= d.ny ? ty - d.ny : ty;
+      const bool in = t >= 0 && !is_wall(d, tx, ty);
+      f4[i - 1] = in ? f1[t] : 0.f;
+      a4[i - 1] = in ? b.a[t] : 0.f;
+      p4[i - 1] = in ? b.pos[t] : 0;   // (of some earlier band where t is not on this one)
+    }
+    const float as = b.a[s], lf = b.lamf[s];
+    float c4[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const bool on = adj_mushy(f4[i]);
+      c4[i] = on ? 1.f / (d.dTt + a4[i]) : 0.f;
+      p4[i] = !on ? j : p4[i] < n0 ? p4[i] : n0 + (n - 1 - p4[i]);
+    }
+    float L = 0.f;
+#pragma unroll
+    for (int i = 0; i < 5; ++i) L += wt(d, i) * lg[i];
+    const float den = 1.f - as * (1.f - d.wt0) / (d.dTt + as);
+    b.bc[j] = make_float4(c4[0], c4[1], c4[2], c4[3]);
+    b.bi[j] = make_int4(p4[0], p4[1], p4[2], p4[3]);
+    b.bk[j] = make_float4((lf - as * L) / den, as * d.wt1 / den, d.dTt + as, 0.f);
+  }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(b.done, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  if (cnt <= BAND_CAP) {
+    float4* ct = band_smem;
+    ushort4* ix = reinterpret_cast<ushort4*>(ct + BAND_CAP);
+    float* rhs = reinterpret_cast<float*>(ix + BAND_CAP);
+    float* kk = rhs + BAND_CAP;
+    float* mu = kk + BAND_CAP;
+    for (int j = threadIdx.x; j < cnt; j += BAND_THREADS) {
+      const int4 q = __ldcg(b.bi + j);
+      const float4 k = __ldcg(b.bk + j);
+      ct[j] = __ldcg(b.bc + j);
+      ix[j] = make_ushort4(q.x, q.y, q.z, q.w);
+      rhs[j] = k.x;
+      kk[j] = k.y;
       mu[j] = 0.f;
-      col[j] = (unsigned char)((x + y) & 1);
     }
     __syncthreads();
     bool more = true;
@@ -163,8 +182,7 @@ __global__ void __launch_bounds__(BAND_THREADS) adj_band_kernel(Dev d, AdjBuffer
       const float om = k < MU_SOR ? MU_OMEGA : 1.f;
       int moved = 0;
       for (int c0 = 0; c0 < 2; ++c0) {
-        for (int j = threadIdx.x; j < cnt; j += blockDim.x) {
-          if (col[j] != c0) continue;
+        for (int j = (c0 ? n0 : 0) + threadIdx.x; j < (c0 ? cnt : n0); j += BAND_THREADS) {
           const float4 c = ct[j];
           const ushort4 q = ix[j];
           const float nb = c.x * mu[q.x] + c.y * mu[q.y] + c.z * mu[q.z] + c.w * mu[q.w];
@@ -178,52 +196,38 @@ __global__ void __launch_bounds__(BAND_THREADS) adj_band_kernel(Dev d, AdjBuffer
       }
       more = __syncthreads_or(moved);
     }
-    for (int j = threadIdx.x; j < cnt; j += blockDim.x) {
-      const int s = list[j];
-      add_nu(d, b, s, mu[j] / (d.dTt + b.a[s]));
-    }
+    for (int j = threadIdx.x; j < cnt; j += BAND_THREADS)
+      b.nu[list[j < n0 ? j : n - 1 - (j - n0)]] = mu[j] / __ldcg(b.bk + j).z;
   } else {
-    float* mu = b.mu0;
-    for (int j = threadIdx.x; j < cnt; j += blockDim.x) {
-      const int s = list[j];
-      const float as = b.a[s];
-      b.rhs[s] = band_rhs(d, b, s) / (1.f - as * (1.f - d.wt0) / (d.dTt + as));
-      mu[s] = 0.f;
-    }
+    float* mu = b.mu;
+    for (int j = threadIdx.x; j < cnt; j += BAND_THREADS) mu[j] = 0.f;
     __syncthreads();
     bool more = true;
     for (int k = 0; k < max_sweeps && more; ++k) {
       const float om = k < MU_SOR ? MU_OMEGA : 1.f;
       int moved = 0;
       for (int c0 = 0; c0 < 2; ++c0) {
-        for (int j = threadIdx.x; j < cnt; j += blockDim.x) {
-          const int s = list[j];
-          const int y = s / d.nx, x = s - y * d.nx;
-          if (((x + y) & 1) != c0) continue;
-          float nb = 0.f;
-#pragma unroll
-          for (int i = 1; i < 5; ++i) {
-            const int t = adj_nb(d, x, y, ex9(i), ey9(i));
-            nb += band_node(d, f1, t) ? mu[t] / (d.dTt + b.a[t]) : 0.f;
-          }
-          const float as = b.a[s];
-          const float raw = b.rhs[s] - as * d.wt1 / (1.f - as * (1.f - d.wt0) / (d.dTt + as)) * nb;
-          const float o = mu[s];
+        for (int j = (c0 ? n0 : 0) + threadIdx.x; j < (c0 ? cnt : n0); j += BAND_THREADS) {
+          const float4 c = __ldcg(b.bc + j), kj = __ldcg(b.bk + j);
+          const int4 q = __ldcg(b.bi + j);
+          const float nb = c.x * mu[q.x] + c.y * mu[q.y] + c.z * mu[q.z] + c.w * mu[q.w];
+          const float raw = kj.x - kj.y * nb;
+          const float o = mu[j];
           const float v = o + om * (raw - o);
           moved |= fabsf(v - o) > MU_RTOL * fabsf(v);
-          mu[s] = v;
+          mu[j] = v;
         }
         if (c0 == 0) __syncthreads();
       }
       more = __syncthreads_or(moved);
     }
-    for (int j = threadIdx.x; j < cnt; j += blockDim.x) {
-      const int s = list[j];
-      add_nu(d, b, s, mu[s] / (d.dTt + b.a[s]));
-    }
+    for (int j = threadIdx.x; j < cnt; j += BAND_THREADS)
+      b.nu[list[j < n0 ? j : n - 1 - (j - n0)]] = mu[j] / __ldcg(b.bk + j).z;
   }
-  __syncthreads();
-  if (threadIdx.x == 0) *old_count = 0;
+  if (threadIdx.x == 0) {
+    old_count[0] = old_count[1] = 0;
+    *b.done = 0;
+  }
 }
 
 // lam_g+ of node (x, y) (rows yu = y + 1, yd = y - 1, periodic) and A^T of it
@@ -235,7 +239,7 @@ __device__ __forceinline__ void pre_pops(const Dev& d, const AdjBuffers& b, cons
                     yd * d.nx + x};
 #pragma unroll
   for (int i = 0; i < 5; ++i)
-    lp[i] = (t[i] >= 0) ? __ldg(b.lamg + i * n + t[i]) : 0.f;
+    lp[i] = (t[i] >= 0) ? __ldg(b.lamg + i * n + t[i]) + __ldg(b.nu + t[i]) : 0.f;
 #pragma unroll
   for (int k = 0; k < 5; ++k) {
     float v = 0.f;
@@ -290,7 +294,7 @@ __global__ void __launch_bounds__(AB) adj_full_kernel(Dev d, AdjBuffers b, Mat5 
     const float fa = f0[s], fb = f1[s];
     b.lamf[s] = __ldg(b.a + s) * S;
     if (fb != fa) b.lama[s] += -(fb - fa) * S;   // (adds 0 elsewhere)
-    if (adj_mushy(fa)) next_list[atomicAdd(next_count, 1)] = s;
+    if (adj_mushy(fa)) band_append(next_list, next_count, b.pos, n, s, (x + y) & 1);
   }
 }
 
@@ -396,9 +400,9 @@ __global__ void __launch_bounds__(128, 8) adj_coupled_kernel(CoupledStep<float> 
 }
 
 void adj_coupled_step(const Dev& d, const AdjBuffers& b, const CoupledStep<float>& A, int* list,
-                      int* count, int* old_count, int mu_sweeps, cudaStream_t s) {
-  adj_band_kernel<<<1, BAND_THREADS, BAND_SMEM, s>>>(d, b, A.fl1, list, count, old_count,
-                                                     mu_sweeps);
+                      int* count, int mu_sweeps, cudaStream_t s) {
+  adj_band_kernel<<<BAND_CTAS, BAND_THREADS, BAND_SMEM, s>>>(d, b, A.fl1, list, count, A.next_list,
+                                                             A.next_count, mu_sweeps);
   const dim3 grid((d.nx + 127) / 128, d.ny < 65535 ? d.ny : 65535);
   adj_coupled_kernel<<<grid, 128, 0, s>>>(A);
 }
@@ -408,8 +412,8 @@ bool adj_init() {
                               BAND_SMEM) == cudaSuccess;
 }
 
-void adj_list(const Dev& d, const float* f, int* list, int* count, cudaStream_t s) {
-  adj_list_kernel<<<blocks(d.n), AB, 0, s>>>(d, f, list, count);
+void adj_list(const Dev& d, const float* f, int* list, int* count, int* pos, cudaStream_t s) {
+  adj_list_kernel<<<blocks(d.n), AB, 0, s>>>(d, f, list, count, pos);
 }
 
 void adj_save(const Dev& d, float* base, unsigned* ctr, cudaStream_t s) {
@@ -421,8 +425,8 @@ void adj_save(const Dev& d, float* base, unsigned* ctr, cudaStream_t s) {
 void adj_step(const Dev& d, const AdjBuffers& b, const float* f0, const float* f1, int* list,
               int* count, int* old_list, int* old_count, int mu_sweeps, NuSrc nu,
               cudaStream_t s) {
-  adj_band_kernel<<<1, BAND_THREADS, BAND_SMEM, s>>>(d, b, f1, list, count, old_count,
-                                                     mu_sweeps);
+  adj_band_kernel<<<BAND_CTAS, BAND_THREADS, BAND_SMEM, s>>>(d, b, f1, list, count, old_list,
+                                                             old_count, mu_sweeps);
   Mat5 At;
   for (int k = 0; k < 25; ++k) At.m[k] = b.At[k];
   const dim3 grid((d.nx + AB - 1) / AB, d.ny < 65535 ? d.ny : 65535);

@@ -10,13 +10,17 @@ struct AdjBuffers {
   float* a;          // a = phi dT / (sigma St)
   float* lamg;       // 5 n: adjoint of the populations after the step being reversed
   float* lamf;       // adjoint of f_l after the step (in), before it (out)
-  float* rhs;        // band nodes (wide bands): right-hand side of mu's equation
-  float* mu0;        // mu in global memory (wide bands), ping-pong
-  float* mu1;
+  // band nodes, by place in the band's order (colour 0, then colour 1):
+  float4* bc;        // c of the four neighbours, 0 off the band
+  int4* bi;          // their places
+  float4* bk;        // right-hand side, a w~_1 (both divided by the self term), T_l - T_s + a
+  float* mu;         // mu (bands too wide for shared memory)
+  float* nu;         // nu = c mu of the step being reversed by node, 0 off the band
+  unsigned* done;    // CTAs of the band kernel that are done (0 between launches)
   float* lamgpre;    // 5 n: adjoint of the populations before the step
   float* lama;       // accumulated adjoint of a
   float* lamtw;      // ny: accumulated adjoint of the left wall profile
-  int* pos;          // n: a band node's place in the band list
+  int* pos;          // n: a band node's place in the band list (band_append)
   float At[25];      // transposed collision matrix (u = 0), passed to kernels by value
 };
 struct Mat5 {
@@ -47,15 +51,15 @@ void adj_mul(long long n, float* v, const float* w, cudaStream_t s);
 void adj_a(const Dev& d, float* a, cudaStream_t s);
 // J into out[0]; out holds 129 doubles (the rest: partial sums)
 void adj_objective(const Dev& d, const float* fl, double* out, cudaStream_t s);
-// the band (non-wall nodes with 0 < f < 1), appended at list[*count]
-void adj_list(const Dev& d, const float* f, int* list, int* count, cudaStream_t s);
+// the band (non-wall nodes with 0 < f < 1) on a list of n entries (band_append)
+void adj_list(const Dev& d, const float* f, int* list, int* count, int* pos, cudaStream_t s);
 // d.fl to base + k n, k = ctr[0], which then advances (ctr[1]: scratch, 0)
 void adj_save(const Dev& d, float* base, unsigned* ctr, cudaStream_t s);
 // One step of the reverse sweep, given f_l before (f0) and after (f1) it and
 // the band after it (list, count): from b.lamg / b.lamf (after the step) to
 // b.lamgpre / b.lamf (before it), the Nusselt terms (nu) of the state before
-// it included.  old_list / old_count hold the band the
-// previous call solved on; they are emptied and refilled with the band before
+// it included.  old_list / old_count hold the band the previous call solved on
+// (b.nu is still set there); they are emptied and refilled with the band before
 // this step, for the next call.  The caller swaps b.lamg and b.lamgpre and the
 // two lists.
 void adj_step(const Dev& d, const AdjBuffers& b, const float* f0, const float* f1, int* list,
@@ -64,9 +68,10 @@ void adj_step(const Dev& d, const AdjBuffers& b, const float* f0, const float* f
 // One reversed step of the coupled adjoint (flow on): the band kernel on
 // b.lamg / b.lamf (A.lg1 is b.lamg, A.lfl is b.lamf, A.fl1 the band's f_l),
 // then lbm::coupled_reverse_node over every node; the band before the step is
-// listed at A.next_list (its count at old_count, emptied first).
+// listed at A.next_list (its counts at A.next_count), which hold the previous
+// call's band until then.
 void adj_coupled_step(const Dev& d, const AdjBuffers& b, const CoupledStep<float>& A, int* list,
-                      int* count, int* old_count, int mu_sweeps, cudaStream_t s);
+                      int* count, int mu_sweeps, cudaStream_t s);
 // once per process before adj_step: the band kernel's shared-memory opt-in
 bool adj_init();
 

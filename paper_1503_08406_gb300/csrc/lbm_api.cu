@@ -1296,6 +1296,17 @@ struct DevMem {
 
 }  // namespace
 
+// the band solver's buffers (n nodes)
+static bool band_buffers(DevMem& mem, lbm::AdjBuffers& b, size_t n) {
+  b.bc = reinterpret_cast<float4*>(mem.get(4 * n));
+  b.bi = reinterpret_cast<int4*>(mem.get(4 * n));
+  b.bk = reinterpret_cast<float4*>(mem.get(4 * n));
+  b.mu = mem.get(n);
+  b.nu = mem.get(n);
+  b.done = reinterpret_cast<unsigned*>(mem.get(1));
+  return b.bc && b.bi && b.bk && b.mu && b.nu && b.done;
+}
+
 // A graph of `steps` steps from parity 0 like capture(), each step followed
 // by the hooks.
 static cudaGraphExec_t capture_keep(lbm_ctx* c, int steps, const Hooks& h) {
@@ -1397,21 +1408,19 @@ int lbm_adjoint(lbm_ctx* c, int objective, int64_t nsteps, int32_t checkpoint_ev
   b.a = mem.get(n);
   b.lamg = mem.get(5 * n);
   b.lamf = mem.get(n);
-  b.rhs = mem.get(n);
-  b.mu0 = mem.get(n);
-  b.mu1 = mem.get(n);
+  const bool band = band_buffers(mem, b, n);
   b.lamgpre = mem.get(5 * n);
   b.lama = mem.get(n);
   b.lamtw = mem.get((size_t)c->d.ny);
   b.pos = reinterpret_cast<int*>(mem.get(n));
   int* lists[2] = {reinterpret_cast<int*>(mem.get(n)), reinterpret_cast<int*>(mem.get(n))};
-  int* counts = reinterpret_cast<int*>(mem.get(2));
+  int* counts = reinterpret_cast<int*>(mem.get(4));   // two a list
   unsigned* ctr = reinterpret_cast<unsigned*>(mem.get(2));
   double* nu_acc = reinterpret_cast<double*>(mem.get(2));
   double* nu_rows = reinterpret_cast<double*>(mem.get(2 * (size_t)c->d.ny));
   double* dJ = reinterpret_cast<double*>(mem.get(2 * 129));
-  if (!flS || (!keep_all && (!cps || !fin)) || !b.a || !b.lamg || !b.lamf || !b.rhs ||
-      !b.mu0 || !b.mu1 || !b.lamgpre || !b.lama || !b.lamtw || !b.pos || !lists[0] ||
+  if (!flS || (!keep_all && (!cps || !fin)) || !b.a || !b.lamg || !b.lamf || !band ||
+      !b.lamgpre || !b.lama || !b.lamtw || !b.pos || !lists[0] ||
       !lists[1] || !counts || !ctr || !nu_acc || !nu_rows || !dJ)
     return LBM_ERR_OOM;
   // transposed collision matrix with u = 0: g+ = A g,
@@ -1485,15 +1494,17 @@ int lbm_adjoint(lbm_ctx* c, int objective, int64_t nsteps, int32_t checkpoint_ev
   // reverse sweep
   LBM_CUDA(cudaMemsetAsync(b.lama, 0, n * sizeof(float), c->stream));
   LBM_CUDA(cudaMemsetAsync(b.lamtw, 0, c->d.ny * sizeof(float), c->stream));
-  LBM_CUDA(cudaMemsetAsync(counts, 0, 2 * sizeof(int), c->stream));
-  lbm::adj_list(c->d, fl_end, lists[0], counts, c->stream);
+  LBM_CUDA(cudaMemsetAsync(counts, 0, 4 * sizeof(int), c->stream));
+  LBM_CUDA(cudaMemsetAsync(b.nu, 0, n * sizeof(float), c->stream));
+  LBM_CUDA(cudaMemsetAsync(b.done, 0, sizeof(unsigned), c->stream));
+  lbm::adj_list(c->d, fl_end, lists[0], counts, b.pos, c->stream);
   int cur = 0;
   // reversed steps m = hi - 1 .. lo, f_l of step m at F + (m - lo) n
   auto reverse = [&](cudaStream_t sm, const float* F, int64_t lo, int64_t hi) {
     for (int64_t m = hi - 1; m >= lo; --m) {
       const float* f0 = F + (size_t)(m - lo) * n;
-      lbm::adj_step(c->d, b, f0, f0 + n, lists[cur], counts + cur, lists[1 - cur],
-                    counts + 1 - cur, sweeps, nu, sm);
+      lbm::adj_step(c->d, b, f0, f0 + n, lists[cur], counts + 2 * cur, lists[1 - cur],
+                    counts + 2 * (1 - cur), sweeps, nu, sm);
       std::swap(b.lamg, b.lamgpre);
       cur ^= 1;
     }
@@ -1627,20 +1638,18 @@ int lbm_adjoint_coupled(lbm_ctx* c, int objective, int64_t nsteps, int32_t check
   lbm::AdjBuffers b;
   b.a = mem.get(n);
   b.lamf = mem.get(n);
-  b.rhs = mem.get(n);
-  b.mu0 = mem.get(n);
-  b.mu1 = mem.get(n);
+  const bool band = band_buffers(mem, b, n);
   b.lama = mem.get(n);   // adjoint of phi
   b.lamtw = mem.get((size_t)d.ny);
   b.pos = reinterpret_cast<int*>(mem.get(n));
   float* lK = mem.get(n);
   int* lists[2] = {reinterpret_cast<int*>(mem.get(n)), reinterpret_cast<int*>(mem.get(n))};
-  int* counts = reinterpret_cast<int*>(mem.get(2));
+  int* counts = reinterpret_cast<int*>(mem.get(4));   // two a list
   double* nu_acc = reinterpret_cast<double*>(mem.get(2));
   double* nu_rows = reinterpret_cast<double*>(mem.get(2 * (size_t)d.ny));
   unsigned* ctr = reinterpret_cast<unsigned*>(mem.get(4));   // two counter pairs
   if (!S || (!keep_all && (!cps || !fin || !S2)) || !lf[0] || !lf[1] || !lg[0] || !lg[1] || !b.a ||
-      !b.lamf || !b.rhs || !b.mu0 || !b.mu1 || !b.lama || !b.lamtw || !b.pos || !lK ||
+      !b.lamf || !band || !b.lama || !b.lamtw || !b.pos || !lK ||
       !lists[0] || !lists[1] || !counts || !nu_acc || !nu_rows || !ctr)
     return LBM_ERR_OOM;
   // rows of the Nusselt number (lbm_reduce's): all but horizontal wall rows
@@ -1719,9 +1728,11 @@ int lbm_adjoint_coupled(lbm_ctx* c, int objective, int64_t nsteps, int32_t check
   LBM_CUDA(cudaMemsetAsync(b.lama, 0, n * sizeof(float), c->stream));
   LBM_CUDA(cudaMemsetAsync(lK, 0, n * sizeof(float), c->stream));
   LBM_CUDA(cudaMemsetAsync(b.lamtw, 0, d.ny * sizeof(float), c->stream));
-  LBM_CUDA(cudaMemsetAsync(counts, 0, 2 * sizeof(int), c->stream));
+  LBM_CUDA(cudaMemsetAsync(counts, 0, 4 * sizeof(int), c->stream));
+  LBM_CUDA(cudaMemsetAsync(b.nu, 0, n * sizeof(float), c->stream));
+  LBM_CUDA(cudaMemsetAsync(b.done, 0, sizeof(unsigned), c->stream));
   lbm::adj_a(c->d, b.a, c->stream);
-  lbm::adj_list(c->d, last + 14 * n, lists[0], counts, c->stream);
+  lbm::adj_list(c->d, last + 14 * n, lists[0], counts, b.pos, c->stream);
   // the step's parameters
   lbm::CoupledStep<float> A;
   A.geo = lbm::CoupledGeo{d.nx, d.ny, d.per_x, d.per_y, {d.bc[0], d.bc[1], d.bc[2], d.bc[3]}};
@@ -1762,6 +1773,8 @@ int lbm_adjoint_coupled(lbm_ctx* c, int objective, int64_t nsteps, int32_t check
   A.lphi = b.lama;
   A.lK = lK;
   A.lTw = b.lamtw;
+  A.nu = b.nu;
+  A.next_pos = b.pos;
   // reverse sweep: step m of a stretch whose states sit at F (index m - lo)
   int cur = 0;
   auto reverse = [&](cudaStream_t sm, const float* F, int64_t lo, int64_t hi) {
@@ -1777,9 +1790,9 @@ int lbm_adjoint_coupled(lbm_ctx* c, int objective, int64_t nsteps, int32_t check
       A.lf0 = lf[1 - cur];
       A.lg0 = lg[1 - cur];
       A.next_list = lists[1 - cur];
-      A.next_count = counts + 1 - cur;
+      A.next_count = counts + 2 * (1 - cur);
       b.lamg = lg[cur];
-      lbm::adj_coupled_step(c->d, b, A, lists[cur], counts + cur, counts + 1 - cur, sweeps, sm);
+      lbm::adj_coupled_step(c->d, b, A, lists[cur], counts + 2 * cur, sweeps, sm);
       cur ^= 1;
     }
   };

@@ -431,7 +431,20 @@ struct CoupledStep {
   R* lfl;                                    // adjoint of f_l: after the step in, before it out
   R *lphi, *lK, *lTw;                        // accumulated
   int *next_list, *next_count;               // band of the state before the step
+  // optional: nu = c mu where lg1 does not hold it yet (0 off the band), and the
+  // band listed by colour (band_append): each node's place, and n list entries
+  const R* nu = nullptr;
+  int* next_pos = nullptr;
 };
+
+// Put node s of colour c = (x + y) & 1 on a band list of n entries: colour 0 from
+// the front (count[0] of them), colour 1 from the back (count[1]).
+LBM_HD void band_append(int* list, int* count, int* pos, int n, int s, int c) {
+  const int i = hd_fetch_add(count + c, 1);
+  const int at = c ? n - 1 - i : i;
+  list[at] = s;
+  pos[s] = at;
+}
 
 // the flux moments' rate at liquid fraction fl, and its derivative
 template <typename R>
@@ -465,6 +478,7 @@ LBM_HD void coupled_lp(const CoupledStep<R>& A, int x, int y, R lp[5]) {
   for (int i = 0; i < 5; ++i) {
     const int t = A.geo.nb(x, y, ex[i], ey[i]);
     lp[i] = t >= 0 ? A.lg1[i * A.n + t] : R(0);
+    if (A.nu && t >= 0) lp[i] += A.nu[t];
   }
 }
 
@@ -591,7 +605,10 @@ LBM_HD void coupled_reverse_node(const CoupledStep<R>& A, int x, int y) {
   for (int i = 0; i < 5; ++i) A.lg0[i * n + s] = lg[i];
   A.lfl[s] = lfl;
   const R fa = A.fl0[s];
-  if (!wall && adj_mushy(fa)) A.next_list[hd_fetch_add(A.next_count, 1)] = s;
+  if (!wall && adj_mushy(fa)) {
+    if (A.next_pos) band_append(A.next_list, A.next_count, A.next_pos, (int)n, s, (x + y) & 1);
+    else A.next_list[hd_fetch_add(A.next_count, 1)] = s;
+  }
 }
 
 }  // namespace lbm
