@@ -432,15 +432,9 @@ int lbm_set_fields(lbm_ctx* c, const float* phi, const float* K, const float* T0
   LBM_CUDA(cudaMemcpyAsync((float*)d.K, src[1], n * sizeof(float), cudaMemcpyDeviceToDevice,
                            c->stream));
   LBM_CUDA(cudaMemcpyAsync(d.fl, src[3], n * sizeof(float), cudaMemcpyDeviceToDevice, c->stream));
-  if (wall_T_left) {
+  if (wall_T_left)
     LBM_TRY(copy_in(c, (float*)d.wallTl, wall_T_left, (size_t)c->p.ny, device_ptrs));
-  } else {
-    std::vector<float> w((size_t)c->p.ny, (float)c->p.T_bc[LBM_SIDE_LEFT]);
-    LBM_CUDA(cudaMemcpyAsync((float*)d.wallTl, w.data(), w.size() * sizeof(float),
-                             cudaMemcpyHostToDevice, c->stream));
-    LBM_CUDA(cudaStreamSynchronize(c->stream));
-  }
-  lbm::launch_init(d, src[2], c->stream);
+  lbm::launch_init(d, src[2], wall_T_left ? nullptr : (float*)d.wallTl, c->stream);
   LBM_CUDA(cudaGetLastError());
   LBM_TRY(reset_lists(c));
   c->steps = 0;

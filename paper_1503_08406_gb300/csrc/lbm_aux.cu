@@ -86,9 +86,12 @@ __device__ float node_T(const Dev& d, int x, int y, int layout) {
 
 // ---- kernels ----------------------------------------------------------------
 
-__global__ void init_kernel(Dev d, const float* T0) {
+// rest equilibria at T0; the left wall's profile from the side's value when
+// wallTl (the profile, if it is to be set) is not null
+__global__ void init_kernel(Dev d, const float* T0, float* wallTl) {
   const long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (s >= d.n) return;
+  if (wallTl && s < d.ny) wallTl[s] = d.Tbc[0];
   // f^eq(rho0, u = 0) = w_i rho0, Eq. (29); stored as the deviation f - w_i rho0 = 0
   for (int i = 0; i < 9; ++i) st_f(d, i, s, 0.f);
   // g^eq(T0, u = 0), Eq. (39): w~_i T0
@@ -455,8 +458,8 @@ __global__ void nonfinite_kernel(Dev d) {
 
 static unsigned grid1(long long n, int b) { return (unsigned)((n + b - 1) / b); }
 
-void launch_init(const Dev& d, const float* T0, cudaStream_t s) {
-  init_kernel<<<grid1(d.n, 256), 256, 0, s>>>(d, T0);
+void launch_init(const Dev& d, const float* T0, float* wallTl, cudaStream_t s) {
+  init_kernel<<<grid1(d.n, 256), 256, 0, s>>>(d, T0, wallTl);
 }
 // one CTA per enthalpy tile: does a non-wall node of it carry flow?
 __global__ void __launch_bounds__(256) tile_activity_kernel(Dev d) {

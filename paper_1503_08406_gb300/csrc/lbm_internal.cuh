@@ -449,7 +449,7 @@ void launch_enthalpy_solve_batch(const BatchPlan& P, int parity, cudaStream_t s)
 void launch_enthalpy_commit_batch(const BatchPlan& P, int parity, cudaStream_t s);
 void enthalpy_setup();
 size_t enthalpy_solve_smem();
-void launch_init(const Dev& d, const float* T0, cudaStream_t s);
+void launch_init(const Dev& d, const float* T0, float* wallTl, cudaStream_t s);
 void launch_macros(const Dev& d, int parity, float* ux, float* uy, float* rho, float* T,
                    float* fl, cudaStream_t s);
 void launch_reduce(const Dev& d, int parity, double* partials, double* out, int nblocks,
