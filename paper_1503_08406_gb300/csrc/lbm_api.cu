@@ -153,7 +153,7 @@ Layout layout_of(const lbm_params* p, int nred) {
   L.nearmap = o; o += 2 * tiles * sizeof(int);
   L.proc = o; o += up(o + tiles * sizeof(int)) - o;
   L.list = o; o += up(2 * tiles * sizeof(int));
-  L.lcount = o; o += up(2 * sizeof(int));
+  L.lcount = o; o += up(4 * sizeof(int));
   L.ctr = o; o += up(2 * sizeof(int));
   L.tact = o; o += up(tiles);
   L.scr = o; o += up(n * sizeof(float2));
@@ -389,7 +389,7 @@ int64_t lbm_steps_done(const lbm_ctx* c) { return c ? c->steps : -1; }
 static int reset_lists(lbm_ctx* c) {
   const Dev& d = c->d;
   LBM_CUDA(cudaMemsetAsync(d.flags, 0, 5 * sizeof(int) * d.ntiles, c->stream));   // to proc's end
-  LBM_CUDA(cudaMemsetAsync(d.lcount, 0, 2 * sizeof(int), c->stream));
+  LBM_CUDA(cudaMemsetAsync(d.lcount, 0, 4 * sizeof(int), c->stream));
   LBM_CUDA(cudaMemsetAsync(d.stats + 5, 0, sizeof(int), c->stream));
   lbm::launch_tile_activity(d, c->stream);   // f_l was just loaded
   c->since_check = 0;
@@ -1811,7 +1811,7 @@ int lbm_adjoint_coupled(lbm_ctx* c, int objective, int64_t nsteps, int32_t check
       cudaMemcpyAsync(c->d.fl, SS + 14 * n, n * sizeof(float), cudaMemcpyDeviceToDevice, sm);
       lbm::launch_tile_activity(c->d, sm);
       cudaMemsetAsync(c->d.flags, 0, 5 * sizeof(int) * c->d.ntiles, sm);   // to proc's end
-      cudaMemsetAsync(c->d.lcount, 0, 2 * sizeof(int), sm);
+      cudaMemsetAsync(c->d.lcount, 0, 4 * sizeof(int), sm);
       if (sm == c->cap) {
         // in a capture: the step sequence of lbm_step's graphs (the next step's
         // far tiles beside each step's enthalpy kernels), the state after each

@@ -463,10 +463,11 @@ __device__ __forceinline__ void enthalpy_solve_body(const Dev& d, int bid, int n
       if (li != bid) tile = d.list[PAR * d.ntiles + li];
       solve_tile<PAR, S>(d, sm, tile, ctr, nullptr);
     }
+    if (tid == 0 && bid == 0) d.lcount[2 + PAR] = cnt;
   } else {
     const int rank = count_tiles<PAR>(d, sm, ctr, bid, nblk);
     for (int i = 0; i < sm.mine; ++i) solve_tile<PAR, S>(d, sm, sm.tile[i], ctr, nullptr);
-    if (tid == 0 && bid == 0) d.lcount[PAR] = rank;
+    if (tid == 0 && bid == 0) d.lcount[PAR] = d.lcount[2 + PAR] = rank;
   }
   if (tid == 0 && d.trace) trace_end(d, 100 * PAR + 20, ctr, tr0);
 }

@@ -502,25 +502,12 @@ __device__ __forceinline__ bool takes_tile(const Dev& d, int et, int prev) {
 
 // ---- ordinary-load kernel ----------------------------------------------------
 
-template <typename S, int PAR, int FLOW, int MODE>
-__global__ void __launch_bounds__(TX* TY, 4) fused_step_kernel(Dev d) {
+// the 32x8 nodes from (x0, y0) on
+template <typename S, int PAR, int FLOW>
+__device__ __forceinline__ void step_tile(const Dev& d, int x0, int y0, int prev, int stamp) {
   constexpr unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x;
-  const int prev = d.ctr[1 - PAR], stamp = prev + 1;   // (no launch of this step changes it)
-  const bool first = blockIdx.x == 0 && blockIdx.y == 0;
-  if (MODE != 1 && first) {
-    if (MODE == 2) wait_for_previous();
-    if (lane == 0 && threadIdx.y == 0) step_prologue<PAR>(d);
-  }
-  if (MODE != 0) {   // (one tile per CTA: a warp's first nine lanes look at its surroundings)
-    const int et = ((blockIdx.y * TY) / TE) * d.etx + (blockIdx.x * TX) / TE;
-    const bool hit = d.ntiles > COUNT_TILES
-                         ? lane == 0 && d.nearmap[(1 - PAR) * d.ntiles + et] == prev
-                         : lane < 9 && listed_at(d, et, lane, 1 - PAR, prev);
-    if ((MODE == 2) != __any_sync(FULL, hit)) return;
-    if (MODE == 2) wait_for_previous();
-  }
-  const int x = blockIdx.x * TX + lane, y = blockIdx.y * TY + threadIdx.y;
+  const int x = x0 + lane, y = y0 + threadIdx.y;
   const int nx = d.nx, ny = d.ny;
   if (y >= ny) return;  // whole warp: one warp is one row segment
   const bool node = x < nx && !is_wall(d, x, y);
@@ -576,7 +563,40 @@ __global__ void __launch_bounds__(TX* TY, 4) fused_step_kernel(Dev d) {
     unsafe = node_update<S, PAR, FLOW>(d, x, y, q, fln, g, f, fb, phi, K, wact, seed, &stamp);
   }
   if (__any_sync(FULL, unsafe) && lane == 0)
-    mark_tile(d, (y / TE) * d.etx + (blockIdx.x * TX) / TE, PAR, stamp);
+    mark_tile(d, (y / TE) * d.etx + x0 / TE, PAR, stamp);
+}
+
+template <typename S, int PAR, int FLOW, int MODE>
+__global__ void __launch_bounds__(TX* TY, 4) fused_step_kernel(Dev d) {
+  constexpr unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x;
+  const int prev = d.ctr[1 - PAR], stamp = prev + 1;   // (no launch of this step changes it)
+  if (MODE != 1 && blockIdx.x == 0 && blockIdx.y == 0) {
+    if (MODE == 2) wait_for_previous();
+    if (lane == 0 && threadIdx.y == 0) step_prologue<PAR>(d);
+  }
+  const bool listed = MODE == 2 && near_from_list_step(d);
+  const int cnt = listed ? d.lcount[2 + 1 - PAR] : 0;
+  for (int u = blockIdx.x;; u += gridDim.x) {
+    int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
+    bool take = true;
+    if (listed) {
+      if (u >= 36 * cnt) return;
+      int t = 0, k = 0;
+      take = near_tile(d, u, cnt, 1 - PAR, t, k, x0, y0);
+      const bool at = take && lane < 9 && listed_at(d, t, lane, 1 - PAR, prev);
+      take = take && __ffs(__ballot_sync(FULL, at)) - 1 == 8 - k;
+    } else if (MODE != 0) {   // (a warp's first nine lanes look at the tile's surroundings)
+      const int et = (y0 / TE) * d.etx + x0 / TE;
+      const bool hit = d.ntiles > COUNT_TILES
+                           ? lane == 0 && d.nearmap[(1 - PAR) * d.ntiles + et] == prev
+                           : lane < 9 && listed_at(d, et, lane, 1 - PAR, prev);
+      take = (MODE == 2) == (__any_sync(FULL, hit) != 0);
+      if (MODE == 2 && take) wait_for_previous();
+    }
+    if (take) step_tile<S, PAR, FLOW>(d, x0, y0, prev, stamp);
+    if (!listed) return;
+  }
 }
 
 // ---- TMA-staged kernel ----------------------------------------------
@@ -615,8 +635,8 @@ struct TmaLayout {
   // measured no faster on the 2048^2 cavity)
   static constexpr int NBUF = PAR ? TMA_NBUF_ODD : TMA_NBUF_EVEN;
   static constexpr int BAR_OFF = NBUF * BYTES;
-  static constexpr int IDX_OFF = BAR_OFF + 8 * NBUF;
-  static constexpr int SMEM = IDX_OFF + 16;
+  static constexpr int IDX_OFF = BAR_OFF + 8 * NBUF;   // tile mask, stamp, then 32 tile origins
+  static constexpr int SMEM = IDX_OFF + 16 + 32 * 8;
 };
 
 __device__ __forceinline__ unsigned smem_u32(const void* p) {
@@ -754,6 +774,8 @@ __device__ __forceinline__ bool tma_node(const Dev& d, const unsigned char* sb, 
 
 // One CTA's share of the pass over one lattice: CTA bid of nblk (blockIdx.x
 // and gridDim.x of a single lattice's launch; its range in a batched launch).
+// The first warp picks up to 32 tiles, one a lane; they are then staged and
+// updated in turn.
 template <typename S, int PAR, int FLOW, int MODE>
 __device__ __forceinline__ void fused_tma_body(const Dev& d, const TmaMaps& m, int bid,
                                                int nblk) {
@@ -762,17 +784,12 @@ __device__ __forceinline__ void fused_tma_body(const Dev& d, const TmaMaps& m, i
   extern __shared__ __align__(128) unsigned char smem[];
   unsigned* s_mask = reinterpret_cast<unsigned*>(smem + L::IDX_OFF);
   int* s_stamp = reinterpret_cast<int*>(s_mask + 1);   // this step's stamp
+  int2* s_xy = reinterpret_cast<int2*>(smem + L::IDX_OFF + 16);   // the picked tiles' first nodes
   const int lane = threadIdx.x, ty = threadIdx.y;
   const int tid = ty * TX + lane;
   const int nx = d.nx, ny = d.ny;
   const int tiles_x = (nx + TX - 1) / TX;
   const int ntile = tiles_x * ((ny + TY - 1) / TY);
-  // this CTA's tiles: blockIdx.x + k gridDim.x, k < cnt <= 32 (the grid is sized for
-  // it).  The CTAs resident at any moment so work on one band of tiles, which keeps
-  // the DRAM traffic of a moment within a few rows of each plane (measured 4% faster
-  // than runs of consecutive tiles per CTA).
-  const int t0 = bid, dt = nblk;
-  const int cnt = (ntile - t0 + dt - 1) / dt;
   const long long tr0 = trace_start(d);
   const int prev = d.ctr[1 - PAR];   // the previous step's stamp (no launch of this step changes it)
   // 16-bit storage: the step's part of every node's rounding seed
@@ -788,81 +805,119 @@ __device__ __forceinline__ void fused_tma_body(const Dev& d, const TmaMaps& m, i
   // node that carries flow, read once, one lane per tile, by the thread that
   // issues every copy)
   unsigned fmask = 0u;
-  auto issue = [&](int k, int j) {   // tile k of this CTA into buffer j
-    const int t = t0 + k * dt;
-    tma_issue<S, PAR, FLOW>(m, buf0 + j * L::BYTES, bar0 + 8 * j, (t % tiles_x) * TX,
-                            (t / tiles_x) * TY, (fmask >> k) & 1u);
+  auto issue = [&](int k, int j) {   // picked tile k into buffer j
+    const int2 o = s_xy[k];
+    tma_issue<S, PAR, FLOW>(m, buf0 + j * L::BYTES, bar0 + 8 * j, o.x, o.y, (fmask >> k) & 1u);
   };
-  if (ty == 0) {
-    // which of this CTA's tiles this launch takes, one lane per tile
-    const int t = t0 + lane * dt;
-    const int et = ((t / tiles_x) * TY / TE) * d.etx + (t % tiles_x) * TX / TE;
-    bool take = lane < cnt;
-    if (take && MODE != 0) take = takes_tile<PAR, MODE>(d, et, prev);
-    // (the near map is older than the kernel before this one, the state is not)
-    if (MODE == 2 && (bid == 0 || __any_sync(FULL, take))) wait_for_previous();
-    if (MODE != 1 && bid == 0 && lane == 0) step_prologue<PAR>(d);
-    fmask = !FLOW ? 0u : d.tskip ? __ballot_sync(FULL, take && d.tact[et]) : ~0u;
-    const unsigned mask = __ballot_sync(FULL, take);
-    if (lane == 0) {
-      *s_mask = mask;
-      *s_stamp = prev + 1;
-      if (mask) {
-        for (int j = 0; j < NB; ++j)
-          asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar0 + 8 * j) : "memory");
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        unsigned rest = mask;   // the first NB tiles fill the ring
-        for (int j = 0; j < NB && rest; ++j, rest &= rest - 1) issue(__ffs(rest) - 1, j);
-      }
-    }
+  if (tid == 0) {
+    for (int j = 0; j < NB; ++j)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar0 + 8 * j) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    *s_stamp = prev + 1;
   }
-  __syncthreads();
-  unsigned mask = *s_mask;   // tiles not yet processed (the same in every thread)
-  // tile coordinates of this CTA's k-th tile, advanced tile by tile
-  const int gq = dt / tiles_x, gr = dt - gq * tiles_x;
-  int cur_k = 0, ctx = t0 % tiles_x, cty = t0 / tiles_x;
+  // Which tiles: bid + k nblk, k < 32 (the grid is sized for it).  The CTAs
+  // resident at any moment so work on one band of tiles, which keeps the DRAM
+  // traffic of a moment within a few rows of each plane (measured 4% faster than
+  // runs of consecutive tiles per CTA).  The near-tile pass of a larger lattice
+  // takes units of the previous step's list instead, 32 at a time.
+  const bool listed = MODE == 2 && near_from_list(d);
+  const int units = listed ? 36 * d.lcount[2 + 1 - PAR] : ntile;
+  // A far-tile pass takes nearly every tile: its first copies are issued before
+  // it is known whether it takes them (a batch member first reads what to copy).
+  // With the near pass from the list: 2048^2 103.3 -> 100.0 us a step, 4096 x
+  // 2048 BF16 173 -> 159, 1024^2 FP16 40.4 -> 32.8 (its near tiles sat in one
+  // column of tiles, seven to a CTA).
+  const bool eager = MODE == 1 && !d.tskip;
   unsigned phases = 0u;      // bit j: phase parity the next wait on buffer j expects
   bool failed = false;
   int b = 0;                 // buffer of the current tile (tiles take the buffers in turn)
-  for (; mask; b = (b + 1 == NB) ? 0 : b + 1) {
-    const int k = __ffs(mask) - 1;
-    mask &= mask - 1;
-    const unsigned bar = bar0 + 8 * b;
-    const bool ok = mbar_wait(bar, (phases >> b) & 1u);
-    if (__syncthreads_or(!ok)) {   // the whole CTA gives up together
-      failed = true;
-      break;
-    }
-    phases ^= 1u << b;
-    const unsigned char* sb = smem + b * L::BYTES;
-    for (; cur_k < k; ++cur_k) {
-      ctx += gr;
-      cty += gq;
-      if (ctx >= tiles_x) {
-        ctx -= tiles_x;
-        ++cty;
+  unsigned mask = 0u;        // picked tiles not yet processed (the same in every thread)
+  for (int u0 = bid; MODE == 2 ? u0 < units || u0 == bid : u0 == bid; u0 += 32 * nblk) {
+    if (ty == 0) {
+      const int u = u0 + lane * nblk;
+      bool take = u < units;
+      int et = 0, px = 0, py = 0;
+      if (listed) {
+        int k = 0;
+        take = near_tile(d, u, units / 36, 1 - PAR, et, k, px, py);
+        if (take) {
+          unsigned at = 0u;
+#pragma unroll
+          for (int j = 0; j < 9; ++j) at |= listed_at(d, et, j, 1 - PAR, prev) ? 1u << j : 0u;
+          take = __ffs(at) - 1 == 8 - k;
+        }
+      } else if (take) {
+        py = u / tiles_x;
+        px = (u - py * tiles_x) * TX;
+        py *= TY;
+        et = (py / TE) * d.etx + px / TE;
+      }
+      s_xy[lane] = make_int2(px, py);
+      __syncwarp();
+      const unsigned all = __ballot_sync(FULL, take);
+      if (eager) {
+        fmask = FLOW ? ~0u : 0u;
+        if (lane == 0)
+          for (int j = 0; j < NB; ++j)
+            if ((all >> j) & 1u) issue(j, j);
+      }
+      if (MODE != 0 && !listed && take) take = takes_tile<PAR, MODE>(d, et, prev);
+      // (the near map is older than the kernel before this one, the state is not)
+      if (MODE == 2 && (bid == 0 || __any_sync(FULL, take))) wait_for_previous();
+      if (MODE != 1 && u0 == bid && bid == 0 && lane == 0) step_prologue<PAR>(d);
+      if (!eager)
+        fmask = !FLOW ? 0u : d.tskip ? __ballot_sync(FULL, take && d.tact[et]) : ~0u;
+      const unsigned mine = __ballot_sync(FULL, take);
+      if (lane == 0) {
+        *s_mask = mine;
+        if (!eager) {
+          unsigned rest = mine;   // the first NB tiles fill the ring
+          for (int j = 0; j < NB && rest; ++j, rest &= rest - 1)
+            issue(__ffs(rest) - 1, (b + j) % NB);
+        }
       }
     }
-    const int x0 = ctx * TX, y0 = cty * TY;
-    const int y = y0 + ty;
-    // interior tiles (no wall node and no wall neighbour in them) take a copy
-    // of the update with the wall logic compiled out
-    const bool edge = x0 < 2 || x0 + TX > nx - 2 || y0 < 2 || y0 + TY > ny - 2;
-    const bool unsafe = edge ? tma_node<S, PAR, FLOW, true>(d, sb, x0, y0, lane, ty, seed, s_stamp)
-                             : tma_node<S, PAR, FLOW, false>(d, sb, x0, y0, lane, ty, seed, s_stamp);
-    if (__any_sync(FULL, unsafe) && lane == 0)
-      mark_tile(d, ((unsigned)y / TE) * d.etx + (unsigned)x0 / TE, PAR, *s_stamp);
-    // every thread is done with buffer b before it is refilled with the tile
-    // NB places further on
     __syncthreads();
-    if (tid == 0) {
-      unsigned nxt = mask;   // the next NB - 1 tiles are already in flight
-      for (int j = 0; j < NB - 1 && nxt; ++j) nxt &= nxt - 1;
-      if (nxt) {
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        issue(__ffs(nxt) - 1, b);
+    mask = *s_mask;
+    const unsigned takes = mask;
+    // (the first NB tiles are under way whether they are taken or not)
+    if (eager) mask |= (1u << min(NB, (ntile - bid + nblk - 1) / nblk)) - 1u;
+    for (; mask; b = (b + 1 == NB) ? 0 : b + 1) {
+      const int k = __ffs(mask) - 1;
+      mask &= mask - 1;
+      const unsigned bar = bar0 + 8 * b;
+      const bool ok = mbar_wait(bar, (phases >> b) & 1u);
+      if (__syncthreads_or(!ok)) {   // the whole CTA gives up together
+        failed = true;
+        break;
+      }
+      phases ^= 1u << b;
+      const unsigned char* sb = smem + b * L::BYTES;
+      if (!eager || ((takes >> k) & 1u)) {
+        const int x0 = s_xy[k].x, y0 = s_xy[k].y;
+        // interior tiles (no wall node and no wall neighbour in them) take a copy
+        // of the update with the wall logic compiled out
+        const bool edge = x0 < 2 || x0 + TX > nx - 2 || y0 < 2 || y0 + TY > ny - 2;
+        const bool unsafe =
+            edge ? tma_node<S, PAR, FLOW, true>(d, sb, x0, y0, lane, ty, seed, s_stamp)
+                 : tma_node<S, PAR, FLOW, false>(d, sb, x0, y0, lane, ty, seed, s_stamp);
+        if (__any_sync(FULL, unsafe) && lane == 0)
+          mark_tile(d, ((unsigned)(y0 + ty) / TE) * d.etx + (unsigned)x0 / TE, PAR, *s_stamp);
+      }
+      // every thread is done with buffer b before it is refilled with the tile
+      // NB places further on
+      __syncthreads();
+      if (tid == 0) {
+        unsigned nxt = mask;   // the next NB - 1 tiles are already in flight
+        for (int j = 0; j < NB - 1 && nxt; ++j) nxt &= nxt - 1;
+        if (nxt) {
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+          issue(__ffs(nxt) - 1, b);
+        }
       }
     }
+    if (failed) break;
+    if (MODE == 2 && listed) __syncthreads();   // s_mask and s_xy are free
   }
   if (failed) {
     // a copy did not arrive in time: report it, and give the copies still in
@@ -901,7 +956,9 @@ __global__ void __launch_bounds__(TX* TY, TMA_MIN_CTAS)
 // variant of its own, which leaves the common one's registers alone)
 template <typename S, int PAR, int FLOW, int MODE>
 static void launch_step_one(const Dev& d, cudaStream_t s) {
-  const dim3 block(TX, TY), grid((d.nx + TX - 1) / TX, (d.ny + TY - 1) / TY);
+  const dim3 block(TX, TY);
+  dim3 grid((d.nx + TX - 1) / TX, (d.ny + TY - 1) / TY);
+  if (MODE == 2 && near_from_list_step(d)) grid = dim3(8 * d.egrid);
   if (MODE == 2 && early_launches(d))
     launch_early(fused_step_kernel<S, PAR, FLOW, MODE>, grid, block, 0, s, d);
   else fused_step_kernel<S, PAR, FLOW, MODE><<<grid, block, 0, s>>>(d);
@@ -924,9 +981,11 @@ static void launch_mode(const Dev& d, int parity, cudaStream_t s) {
 template <typename S, int PAR, int FLOW, int MODE>
 static void launch_tma_one(const Dev& d, const TmaMaps& m, cudaStream_t s) {
   const size_t sm = TmaLayout<PAR, S>::SMEM;
+  // (near tiles found from the list: two CTAs for each of the solve's, all resident)
+  const int grid = MODE == 2 && near_from_list(d) ? 2 * d.egrid : d.tgrid;
   if (MODE == 2 && early_launches(d))
-    launch_early(fused_tma_kernel<S, PAR, FLOW, MODE>, dim3(d.tgrid), dim3(TX, TY), sm, s, d, m);
-  else fused_tma_kernel<S, PAR, FLOW, MODE><<<d.tgrid, dim3(TX, TY), sm, s>>>(d, m);
+    launch_early(fused_tma_kernel<S, PAR, FLOW, MODE>, dim3(grid), dim3(TX, TY), sm, s, d, m);
+  else fused_tma_kernel<S, PAR, FLOW, MODE><<<grid, dim3(TX, TY), sm, s>>>(d, m);
 }
 
 template <typename S, int MODE>

@@ -90,7 +90,8 @@ struct Dev {
   const float* wallTl;
   int* flags;                // [2][ntiles]: per parity, the stamp of the last step that listed the tile
   int* list;                 // [2][ntiles]: the step's listed tiles, as the solve counted them
-  int* lcount;               // [2]: entries in each list
+  int* lcount;               // [2]: entries in each list; [2 + parity]: the same, kept for the
+                             // next step's near-tile pass
   int* ctr;                  // [2]: step stamp per parity (the fused pass sets ctr[p] = ctr[1-p] + 1)
   int* nearmap;              // [2][ntiles], lattices of more than COUNT_TILES tiles: per parity,
                              // the stamp of the step that listed a tile within one of this one
@@ -343,6 +344,35 @@ __device__ __forceinline__ bool near_listed(const Dev& d, int t, int par, int st
 #pragma unroll
   for (int k = 0; k < 9; ++k) hit |= listed_at(d, t, k, par, stamp);
   return hit;
+}
+// Near-tile pass of a lattice whose step keeps a list (more tiles than CTAs in
+// the solve): its work is found from the list, not by asking every tile.  Unit u
+// of 36 a listed tile: one of the nine tiles around it and four 32x8 parts of
+// that, taken by the first listed tile (row by row) among the nine around it.
+// cnt: listed tiles of the step of parity par with this stamp.  (px, py): the
+// part's first node.
+__host__ __device__ __forceinline__ bool near_from_list(const Dev& d) { return d.ntiles > d.egrid; }
+// The ordinary-load pass, one 32x8 tile per CTA, asks every tile as long as there
+// are few: at 768 x 640 (1920 of them) it ends 3 us sooner so.
+__host__ __device__ __forceinline__ bool near_from_list_step(const Dev& d) {
+  return near_from_list(d) &&
+         (long long)((d.nx + TX - 1) / TX) * ((d.ny + TY - 1) / TY) > 8 * d.egrid;
+}
+__device__ __forceinline__ bool near_tile(const Dev& d, int u, int cnt, int par, int& t, int& k,
+                                          int& px, int& py) {
+  if (u >= 36 * cnt) return false;
+  const int li = u / 36, r = u - 36 * li;
+  k = r >> 2;
+  const int l = d.list[par * d.ntiles + li];
+  const int ly = l / d.etx, lx = l - ly * d.etx;
+  int xx = lx + k % 3 - 1, yy = ly + k / 3 - 1;
+  if (d.per_x) xx = xx < 0 ? d.etx - 1 : xx >= d.etx ? 0 : xx;
+  if (d.per_y) yy = yy < 0 ? d.ety - 1 : yy >= d.ety ? 0 : yy;
+  if (xx < 0 || xx >= d.etx || yy < 0 || yy >= d.ety) return false;
+  t = yy * d.etx + xx;
+  px = xx * TE;
+  py = yy * TE + 8 * (r & 3);
+  return py < d.ny;
 }
 // inward neighbour of wall node (x, y): one node into the lattice from each wall
 // it lies on (the diagonal neighbour at a corner)
