@@ -162,11 +162,86 @@ __device__ __forceinline__ Geo node_geo(const Dev& d, int x, int y) {
   return q;
 }
 
+// Velocity and force of one flow node as in velocity(), with a1 = varphi nu_l /
+// K_eff and a2 = varphi C_F / sqrt(K_eff) as the drag's two coefficients, |u| from
+// |v|, and one reciprocal root for both powers of K_eff.
+__device__ __forceinline__ void flow_velocity(const Dev& d, float jx, float jy, float T, float fl,
+                                              float phi, float K, float varphi, float& ux,
+                                              float& uy, float& Fx, float& Fy) {
+  const float vG = varphi * (d.g_beta * (T - d.T_ref));
+  const float r = fl == 1.f ? 1.f : (1.f - phi) / (1.f - varphi);
+  const float rs = rsqrtf(K * fl * fl * fl * r * r);   // 1 / sqrt(K_eff); 0 for K = +inf
+  const float a1 = varphi * d.nu_l * rs * rs;
+  const float a2 = varphi * 1.75f * rsqrtf(175.f * varphi * varphi * varphi) * rs;
+  const float vx = jx * d.inv_rho0, vy = jy * d.inv_rho0 + 0.5f * vG;
+  const float l0 = 0.5f + 0.25f * a1;
+  const float vm = sqrtf(vx * vx + vy * vy);
+  const float inv = 1.f / (l0 + sqrtf(l0 * l0 + 0.5f * a2 * vm));
+  ux = vx * inv;
+  uy = vy * inv;
+  const float drag = a1 + a2 * (vm * inv);
+  Fx = -drag * ux;
+  Fy = vG - drag * uy;
+}
+
 // The flow collision of one node, Eq. (16)-(28): f (nine populations as
 // deviations f_i - w_i rho0) relaxed in moment space with the porous force and
 // buoyancy at temperature T, liquid fraction flc, porosity phi and
 // permeability K; fp gets the post-collision deviations, (ux, uy) the velocity.
+//
+// Written for few instructions, of which the pass is short (about 190 for this
+// function where the moments written out one by one took 270): opposite
+// populations are added and subtracted once; the density drops out (f+ needs
+// e + 2 rho and eps - rho only); the rates come divided by the rows' norms.
+// The pass at 2048^2 issues 53 instead of 64 million instructions; 768 x 640
+// 22.4 -> 21.2 us a step, 48^2 17.4 -> 16.6; u ends a third closer to FP64.
 __device__ __forceinline__ void flow_collide(const Dev& d, const float f[9], float T, float flc,
+                                             float phi, float K, float fp[9], float& ux,
+                                             float& uy) {
+  // sums and differences of opposite populations (sum_i e_i w_i = 0, so the
+  // momentum of the deviations is the momentum)
+  const float sx = f[1] + f[3], sy = f[2] + f[4], s57 = f[5] + f[7], s68 = f[6] + f[8];
+  const float ex = f[1] - f[3], ey = f[2] - f[4], e57 = f[5] - f[7], e68 = f[6] - f[8];
+  const float gx = e57 - e68, gy = e57 + e68;   // the diagonals' share of j
+  const float sa = sx + sy, sd = s57 + s68;
+  const float varphi = phi * flc;
+  float Fx, Fy;
+  flow_velocity(d, ex + gx, ey + gy, T, flc, phi, K, varphi, ux, uy, Fx, Fy);
+  const float A = d.rho0 / varphi;
+  const float RFx = d.rho0 * Fx, RFy = d.rho0 * Fy;
+  // m+ - m = -Lambda (m - m^eq) + (I - Lambda/2) S, Eq. (20) with Eq. (19), (22),
+  // (23), over the norms of M's rows: M^-1 = M^T diag(1/9, 1/36, 1/36, 1/6, 1/12,
+  // 1/6, 1/12, 1/4, 1/4); 0 for rho, rho0 F for the momentum (with Eq. 25)
+  const float xx = ux * ux, yy = uy * uy;
+  const float auu = A * (xx + yy), auF = A * (ux * Fx + uy * Fy);
+  const float a1 = d.c_e * auF - d.k_e * (sa - 2.f * f[0] + 4.f * sd - 3.f * auu);
+  const float a2 = -d.c_eps * auF - d.k_eps * (f[0] - sa + auu);
+  const float a3 = RFx * (1.f / 6.f), a5 = RFy * (1.f / 6.f);
+  const float a4 = -d.k_q * (gx - 2.f * ex + d.rho0 * ux) - d.c_q * RFx;
+  const float a6 = -d.k_q * (gy - 2.f * ey + d.rho0 * uy) - d.c_q * RFy;
+  const float a7 = 2.f * d.c_nu * (A * (ux * Fx - uy * Fy)) - d.k_nu * (sx - sy - A * (xx - yy));
+  const float a8 = d.c_nu * (A * (ux * Fy + uy * Fx)) - d.k_nu * (s57 - s68 - A * (ux * uy));
+  // f+ = f + M^-1 (m+ - m)
+  const float cx = a7 - a1 - 2.f * a2, cy = -a7 - a1 - 2.f * a2;   // axis directions
+  const float cd = 2.f * a1 + a2;                                  // diagonals
+  const float hx = a3 - 2.f * a4, hy = a5 - 2.f * a6;
+  const float tx = a3 + a4, ty = a5 + a6;
+  const float p = cd + a8, m = cd - a8, tp = tx + ty, tm = tx - ty;
+  fp[0] = f[0] + 4.f * (a2 - a1);
+  fp[1] = f[1] + (cx + hx);
+  fp[2] = f[2] + (cy + hy);
+  fp[3] = f[3] + (cx - hx);
+  fp[4] = f[4] + (cy - hy);
+  fp[5] = f[5] + (p + tp);
+  fp[6] = f[6] + (m - tm);
+  fp[7] = f[7] + (p - tp);
+  fp[8] = f[8] + (m + tm);
+}
+
+// The same collision, moment by moment.  16-bit storage keeps it: its stores
+// round stochastically, so that another last bit in FP32 stores another value for
+// one population in some thousands, and a run ends 1e-3 away in u.
+__device__ __forceinline__ void flow_collide_moments(const Dev& d, const float f[9], float T, float flc,
                                              float phi, float K, float fp[9], float& ux,
                                              float& uy) {
   // populations are stored as deviations from the rest equilibrium,
@@ -225,13 +300,48 @@ __device__ __forceinline__ void flow_collide(const Dev& d, const float f[9], flo
   fp[8] = f[8] + c_dg + a3 + a4 - a5 - a6 - a8;
 }
 
+template <typename S>
+__device__ __forceinline__ void collide(const Dev& d, const float f[9], float T, float flc,
+                                        float phi, float K, float fp[9], float& ux, float& uy) {
+  if constexpr (std::is_same<S, float>::value) flow_collide(d, f, T, flc, phi, K, fp, ux, uy);
+  else flow_collide_moments(d, f, T, flc, phi, K, fp, ux, uy);
+}
+
+// The thermal collision of one node without the latent source, Eq. (34)-(37):
+// g relaxed in moment space at temperature T, velocity (ux, uy) and liquid
+// fraction flc (sr: sigma_l / sigma(flc)), into gp.
+__device__ __forceinline__ void thermal_collide(const Dev& d, const float g[5], float T, float ux,
+                                                float uy, float flc, float sr, float gp[5]) {
+  const float n1 = g[1] - g[3], n2 = g[2] - g[4];
+  const float n3 = -4.f * g[0] + g[1] + g[2] + g[3] + g[4];
+  const float n4 = g[1] - g[2] + g[3] - g[4];
+  const float th = d.conv * d.csT2 * sr;   // vartheta / sigma
+  // zeta_alpha = 1/tau_T = 1/(1/2 + alpha_e / (sigma c_sT^2)); alpha_e follows
+  // f_l(n) with alpha_l != alpha_s (Sec. 4.1), sigma with sigma_s != sigma_l
+  const float za =
+      (d.alpha_var | d.sigma_var)
+          ? 1.f / (0.5f + (d.tauT_l - 0.5f) * (d.alpha_var ? flc + (1.f - flc) * d.inv_aratio
+                                                           : 1.f) * sr)
+          : d.z_a;
+  const float b1 = -0.5f * za * (n1 - th * ux * T);
+  const float b2 = -0.5f * za * (n2 - th * uy * T);
+  const float b3 = -0.05f * d.z_e * (n3 - d.varpi * T);
+  const float b4 = -0.25f * d.z_nu * n4;
+  gp[0] = g[0] - 4.f * b3;
+  gp[1] = g[1] + b1 + b3 + b4;
+  gp[2] = g[2] + b2 + b3 - b4;
+  gp[3] = g[3] - b1 + b3 + b4;
+  gp[4] = g[4] - b2 + b3 - b4;
+}
+
 // Non-equilibrium extrapolation of Sec. 4 from a flow node: the boundary
 // node's state f^eq(rho, 0) + f - f^eq(rho, u) (deviations: f minus the
 // velocity part of f^eq at the node's rho and u), collided with the flow
 // node's T, f_l, phi and K, into fe
-static __device__ __noinline__ void extrapolated_post(const Dev& d, const float f[9], float T, float fl,
-                                               float phi, float K, float ux, float uy,
-                                               float fe[9]) {
+template <typename S>
+static __device__ __noinline__ void extrapolated_post(const Dev& d, const float f[9], float T,
+                                                      float fl, float phi, float K, float ux,
+                                                      float uy, float fe[9]) {
   const float w9[9] = {4.f / 9.f, 1.f / 9.f, 1.f / 9.f, 1.f / 9.f, 1.f / 9.f,
                        1.f / 36.f, 1.f / 36.f, 1.f / 36.f, 1.f / 36.f};
   const float ivp = 1.f / (phi * fl);
@@ -243,7 +353,21 @@ static __device__ __noinline__ void extrapolated_post(const Dev& d, const float 
     fb[i] = f[i] - w9[i] * d.rho0 * (3.f * eu + 4.5f * eu * eu * ivp - 1.5f * uu * ivp);
   }
   float ub, vb;
-  flow_collide(d, fb, T, fl, phi, K, fe, ub, vb);
+  collide<S>(d, fb, T, fl, phi, K, fe, ub, vb);
+}
+
+// List the enthalpy tiles that hold the 3x3 neighbourhood of node (x, y), other
+// than its own (which the caller lists with one vote per warp).
+__device__ __forceinline__ void mark_around(const Dev& d, int x, int y, int xm, int xp, int ym,
+                                                int yp, int par, int stamp) {
+  const int cx = (unsigned)x / TE, cy = (unsigned)y / TE;
+  const int txs[3] = {(int)((unsigned)xm / TE), cx, (int)((unsigned)xp / TE)};
+  const int tys[3] = {(int)((unsigned)ym / TE), cy, (int)((unsigned)yp / TE)};
+#pragma unroll
+  for (int j = 0; j < 3; ++j)
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+      if (txs[i] != cx || tys[j] != cy) mark_tile(d, tys[j] * d.etx + txs[i], par, stamp);
 }
 
 // Flow walls (Sec. 4, non-equilibrium extrapolation).  A wall node x_b whose
@@ -322,8 +446,7 @@ __device__ __forceinline__ bool node_update(const Dev& d, int x, int y, const Ge
   if constexpr (!std::is_same<S, float>::value)
     rnd = mix32((unsigned)s ^ seed);
   const float flc = fln[0];
-  const float g0 = gin[0], g1 = gin[1], g2 = gin[2], g3 = gin[3], g4 = gin[4];
-  const float T = g0 + g1 + g2 + g3 + g4;
+  const float T = gin[0] + gin[1] + gin[2] + gin[3] + gin[4];
 
   // ---- flow lattice ------------------------------------------------------
   float ux = 0.f, uy = 0.f;
@@ -339,7 +462,7 @@ __device__ __forceinline__ bool node_update(const Dev& d, int x, int y, const Ge
         if (!act[opp9(i)]) f[i] = fb[i];
     }
     float fp[9];
-    flow_collide(d, f, T, flc, phi, K, fp, ux, uy);
+    collide<S>(d, f, T, flc, phi, K, fp, ux, uy);
     if (FLOW == 2) {
       // links into non-flow lattice nodes (the front; walls keep their own
       // rule): what arrives from the solid node is its extrapolated population
@@ -354,7 +477,7 @@ __device__ __forceinline__ bool node_update(const Dev& d, int x, int y, const Ge
       }
       if (fm || wm) {
         float fe[9];
-        extrapolated_post(d, f, T, flc, phi, K, ux, uy, fe);
+        extrapolated_post<S>(d, f, T, flc, phi, K, ux, uy, fe);
 #pragma unroll
         for (int i = 1; i < 9; ++i)
           if ((fm >> i) & 1u) fp[i] = fe[opp9(i)];
@@ -376,28 +499,10 @@ __device__ __forceinline__ bool node_update(const Dev& d, int x, int y, const Ge
   }
 
   // ---- thermal collision (no latent source) ------------------------------
-  const float n1 = g1 - g3, n2 = g2 - g4;
-  const float n3 = -4.f * g0 + g1 + g2 + g3 + g4;
-  const float n4 = g1 - g2 + g3 - g4;
-  // sigma_l / sigma(f_l(n)) (Eq. (7)); 1 with one sigma for both phases
-  const float sr = sigma_ratio(d, flc);
-  const float th = d.conv * d.csT2 * sr;   // vartheta / sigma
-  // zeta_alpha = 1/tau_T = 1/(1/2 + alpha_e / (sigma c_sT^2)); alpha_e follows
-  // f_l(n) with alpha_l != alpha_s (Sec. 4.1), sigma with sigma_s != sigma_l
-  const float za =
-      (d.alpha_var | d.sigma_var)
-          ? 1.f / (0.5f + (d.tauT_l - 0.5f) * (d.alpha_var ? flc + (1.f - flc) * d.inv_aratio
-                                                           : 1.f) * sr)
-          : d.z_a;
-  const float b1 = -0.5f * za * (n1 - th * ux * T);
-  const float b2 = -0.5f * za * (n2 - th * uy * T);
-  const float b3 = -0.05f * d.z_e * (n3 - d.varpi * T);
-  const float b4 = -0.25f * d.z_nu * n4;
-  const float gp0 = g0 - 4.f * b3;
-  const float gp1 = g1 + b1 + b3 + b4;
-  const float gp2 = g2 + b2 + b3 - b4;
-  const float gp3 = g3 - b1 + b3 + b4;
-  const float gp4 = g4 - b2 + b3 - b4;
+  const float sr = sigma_ratio(d, flc);   // sigma_l / sigma(f_l(n)) (Eq. (7))
+  float gp[5];
+  thermal_collide(d, gin, T, ux, uy, flc, sr, gp);
+  const float gp0 = gp[0], gp1 = gp[1], gp2 = gp[2], gp3 = gp[3], gp4 = gp[4];
   if (PAR == 0) {
     gstore(&G[s], gp0, r0, rnd);
     gstore(&G[3 * n + s], gp1, r1, rnd);
@@ -450,19 +555,46 @@ __device__ __forceinline__ bool node_update(const Dev& d, int x, int y, const Ge
 #undef LBM_WALL_POP
 
   const bool unsafe = d.screen_off || !(cold || hot);
-  if (unsafe) {
-    // list the enthalpy tiles holding this node's 3x3 neighbourhood (other
-    // than its own, which the caller lists with one vote per warp)
-    const int cx = (unsigned)x / TE, cy = (unsigned)y / TE;
-    const int txs[3] = {(int)((unsigned)q.xm / TE), cx, (int)((unsigned)q.xp / TE)};
-    const int tys[3] = {(int)((unsigned)q.ym / TE), cy, (int)((unsigned)q.yp / TE)};
-#pragma unroll
-    for (int j = 0; j < 3; ++j)
-#pragma unroll
-      for (int i = 0; i < 3; ++i)
-        if (txs[i] != cx || tys[j] != cy) mark_tile(d, tys[j] * d.etx + txs[i], PAR, *stamp);
-  }
+  if (unsafe) mark_around(d, x, y, q.xm, q.xp, q.ym, q.yp, PAR, *stamp);
   return unsafe;
+}
+
+// The update of a node of a warp that is liquid through and through (f_l = 1
+// exactly at every node and neighbour of the warp, none of them a wall node):
+// the same arithmetic on the same inputs, so the same bits, with f_l = 1 put in
+// and everything that asks about the neighbours left out.  Every store goes to
+// one plane's base (uniform over the warp) plus the node's offset.  The kernel
+// issues instructions at 70% of the rate that the SM can, so these count (with
+// the backward odd steps, 2048^2: 100.0 -> 97.8 us a step, 4096 x 2048 BF16
+// 158.8 -> 154.9).
+template <typename S, int PAR>
+__device__ __forceinline__ bool liquid_update(const Dev& d, int s, const float g[5],
+                                              const float f[9], float phi, float K,
+                                              unsigned seed) {
+  const float r0 = d.wt0 * d.g_ref, r1 = d.wt1 * d.g_ref;   // g storage reference
+  unsigned rnd = 0u;
+  if constexpr (!std::is_same<S, float>::value) rnd = mix32((unsigned)s ^ seed);
+  const float T = g[0] + g[1] + g[2] + g[3] + g[4];
+  float fp[9], gp[5], ux, uy;
+  collide<S>(d, f, T, 1.f, phi, K, fp, ux, uy);
+  const unsigned off = (unsigned)s * (unsigned)sizeof(S);
+  const long long n = d.n;
+  char* F = static_cast<char*>(d.f);
+  char* G = static_cast<char*>(d.g);
+  // population i: into the node's own slot opp(i), or the neighbour's slot i
+#define LBM_AT(B, OPP, I)                                                                  \
+  reinterpret_cast<S*>((B) + ((PAR == 0 ? OPP(I) * n : (I) * n + ey9(I) * d.nx + ex9(I)) * \
+                              (long long)sizeof(S)) +                                      \
+                       off)
+#pragma unroll
+  for (int i = 0; i < 9; ++i) fstore(LBM_AT(F, opp9, i), fp[i], rnd);
+  thermal_collide(d, g, T, ux, uy, 1.f, sigma_ratio(d, 1.f), gp);
+#pragma unroll
+  for (int i = 0; i < 5; ++i) gstore(LBM_AT(G, opp5, i), gp[i], i ? r1 : r0, rnd);
+#undef LBM_AT
+  const float hi0 = d.wt0 * (d.T_l - d.scr_T), hi1 = d.wt1 * (d.T_l - d.scr_T);
+  const bool hot = gp[0] >= hi0 && gp[1] >= hi1 && gp[2] >= hi1 && gp[3] >= hi1 && gp[4] >= hi1;
+  return d.screen_off || !hot;
 }
 
 // Flow walls (Sec. 4): which wall neighbours of node (x, y) carry flow, as bits
@@ -566,6 +698,7 @@ __device__ __forceinline__ void step_tile(const Dev& d, int x0, int y0, int prev
     mark_tile(d, (y / TE) * d.etx + x0 / TE, PAR, stamp);
 }
 
+// MODE as for launch_fused; 3: the near tiles, found from the previous step's list
 template <typename S, int PAR, int FLOW, int MODE>
 __global__ void __launch_bounds__(TX* TY, 4) fused_step_kernel(Dev d) {
   constexpr unsigned FULL = 0xffffffffu;
@@ -575,28 +708,25 @@ __global__ void __launch_bounds__(TX* TY, 4) fused_step_kernel(Dev d) {
     if (MODE == 2) wait_for_previous();
     if (lane == 0 && threadIdx.y == 0) step_prologue<PAR>(d);
   }
-  const bool listed = MODE == 2 && near_from_list_step(d);
-  const int cnt = listed ? d.lcount[2 + 1 - PAR] : 0;
-  for (int u = blockIdx.x;; u += gridDim.x) {
-    int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
-    bool take = true;
-    if (listed) {
-      if (u >= 36 * cnt) return;
-      int t = 0, k = 0;
-      take = near_tile(d, u, cnt, 1 - PAR, t, k, x0, y0);
-      const bool at = take && lane < 9 && listed_at(d, t, lane, 1 - PAR, prev);
-      take = take && __ffs(__ballot_sync(FULL, at)) - 1 == 8 - k;
-    } else if (MODE != 0) {   // (a warp's first nine lanes look at the tile's surroundings)
-      const int et = (y0 / TE) * d.etx + x0 / TE;
-      const bool hit = d.ntiles > COUNT_TILES
-                           ? lane == 0 && d.nearmap[(1 - PAR) * d.ntiles + et] == prev
-                           : lane < 9 && listed_at(d, et, lane, 1 - PAR, prev);
-      take = (MODE == 2) == (__any_sync(FULL, hit) != 0);
-      if (MODE == 2 && take) wait_for_previous();
+  if (MODE == 3) {
+    const int cnt = d.lcount[2 + 1 - PAR];
+    for (int u = blockIdx.x; u < 36 * cnt; u += gridDim.x) {
+      int t, k, x0, y0;
+      if (!near_tile(d, u, cnt, 1 - PAR, t, k, x0, y0)) continue;
+      const unsigned at = __ballot_sync(FULL, lane < 9 && listed_at(d, t, lane, 1 - PAR, prev));
+      if (__ffs(at) - 1 == 8 - k) step_tile<S, PAR, FLOW>(d, x0, y0, prev, stamp);
     }
-    if (take) step_tile<S, PAR, FLOW>(d, x0, y0, prev, stamp);
-    if (!listed) return;
+    return;
   }
+  if (MODE != 0) {   // (one tile per CTA: a warp's first nine lanes look at its surroundings)
+    const int et = ((blockIdx.y * TY) / TE) * d.etx + (blockIdx.x * TX) / TE;
+    const bool hit = d.ntiles > COUNT_TILES
+                         ? lane == 0 && d.nearmap[(1 - PAR) * d.ntiles + et] == prev
+                         : lane < 9 && listed_at(d, et, lane, 1 - PAR, prev);
+    if ((MODE == 2) != __any_sync(FULL, hit)) return;
+    if (MODE == 2) wait_for_previous();
+  }
+  step_tile<S, PAR, FLOW>(d, blockIdx.x * TX, blockIdx.y * TY, prev, stamp);
 }
 
 // ---- TMA-staged kernel ----------------------------------------------
@@ -718,10 +848,6 @@ __device__ __forceinline__ bool tma_node(const Dev& d, const unsigned char* sb, 
   const int x = x0 + lane, y = y0 + ty;
   bool unsafe = false;
   if (!EDGE || (x < nx && y < ny && !is_wall(d, x, y))) {
-      Geo q = node_geo_walled(d, x, y);
-      if (!EDGE)
-#pragma unroll
-        for (int i = 0; i < 9; ++i) q.wl[i] = false;
       const S* sF = reinterpret_cast<const S*>(sb + L::F_OFF);
       const S* sG = reinterpret_cast<const S*>(sb + L::G_OFF);
       const float r0 = d.wt0 * d.g_ref, r1 = d.wt1 * d.g_ref;
@@ -729,11 +855,42 @@ __device__ __forceinline__ bool tma_node(const Dev& d, const unsigned char* sb, 
       // f_l of the 3x3 neighbourhood from the halo window (origin x0 - 4, y0 - 1);
       // all four sides are walls, so every neighbour of a non-wall node is in it
       const int c = (ty + HY) * WX + (lane + HX);
+      constexpr int PX = L::PX, PP = L::PX * L::PY;
+      const int pc = PAR ? (ty + HY) * PX + (lane + L::HS) : ty * PX + lane;
+      if (FLOW && !EDGE) {
+        // f_l = 1 in the warp's row and around it: each lane looks at its
+        // column, the outer lanes also at the one beyond
+        const int e = c + (lane == 0 ? -1 : lane == TX - 1 ? 1 : 0);
+        const bool liquid = sFL[c - WX] == 1.f && sFL[c] == 1.f && sFL[c + WX] == 1.f &&
+                            sFL[e - WX] == 1.f && sFL[e] == 1.f && sFL[e + WX] == 1.f;
+        if (__all_sync(0xffffffffu, liquid)) {
+          float g[5], f[9];
+          g[0] = gload(&sG[pc], r0);
+          f[0] = Pop<S>::ld(&sF[pc]);
+#pragma unroll
+          for (int i = 1; i < 5; ++i) {
+            const int o = PAR ? opp5(i) : i;
+            g[i] = gload(&sG[o * PP + pc + (PAR ? ey9(o) * PX + ex9(o) : 0)], r1);
+          }
+#pragma unroll
+          for (int i = 1; i < 9; ++i) {
+            const int o = PAR ? opp9(i) : i;
+            f[i] = Pop<S>::ld(&sF[o * PP + pc + (PAR ? ey9(o) * PX + ex9(o) : 0)]);
+          }
+          const float phi = reinterpret_cast<const float*>(sb + L::PHI_OFF)[ty * TX + lane];
+          const float K = reinterpret_cast<const float*>(sb + L::K_OFF)[ty * TX + lane];
+          unsafe = liquid_update<S, PAR>(d, y * nx + x, g, f, phi, K, seed);
+          if (unsafe) mark_around(d, x, y, x - 1, x + 1, y - 1, y + 1, PAR, *stamp);
+          return unsafe;
+        }
+      }
+      Geo q = node_geo_walled(d, x, y);
+      if (!EDGE)
+#pragma unroll
+        for (int i = 0; i < 9; ++i) q.wl[i] = false;
       float fln[9];
 #pragma unroll
       for (int i = 0; i < 9; ++i) fln[i] = q.wl[i] ? -1.f : sFL[c + ey9(i) * WX + ex9(i)];
-      constexpr int PX = L::PX, PP = L::PX * L::PY;
-      const int pc = PAR ? (ty + HY) * PX + (lane + L::HS) : ty * PX + lane;
       float g[5];
       if (PAR == 0) {
 #pragma unroll
@@ -847,8 +1004,11 @@ __device__ __forceinline__ void fused_tma_body(const Dev& d, const TmaMaps& m, i
           take = __ffs(at) - 1 == 8 - k;
         }
       } else if (take) {
-        py = u / tiles_x;
-        px = (u - py * tiles_x) * TX;
+        // odd steps walk the bands backwards: what the even step touched last
+        // is still in L2 (4096 x 2048 BF16: 1% of the step)
+        const int t = PAR ? ntile - 1 - u : u;
+        py = t / tiles_x;
+        px = (t - py * tiles_x) * TX;
         py *= TY;
         et = (py / TE) * d.etx + px / TE;
       }
@@ -958,7 +1118,7 @@ template <typename S, int PAR, int FLOW, int MODE>
 static void launch_step_one(const Dev& d, cudaStream_t s) {
   const dim3 block(TX, TY);
   dim3 grid((d.nx + TX - 1) / TX, (d.ny + TY - 1) / TY);
-  if (MODE == 2 && near_from_list_step(d)) grid = dim3(8 * d.egrid);
+  if (MODE == 3) grid = dim3(8 * d.egrid);
   if (MODE == 2 && early_launches(d))
     launch_early(fused_step_kernel<S, PAR, FLOW, MODE>, grid, block, 0, s, d);
   else fused_step_kernel<S, PAR, FLOW, MODE><<<grid, block, 0, s>>>(d);
@@ -1013,6 +1173,7 @@ static void launch_fused_t(const Dev& d, const TmaMaps* m, int parity, int mode,
   }
   if (mode == 0) launch_mode<S, 0>(d, parity, s);
   else if (mode == 1) launch_mode<S, 1>(d, parity, s);
+  else if (near_from_list_step(d)) launch_mode<S, 3>(d, parity, s);
   else launch_mode<S, 2>(d, parity, s);
 }
 
