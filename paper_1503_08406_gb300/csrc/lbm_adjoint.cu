@@ -316,13 +316,14 @@ __global__ void adj_save_kernel(Dev d, float* base, unsigned* ctr, unsigned* don
   }
 }
 
-// J = mean f_l over non-wall nodes: FP64 partial sums per row block, then
+// J = mean f_l over non-wall nodes (walls left and right): FP64 partial sums per row block, then
 // their sum in a fixed order
 constexpr int OB = 256, OBLOCKS = 128;
 __global__ void __launch_bounds__(OB) adj_partial_kernel(Dev d, const float* fl, double* part) {
   __shared__ double sh[OB];
   double acc = 0.0;
-  for (int y = blockIdx.x; y < d.ny; y += gridDim.x)
+  const int y0 = d.wall_b ? 1 : 0, y1 = d.wall_t ? d.ny - 1 : d.ny;
+  for (int y = y0 + blockIdx.x; y < y1; y += gridDim.x)
     for (int x = 1 + threadIdx.x; x < d.nx - 1; x += OB) acc += fl[(long long)y * d.nx + x];
   sh[threadIdx.x] = acc;
   __syncthreads();
@@ -337,15 +338,17 @@ __global__ void adj_objective_kernel(Dev d, const double* part, int nparts, doub
   if (threadIdx.x != 0) return;
   double acc = 0.0;
   for (int k = 0; k < nparts; ++k) acc += part[k];
-  *out = acc / ((double)(d.nx - 2) * d.ny);
+  const int rows = d.ny - (d.wall_b ? 1 : 0) - (d.wall_t ? 1 : 0);
+  *out = acc / ((double)(d.nx - 2) * rows);
 }
 
-__global__ void adj_seed_kernel(Dev d, float* lamf, float* lamg, bool melt, NuSrc nu) {
+__global__ void adj_seed_kernel(Dev d, float* lamf, float* lamg, float melt, NuSrc nu) {
   const int s = blockIdx.x * AB + threadIdx.x;
   if (s >= (int)d.n) return;
-  const int x = s % d.nx;
-  lamf[s] = (melt && x != 0 && x != d.nx - 1) ? 1.f / ((float)(d.nx - 2) * d.ny) : 0.f;
-  const float src = x == 1 ? nu.g1 : x == 2 ? nu.g2 : 0.f;
+  const int y = s / d.nx, x = s - y * d.nx;
+  const bool row = !(d.wall_b && y == 0) && !(d.wall_t && y == d.ny - 1);
+  lamf[s] = is_wall(d, x, y) ? 0.f : melt;
+  const float src = !row ? 0.f : x == 1 ? nu.g1 : x == 2 ? nu.g2 : 0.f;
   for (int i = 0; i < 5; ++i) lamg[i * (int)d.n + s] = src;
 }
 
@@ -362,7 +365,7 @@ __global__ void adj_a_kernel(Dev d, float* a) {
 
 static unsigned blocks(long long n) { return (unsigned)((n + AB - 1) / AB); }
 
-void adj_seed(const Dev& d, float* lamf, float* lamg, float* a, bool melt, NuSrc nu,
+void adj_seed(const Dev& d, float* lamf, float* lamg, float* a, float melt, NuSrc nu,
               cudaStream_t s) {
   adj_seed_kernel<<<blocks(d.n), AB, 0, s>>>(d, lamf, lamg, melt, nu);
   adj_a_kernel<<<blocks(d.n), AB, 0, s>>>(d, a);
@@ -375,10 +378,6 @@ __global__ void adj_mul_kernel(long long n, float* v, const float* w) {
 
 void adj_mul(long long n, float* v, const float* w, cudaStream_t s) {
   adj_mul_kernel<<<(unsigned)((n + AB - 1) / AB), AB, 0, s>>>(n, v, w);
-}
-
-void adj_a(const Dev& d, float* a, cudaStream_t s) {
-  adj_a_kernel<<<blocks(d.n), AB, 0, s>>>(d, a);
 }
 
 void adj_scale(long long n, float* v, float k, cudaStream_t s) {

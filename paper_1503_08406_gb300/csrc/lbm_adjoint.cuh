@@ -38,17 +38,15 @@ struct NuSrc {
 // leaves the terms of its rows in rows[ny], where mode 2 finds them
 void launch_wall_nusselt(const Dev& d, int layout, int mode, int par, double* rows, double* acc,
                          cudaStream_t s);
-// a = phi dT / (sigma St); lam_g = the Nusselt terms of the last state; lam_f
-// = 1 / (non-wall nodes) on non-wall nodes for the melted fraction (melt),
-// else 0
-void adj_seed(const Dev& d, float* lamf, float* lamg, float* a, bool melt, NuSrc nu,
+// a = phi dT / (sigma St); lam_g = the Nusselt terms of the last state (rows that
+// are no horizontal wall); lam_f = melt on non-wall nodes (1 / their number for
+// the melted fraction, else 0)
+void adj_seed(const Dev& d, float* lamf, float* lamg, float* a, float melt, NuSrc nu,
               cudaStream_t s);
 // v[0..n) *= k
 void adj_scale(long long n, float* v, float k, cudaStream_t s);
 // v[0..n) *= w[0..n)
 void adj_mul(long long n, float* v, const float* w, cudaStream_t s);
-// a = phi dT / (sigma St)
-void adj_a(const Dev& d, float* a, cudaStream_t s);
 // J into out[0]; out holds 129 doubles (the rest: partial sums)
 void adj_objective(const Dev& d, const float* fl, double* out, cudaStream_t s);
 // the band (non-wall nodes with 0 < f < 1) on a list of n entries (band_append)
