@@ -432,22 +432,20 @@ int lbm_set_fields(lbm_ctx* c, const float* phi, const float* K, const float* T0
       for (int y = 0; y < c->p.ny; ++y)
         if (!isfinite(wall_T_left[y])) return LBM_ERR_INVALID_ARG;
   }
-  LBM_CUDA(cudaMemsetAsync(c->bad, 0, sizeof(int), c->stream));
   lbm::launch_validate(d, src[0], src[1], src[2], src[3], c->bad, c->stream);
   int bad = 0;
   LBM_CUDA(cudaMemcpyAsync(&bad, c->bad, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
   LBM_CUDA(cudaStreamSynchronize(c->stream));
-  if (bad) return LBM_ERR_INVALID_ARG;
-  LBM_CUDA(cudaMemcpyAsync((float*)d.phi, src[0], n * sizeof(float), cudaMemcpyDeviceToDevice,
-                           c->stream));
-  LBM_CUDA(cudaMemcpyAsync((float*)d.K, src[1], n * sizeof(float), cudaMemcpyDeviceToDevice,
-                           c->stream));
-  LBM_CUDA(cudaMemcpyAsync(d.fl, src[3], n * sizeof(float), cudaMemcpyDeviceToDevice, c->stream));
+  if (bad) {   // (0 between calls)
+    LBM_CUDA(cudaMemsetAsync(c->bad, 0, sizeof(int), c->stream));
+    return LBM_ERR_INVALID_ARG;
+  }
   if (wall_T_left)
     LBM_TRY(copy_in(c, (float*)d.wallTl, wall_T_left, (size_t)c->p.ny, device_ptrs));
-  lbm::launch_init(d, src[2], wall_T_left ? nullptr : (float*)d.wallTl, c->stream);
+  lbm::launch_load_fields(d, src[0], src[1], src[2], src[3],
+                          wall_T_left ? nullptr : (float*)d.wallTl, c->stream);
   LBM_CUDA(cudaGetLastError());
-  LBM_TRY(reset_lists(c));
+  c->since_check = 0;
   c->steps = 0;
   c->parity = 0;
   if (!device_ptrs) LBM_CUDA(cudaStreamSynchronize(c->stream));

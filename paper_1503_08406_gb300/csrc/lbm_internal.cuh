@@ -92,7 +92,8 @@ struct Dev {
   const float* phi;
   const float* K;
   const float* wallTl;
-  int* flags;                // [2][ntiles]: per parity, the stamp of the last step that listed the tile
+  int* flags;                // (nearmap and proc follow at once, 5 ntiles in all)
+                             // [2][ntiles]: per parity, the stamp of the last step that listed the tile
   int* list;                 // [2][ntiles]: the step's listed tiles, as the solve counted them
   int* lcount;               // [2]: entries in each list; [2 + parity]: the same, kept for the
                              // next step's near-tile pass
@@ -483,7 +484,8 @@ void launch_enthalpy_solve_batch(const BatchPlan& P, int parity, cudaStream_t s)
 void launch_enthalpy_commit_batch(const BatchPlan& P, int parity, cudaStream_t s);
 void enthalpy_setup();
 size_t enthalpy_solve_smem();
-void launch_init(const Dev& d, const float* T0, float* wallTl, cudaStream_t s);
+void launch_load_fields(const Dev& d, const float* phi, const float* K, const float* T0,
+                        const float* fl0, float* wallTl, cudaStream_t s);
 void launch_macros(const Dev& d, int parity, float* ux, float* uy, float* rho, float* T,
                    float* fl, cudaStream_t s);
 void launch_reduce(const Dev& d, int parity, double* partials, double* out, int nblocks,
