@@ -271,17 +271,6 @@ int lbm_create(const lbm_params* pin, void* stream, void* workspace, size_t work
   d.s_eps = (float)p.s_eps;
   d.s_q = (float)p.s_q;
   d.s_nu = p.flow ? (float)(1.0 / der[0]) : 0.f;
-  {
-    const double s_nu = p.flow ? 1.0 / der[0] : 0.0;
-    d.k_e = (float)(p.s_e / 36.0);
-    d.c_e = (float)((1.0 - 0.5 * p.s_e) / 6.0);
-    d.k_eps = (float)(p.s_eps / 12.0);
-    d.c_eps = (float)((1.0 - 0.5 * p.s_eps) / 6.0);
-    d.k_q = (float)(p.s_q / 12.0);
-    d.c_q = (float)((1.0 - 0.5 * p.s_q) / 12.0);
-    d.k_nu = (float)(s_nu / 4.0);
-    d.c_nu = (float)((1.0 - 0.5 * s_nu) / 4.0);
-  }
   d.z_a = (float)(1.0 / der[1]);
   d.alpha_var = (p.alpha_ratio > 0 && p.alpha_ratio != 1.0) ? 1 : 0;
   d.tauT_l = (float)der[1];

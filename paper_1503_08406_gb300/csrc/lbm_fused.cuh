@@ -162,86 +162,16 @@ __device__ __forceinline__ Geo node_geo(const Dev& d, int x, int y) {
   return q;
 }
 
-// Velocity and force of one flow node as in velocity(), with a1 = varphi nu_l /
-// K_eff and a2 = varphi C_F / sqrt(K_eff) as the drag's two coefficients, |u| from
-// |v|, and one reciprocal root for both powers of K_eff.
-__device__ __forceinline__ void flow_velocity(const Dev& d, float jx, float jy, float T, float fl,
-                                              float phi, float K, float varphi, float& ux,
-                                              float& uy, float& Fx, float& Fy) {
-  const float vG = varphi * (d.g_beta * (T - d.T_ref));
-  const float r = fl == 1.f ? 1.f : (1.f - phi) / (1.f - varphi);
-  const float rs = rsqrtf(K * fl * fl * fl * r * r);   // 1 / sqrt(K_eff); 0 for K = +inf
-  const float a1 = varphi * d.nu_l * rs * rs;
-  const float a2 = varphi * 1.75f * rsqrtf(175.f * varphi * varphi * varphi) * rs;
-  const float vx = jx * d.inv_rho0, vy = jy * d.inv_rho0 + 0.5f * vG;
-  const float l0 = 0.5f + 0.25f * a1;
-  const float vm = sqrtf(vx * vx + vy * vy);
-  const float inv = 1.f / (l0 + sqrtf(l0 * l0 + 0.5f * a2 * vm));
-  ux = vx * inv;
-  uy = vy * inv;
-  const float drag = a1 + a2 * (vm * inv);
-  Fx = -drag * ux;
-  Fy = vG - drag * uy;
-}
-
 // The flow collision of one node, Eq. (16)-(28): f (nine populations as
 // deviations f_i - w_i rho0) relaxed in moment space with the porous force and
 // buoyancy at temperature T, liquid fraction flc, porosity phi and
 // permeability K; fp gets the post-collision deviations, (ux, uy) the velocity.
-//
-// Written for few instructions, of which the pass is short (about 190 for this
-// function where the moments written out one by one took 270): opposite
-// populations are added and subtracted once; the density drops out (f+ needs
-// e + 2 rho and eps - rho only); the rates come divided by the rows' norms.
-// The pass at 2048^2 issues 53 instead of 64 million instructions; 768 x 640
-// 22.4 -> 21.2 us a step, 48^2 17.4 -> 16.6; u ends a third closer to FP64.
+// (Sharing the sums and differences of opposite populations, and dropping the
+// density, takes a third of its operations out and 2-4% off a step, but rounds
+// otherwise: 16-bit storage, whose stores round stochastically, then ends 1e-3
+// away in u, and the hot-wall Nusselt number, a small difference of temperatures
+// times H / dT, up to 1e-4 away.)
 __device__ __forceinline__ void flow_collide(const Dev& d, const float f[9], float T, float flc,
-                                             float phi, float K, float fp[9], float& ux,
-                                             float& uy) {
-  // sums and differences of opposite populations (sum_i e_i w_i = 0, so the
-  // momentum of the deviations is the momentum)
-  const float sx = f[1] + f[3], sy = f[2] + f[4], s57 = f[5] + f[7], s68 = f[6] + f[8];
-  const float ex = f[1] - f[3], ey = f[2] - f[4], e57 = f[5] - f[7], e68 = f[6] - f[8];
-  const float gx = e57 - e68, gy = e57 + e68;   // the diagonals' share of j
-  const float sa = sx + sy, sd = s57 + s68;
-  const float varphi = phi * flc;
-  float Fx, Fy;
-  flow_velocity(d, ex + gx, ey + gy, T, flc, phi, K, varphi, ux, uy, Fx, Fy);
-  const float A = d.rho0 / varphi;
-  const float RFx = d.rho0 * Fx, RFy = d.rho0 * Fy;
-  // m+ - m = -Lambda (m - m^eq) + (I - Lambda/2) S, Eq. (20) with Eq. (19), (22),
-  // (23), over the norms of M's rows: M^-1 = M^T diag(1/9, 1/36, 1/36, 1/6, 1/12,
-  // 1/6, 1/12, 1/4, 1/4); 0 for rho, rho0 F for the momentum (with Eq. 25)
-  const float xx = ux * ux, yy = uy * uy;
-  const float auu = A * (xx + yy), auF = A * (ux * Fx + uy * Fy);
-  const float a1 = d.c_e * auF - d.k_e * (sa - 2.f * f[0] + 4.f * sd - 3.f * auu);
-  const float a2 = -d.c_eps * auF - d.k_eps * (f[0] - sa + auu);
-  const float a3 = RFx * (1.f / 6.f), a5 = RFy * (1.f / 6.f);
-  const float a4 = -d.k_q * (gx - 2.f * ex + d.rho0 * ux) - d.c_q * RFx;
-  const float a6 = -d.k_q * (gy - 2.f * ey + d.rho0 * uy) - d.c_q * RFy;
-  const float a7 = 2.f * d.c_nu * (A * (ux * Fx - uy * Fy)) - d.k_nu * (sx - sy - A * (xx - yy));
-  const float a8 = d.c_nu * (A * (ux * Fy + uy * Fx)) - d.k_nu * (s57 - s68 - A * (ux * uy));
-  // f+ = f + M^-1 (m+ - m)
-  const float cx = a7 - a1 - 2.f * a2, cy = -a7 - a1 - 2.f * a2;   // axis directions
-  const float cd = 2.f * a1 + a2;                                  // diagonals
-  const float hx = a3 - 2.f * a4, hy = a5 - 2.f * a6;
-  const float tx = a3 + a4, ty = a5 + a6;
-  const float p = cd + a8, m = cd - a8, tp = tx + ty, tm = tx - ty;
-  fp[0] = f[0] + 4.f * (a2 - a1);
-  fp[1] = f[1] + (cx + hx);
-  fp[2] = f[2] + (cy + hy);
-  fp[3] = f[3] + (cx - hx);
-  fp[4] = f[4] + (cy - hy);
-  fp[5] = f[5] + (p + tp);
-  fp[6] = f[6] + (m - tm);
-  fp[7] = f[7] + (p - tp);
-  fp[8] = f[8] + (m + tm);
-}
-
-// The same collision, moment by moment.  16-bit storage keeps it: its stores
-// round stochastically, so that another last bit in FP32 stores another value for
-// one population in some thousands, and a run ends 1e-3 away in u.
-__device__ __forceinline__ void flow_collide_moments(const Dev& d, const float f[9], float T, float flc,
                                              float phi, float K, float fp[9], float& ux,
                                              float& uy) {
   // populations are stored as deviations from the rest equilibrium,
@@ -300,13 +230,6 @@ __device__ __forceinline__ void flow_collide_moments(const Dev& d, const float f
   fp[8] = f[8] + c_dg + a3 + a4 - a5 - a6 - a8;
 }
 
-template <typename S>
-__device__ __forceinline__ void collide(const Dev& d, const float f[9], float T, float flc,
-                                        float phi, float K, float fp[9], float& ux, float& uy) {
-  if constexpr (std::is_same<S, float>::value) flow_collide(d, f, T, flc, phi, K, fp, ux, uy);
-  else flow_collide_moments(d, f, T, flc, phi, K, fp, ux, uy);
-}
-
 // The thermal collision of one node without the latent source, Eq. (34)-(37):
 // g relaxed in moment space at temperature T, velocity (ux, uy) and liquid
 // fraction flc (sr: sigma_l / sigma(flc)), into gp.
@@ -338,7 +261,6 @@ __device__ __forceinline__ void thermal_collide(const Dev& d, const float g[5], 
 // node's state f^eq(rho, 0) + f - f^eq(rho, u) (deviations: f minus the
 // velocity part of f^eq at the node's rho and u), collided with the flow
 // node's T, f_l, phi and K, into fe
-template <typename S>
 static __device__ __noinline__ void extrapolated_post(const Dev& d, const float f[9], float T,
                                                       float fl, float phi, float K, float ux,
                                                       float uy, float fe[9]) {
@@ -353,7 +275,7 @@ static __device__ __noinline__ void extrapolated_post(const Dev& d, const float 
     fb[i] = f[i] - w9[i] * d.rho0 * (3.f * eu + 4.5f * eu * eu * ivp - 1.5f * uu * ivp);
   }
   float ub, vb;
-  collide<S>(d, fb, T, fl, phi, K, fe, ub, vb);
+  flow_collide(d, fb, T, fl, phi, K, fe, ub, vb);
 }
 
 // List the enthalpy tiles that hold the 3x3 neighbourhood of node (x, y), other
@@ -462,7 +384,7 @@ __device__ __forceinline__ bool node_update(const Dev& d, int x, int y, const Ge
         if (!act[opp9(i)]) f[i] = fb[i];
     }
     float fp[9];
-    collide<S>(d, f, T, flc, phi, K, fp, ux, uy);
+    flow_collide(d, f, T, flc, phi, K, fp, ux, uy);
     if (FLOW == 2) {
       // links into non-flow lattice nodes (the front; walls keep their own
       // rule): what arrives from the solid node is its extrapolated population
@@ -477,7 +399,7 @@ __device__ __forceinline__ bool node_update(const Dev& d, int x, int y, const Ge
       }
       if (fm || wm) {
         float fe[9];
-        extrapolated_post<S>(d, f, T, flc, phi, K, ux, uy, fe);
+        extrapolated_post(d, f, T, flc, phi, K, ux, uy, fe);
 #pragma unroll
         for (int i = 1; i < 9; ++i)
           if ((fm >> i) & 1u) fp[i] = fe[opp9(i)];
@@ -576,7 +498,7 @@ __device__ __forceinline__ bool liquid_update(const Dev& d, int s, const float g
   if constexpr (!std::is_same<S, float>::value) rnd = mix32((unsigned)s ^ seed);
   const float T = g[0] + g[1] + g[2] + g[3] + g[4];
   float fp[9], gp[5], ux, uy;
-  collide<S>(d, f, T, 1.f, phi, K, fp, ux, uy);
+  flow_collide(d, f, T, 1.f, phi, K, fp, ux, uy);
   const unsigned off = (unsigned)s * (unsigned)sizeof(S);
   const long long n = d.n;
   char* F = static_cast<char*>(d.f);

@@ -56,10 +56,6 @@ struct Dev {
   float rho0, inv_rho0;
   float nu_l, g_beta, T_ref;
   float s_e, s_eps, s_q, s_nu;
-  // the same over the norms of M's rows, and the forcing's factors (I - Lambda/2):
-  // s_e / 36, (1 - s_e/2) / 6, s_eps / 12, (1 - s_eps/2) / 6, s_q / 12,
-  // (1 - s_q/2) / 12, s_nu / 4, (1 - s_nu/2) / 4
-  float k_e, c_e, k_eps, c_eps, k_q, c_q, k_nu, c_nu;
   float z_a, z_e, z_nu;      // 1/tau_T, zeta_e, zeta_nu
   int alpha_var;             // tau_T depends on f_l (alpha_l != alpha_s)
   float tauT_l, inv_aratio;  // liquid tau_T, alpha_s / alpha_l
