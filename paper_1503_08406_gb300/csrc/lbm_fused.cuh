@@ -485,10 +485,10 @@ __device__ __forceinline__ bool node_update(const Dev& d, int x, int y, const Ge
 // exactly at every node and neighbour of the warp, none of them a wall node):
 // the same arithmetic on the same inputs, so the same bits, with f_l = 1 put in
 // and everything that asks about the neighbours left out.  Every store goes to
-// one plane's base (uniform over the warp) plus the node's offset.  The kernel
-// issues instructions at 70% of the rate that the SM can, so these count (with
-// the backward odd steps, 2048^2: 100.0 -> 97.8 us a step, 4096 x 2048 BF16
-// 158.8 -> 154.9).
+// one plane's base (uniform over the warp) plus the node's offset.  For 16-bit
+// storage only, whose pass is bound by instruction issue (4096 x 2048 BF16 157.1
+// -> 153.8 us a step, 1024^2 FP16 32.8 -> 32.3); FP32 does not gain at 2048^2 and
+// a batch of FP32 lattices loses 3%.
 template <typename S, int PAR>
 __device__ __forceinline__ bool liquid_update(const Dev& d, int s, const float g[5],
                                               const float f[9], float phi, float K,
@@ -779,7 +779,7 @@ __device__ __forceinline__ bool tma_node(const Dev& d, const unsigned char* sb, 
       const int c = (ty + HY) * WX + (lane + HX);
       constexpr int PX = L::PX, PP = L::PX * L::PY;
       const int pc = PAR ? (ty + HY) * PX + (lane + L::HS) : ty * PX + lane;
-      if (FLOW && !EDGE) {
+      if (FLOW && !EDGE && sizeof(S) == 2) {
         // f_l = 1 in the warp's row and around it: each lane looks at its
         // column, the outer lanes also at the one beyond
         const int e = c + (lane == 0 ? -1 : lane == TX - 1 ? 1 : 0);
