@@ -357,7 +357,9 @@ int lbm_timing_read(lbm_ctx* c, double ms[4], int64_t* steps_timed, int64_t* til
  * + 10 + pass for the stream-collide kernel, pass 0 all tiles, 1 tiles away
  * from the front, 2 tiles near it; + 20 the solve; + 30 the commit), the step
  * stamp (the same for all launches of one step), and the CTA's start and end
- * times in ns of the GPU's global timer.  Records beyond the capacity are
+ * times in ns of the GPU's global timer.  While on, every kernel is launched
+ * after the end of the one before it (small lattices otherwise launch the
+ * commit and the near-tile pass early).  Records beyond the capacity are
  * dropped.  Synchronises; CUDA graphs are captured again afterwards. */
 int lbm_trace(lbm_ctx* c, int64_t capacity);
 /* Copy up to max_records records (4 int64 each, in the order CTAs ended) to

@@ -433,7 +433,7 @@ __device__ __forceinline__ void solve_tile(const Dev& d, SolveSmem& sm, int tile
 // batched one) takes listed tiles bid, bid + nblk, ...
 //
 // Bound by latency: one tile's chain of the stamps, the loads, the fixing pass
-// and some thirteen sweeps, on one SM (10 us of the 20 us step at 256^2).  It
+// and some thirteen sweeps, on one SM (8 us of the 17.5 us step at 256^2).  It
 // took 23 us there (40 us beside the far tiles at 2048^2) when the sweeps ran
 // over the bounding box of the nodes left: solid at exactly T_s is not clamped
 // by the margin test, so the box was half the region, three nodes a thread, and
