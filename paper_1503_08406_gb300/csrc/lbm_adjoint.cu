@@ -49,7 +49,8 @@ __device__ __forceinline__ float wt(const Dev& d, int i) { return i == 0 ? d.wt0
 
 // Each reversed step is two kernels.  adj_band_kernel solves the fixed point's
 // adjoint on the unclamped nodes, a band along the front, and leaves nu = c mu
-// there (0 elsewhere).  adj_full_kernel passes over the whole lattice once: with lam_g+_i(x) = lam_g'_i(x + e_i) + nu(x + e_i) and
+// there (0 elsewhere).  adj_full_kernel passes over the whole lattice once:
+// with lam_g+_i(x) = lam_g'_i(x + e_i) + nu(x + e_i) and
 // S(y) = sum_i w~_i lam_g+_i(y) (the source adjoint of step F, the fixed
 // point's share included),
 //   lam_gpre = A^T lam_g+ per node
