@@ -304,6 +304,7 @@ int lbm_create(const lbm_params* pin, void* stream, void* workspace, size_t work
   d.etx = (p.nx + lbm::TE - 1) / lbm::TE;
   d.ety = (p.ny + lbm::TE - 1) / lbm::TE;
   d.ntiles = d.etx * d.ety;
+  d.seam = lbm::seam_axes(d.nx, d.ny, d.per_x, d.per_y);
   {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
@@ -501,10 +502,10 @@ static int launch_fl_hook(lbm_ctx* c, const Hooks* h, cudaStream_t s) {
 
 // Record `steps` steps starting at parity `start` on c->cap, which is being
 // captured (alone, or as one branch of a batch capture); returns the number of
-// kernels.  The fused pass of step k+1 is split: its tiles more than one tile
-// away from step k's listed tiles run on a second stream concurrently with step
-// k's enthalpy solve and commit (which touch only nodes within eight nodes of a
-// listed tile); the tiles near the front run after the commit.  Everything
+// kernels.  The fused pass of step k+1 is split: its tiles away from step k's
+// listed tiles run on a second stream concurrently with step k's enthalpy solve
+// and commit (which touch only nodes of the listed tiles' regions, so of the
+// tiles around them: near_place); the tiles near the front run after the commit.  Everything
 // forked onto the second stream joins back before the last kernel.
 // Hooks that read populations read the far tiles' before that pass and the
 // others' after the commit.

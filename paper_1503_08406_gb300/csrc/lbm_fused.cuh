@@ -71,8 +71,7 @@ __device__ __forceinline__ void fstore(S* p, float v, unsigned& rnd) {
 // COUNT_TILES tiles that is one store that nothing waits for: the solve kernel
 // counts the stamped tiles itself (an append to a list, a chain of three
 // memory round trips, ends a small lattice's pass 2 us later).  A larger one
-// appends to the step's list, and stamps the tiles within one tile of it in the
-// near map, which costs its long pass nothing and spares every CTA of the solve
+// appends to the step's list, and stamps the tiles around it in the near map, which costs its long pass nothing and spares every CTA of the solve
 // a walk over all the flags.
 __device__ __forceinline__ void mark_tile(const Dev& d, int t, int par, int stamp) {
   int* fl = d.flags + par * d.ntiles + t;
@@ -80,14 +79,7 @@ __device__ __forceinline__ void mark_tile(const Dev& d, int t, int par, int stam
     *fl = stamp;
   } else if (*fl != stamp && atomicExch(fl, stamp) != stamp) {
     d.list[par * d.ntiles + atomicAdd(&d.lcount[par], 1)] = t;
-    const int ty = t / d.etx, tx = t - ty * d.etx;
-    for (int k = 0; k < 9; ++k) {
-      int xx = tx + k % 3 - 1, yy = ty + k / 3 - 1;
-      if (d.per_x) xx = xx < 0 ? d.etx - 1 : xx >= d.etx ? 0 : xx;
-      if (d.per_y) yy = yy < 0 ? d.ety - 1 : yy >= d.ety ? 0 : yy;
-      if (xx >= 0 && xx < d.etx && yy >= 0 && yy < d.ety)
-        d.nearmap[par * d.ntiles + yy * d.etx + xx] = stamp;
-    }
+    mark_near(d, t, par, stamp);
   }
 }
 
@@ -546,8 +538,8 @@ __device__ __forceinline__ void step_prologue(const Dev& d) {
 }
 
 // Split steps: does this launch (MODE 1 far tiles, MODE 2 near tiles) take the
-// tile whose enthalpy tile is et?  Near: within one tile of a tile the previous
-// step (its stamp: prev) listed.
+// tile whose enthalpy tile is et?  Near: around a tile (near_place) that the
+// previous step (its stamp: prev) listed.
 template <int PAR, int MODE>
 __device__ __forceinline__ bool takes_tile(const Dev& d, int et, int prev) {
   if (MODE == 0) return true;
@@ -632,19 +624,21 @@ __global__ void __launch_bounds__(TX* TY, 4) fused_step_kernel(Dev d) {
   }
   if (MODE == 3) {
     const int cnt = d.lcount[2 + 1 - PAR];
-    for (int u = blockIdx.x; u < 36 * cnt; u += gridDim.x) {
+    const int places = near_places(d);
+    for (int u = blockIdx.x; u < 4 * places * cnt; u += gridDim.x) {
       int t, k, x0, y0;
-      if (!near_tile(d, u, cnt, 1 - PAR, t, k, x0, y0)) continue;
-      const unsigned at = __ballot_sync(FULL, lane < 9 && listed_at(d, t, lane, 1 - PAR, prev));
-      if (__ffs(at) - 1 == 8 - k) step_tile<S, PAR, FLOW>(d, x0, y0, prev, stamp);
+      if (!near_tile(d, u, cnt, places, 1 - PAR, t, k, x0, y0)) continue;
+      const unsigned at =
+          __ballot_sync(FULL, lane < places && listed_at(d, t, lane, 1 - PAR, prev));
+      if (__ffs(at) - 1 == near_inverse(k)) step_tile<S, PAR, FLOW>(d, x0, y0, prev, stamp);
     }
     return;
   }
-  if (MODE != 0) {   // (one tile per CTA: a warp's first nine lanes look at its surroundings)
+  if (MODE != 0) {   // (one tile per CTA: a warp's first lanes look at its surroundings)
     const int et = ((blockIdx.y * TY) / TE) * d.etx + (blockIdx.x * TX) / TE;
     const bool hit = d.ntiles > COUNT_TILES
                          ? lane == 0 && d.nearmap[(1 - PAR) * d.ntiles + et] == prev
-                         : lane < 9 && listed_at(d, et, lane, 1 - PAR, prev);
+                         : lane < near_places(d) && listed_at(d, et, lane, 1 - PAR, prev);
     if ((MODE == 2) != __any_sync(FULL, hit)) return;
     if (MODE == 2) wait_for_previous();
   }
@@ -900,7 +894,8 @@ __device__ __forceinline__ void fused_tma_body(const Dev& d, const TmaMaps& m, i
   // runs of consecutive tiles per CTA).  The near-tile pass of a larger lattice
   // takes units of the previous step's list instead, 32 at a time.
   const bool listed = MODE == 2 && near_from_list(d);
-  const int units = listed ? 36 * d.lcount[2 + 1 - PAR] : ntile;
+  constexpr int PLACES = 9;   // (walls on every side: no seam)
+  const int units = listed ? 4 * PLACES * d.lcount[2 + 1 - PAR] : ntile;
   // A far-tile pass takes nearly every tile: its first copies are issued before
   // it is known whether it takes them (a batch member first reads what to copy).
   // With the near pass from the list: 2048^2 103.3 -> 100.0 us a step, 4096 x
@@ -918,11 +913,11 @@ __device__ __forceinline__ void fused_tma_body(const Dev& d, const TmaMaps& m, i
       int et = 0, px = 0, py = 0;
       if (listed) {
         int k = 0;
-        take = near_tile(d, u, units / 36, 1 - PAR, et, k, px, py);
+        take = near_tile(d, u, units / (4 * PLACES), PLACES, 1 - PAR, et, k, px, py);
         if (take) {
           unsigned at = 0u;
 #pragma unroll
-          for (int j = 0; j < 9; ++j) at |= listed_at(d, et, j, 1 - PAR, prev) ? 1u << j : 0u;
+          for (int j = 0; j < PLACES; ++j) at |= listed_at(d, et, j, 1 - PAR, prev) ? 1u << j : 0u;
           take = __ffs(at) - 1 == 8 - k;
         }
       } else if (take) {

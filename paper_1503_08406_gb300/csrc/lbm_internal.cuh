@@ -27,15 +27,11 @@
 
 #include <type_traits>
 
+#include "lbm_tiles.cuh"
+
 namespace lbm {
 
-constexpr int TX = 32;       // fused kernel tile (threads x)
-constexpr int TY = 8;        // fused kernel tile (threads y)
-constexpr int TE = 32;       // enthalpy tile edge
-constexpr int RH = 8;        // enthalpy halo width
-constexpr int RE = TE + 2 * RH;
 constexpr int EB = 576;      // enthalpy solve block size: 12 rows of a region (solve_tile)
-constexpr int COUNT_TILES = 1152;   // up to this many tiles the solve counts the listed ones itself
 constexpr int CB = 1024;     // enthalpy commit block size (one thread per node of a tile:
                              // narrower CTAs measured slower beside the far-tile pass)
 constexpr int RB = 256;      // reduction block size
@@ -75,6 +71,7 @@ struct Dev {
   float H_over_dT;
   int etx, ety;              // enthalpy tiles
   int ntiles;                // etx * ety
+  int seam;                  // seam_axes: axes on which near tiles lie across a narrow last one
   int egrid, cgrid;          // CTAs of the enthalpy solve / commit kernels (they walk the tile list)
   int tgrid;                 // CTAs of the TMA-staged fused kernel
   int tslots;                // its CTAs resident at once (SMs x CTAs per SM)
@@ -95,7 +92,7 @@ struct Dev {
                              // next step's near-tile pass
   int* ctr;                  // [2]: step stamp per parity (the fused pass sets ctr[p] = ctr[1-p] + 1)
   int* nearmap;              // [2][ntiles], lattices of more than COUNT_TILES tiles: per parity,
-                             // the stamp of the step that listed a tile within one of this one
+                             // the stamp of the step that listed a tile around this one (mark_near)
   int* proc;                 // per enthalpy tile: (stamp << 3) | bits, bit 0 solved, bit 1
                              // some f_l changed, bit 2 some node's flow activity changed
   float2* scr;               // per node of solved tiles: (f_l(n), f_l(n+1))
@@ -325,55 +322,6 @@ __device__ __forceinline__ int wrapy(const Dev& d, int y) {
 __device__ __forceinline__ bool is_wall(const Dev& d, int x, int y) {
   return (d.wall_l && x == 0) || (d.wall_r && x == d.nx - 1) || (d.wall_b && y == 0) ||
          (d.wall_t && y == d.ny - 1);
-}
-// Near map.  Up to COUNT_TILES tiles: was neighbour k (0..8, row by row; 4 is t
-// itself) of tile t listed in the step of parity par with this stamp?
-__device__ __forceinline__ bool listed_at(const Dev& d, int t, int k, int par, int stamp) {
-  const int ty = t / d.etx, tx = t - ty * d.etx;
-  int xx = tx + k % 3 - 1, yy = ty + k / 3 - 1;
-  if (d.per_x) xx = xx < 0 ? d.etx - 1 : xx >= d.etx ? 0 : xx;
-  if (d.per_y) yy = yy < 0 ? d.ety - 1 : yy >= d.ety ? 0 : yy;
-  if (xx < 0 || xx >= d.etx || yy < 0 || yy >= d.ety) return false;
-  return d.flags[par * d.ntiles + yy * d.etx + xx] == stamp;
-}
-// Was a tile within one tile of tile t listed?  Nine independent loads on a
-// small lattice, where they wait once; one on a large one, whose CTAs are many
-// (2048^2: nine took 3% of the step) and whose marks keep a map of it.
-__device__ __forceinline__ bool near_listed(const Dev& d, int t, int par, int stamp) {
-  if (d.ntiles > COUNT_TILES) return d.nearmap[par * d.ntiles + t] == stamp;
-  bool hit = false;
-#pragma unroll
-  for (int k = 0; k < 9; ++k) hit |= listed_at(d, t, k, par, stamp);
-  return hit;
-}
-// Near-tile pass of a lattice whose step keeps a list (more tiles than CTAs in
-// the solve): its work is found from the list, not by asking every tile.  Unit u
-// of 36 a listed tile: one of the nine tiles around it and four 32x8 parts of
-// that, taken by the first listed tile (row by row) among the nine around it.
-// cnt: listed tiles of the step of parity par with this stamp.  (px, py): the
-// part's first node.
-__host__ __device__ __forceinline__ bool near_from_list(const Dev& d) { return d.ntiles > d.egrid; }
-// The ordinary-load pass, one 32x8 tile per CTA, asks every tile as long as there
-// are few: at 768 x 640 (1920 of them) it ends 3 us sooner so.
-__host__ __device__ __forceinline__ bool near_from_list_step(const Dev& d) {
-  return near_from_list(d) &&
-         (long long)((d.nx + TX - 1) / TX) * ((d.ny + TY - 1) / TY) > 8 * d.egrid;
-}
-__device__ __forceinline__ bool near_tile(const Dev& d, int u, int cnt, int par, int& t, int& k,
-                                          int& px, int& py) {
-  if (u >= 36 * cnt) return false;
-  const int li = u / 36, r = u - 36 * li;
-  k = r >> 2;
-  const int l = d.list[par * d.ntiles + li];
-  const int ly = l / d.etx, lx = l - ly * d.etx;
-  int xx = lx + k % 3 - 1, yy = ly + k / 3 - 1;
-  if (d.per_x) xx = xx < 0 ? d.etx - 1 : xx >= d.etx ? 0 : xx;
-  if (d.per_y) yy = yy < 0 ? d.ety - 1 : yy >= d.ety ? 0 : yy;
-  if (xx < 0 || xx >= d.etx || yy < 0 || yy >= d.ety) return false;
-  t = yy * d.etx + xx;
-  px = xx * TE;
-  py = yy * TE + 8 * (r & 3);
-  return py < d.ny;
 }
 // inward neighbour of wall node (x, y): one node into the lattice from each wall
 // it lies on (the diagonal neighbour at a corner)
