@@ -78,16 +78,19 @@ __device__ __forceinline__ bool band_node(const Dev& d, const float* f, int t) {
 __global__ void adj_list_kernel(Dev d, const float* f, int* list, int* count, int* pos) {
   const int s = blockIdx.x * AB + threadIdx.x;
   if (s >= (int)d.n) return;
-  if (band_node(d, f, s)) band_append(list, count, pos, (int)d.n, s, (s / d.nx + s % d.nx) & 1);
+  if (band_node(d, f, s))
+    band_append(list, count, pos, (int)d.n, band_main(d.nx, d.ny, d.per_y), s,
+                band_colour(s % d.nx, s / d.nx, d.ny, d.per_y));
 }
 
 // The fixed point's adjoint on the band: right-hand side
 // lam_f'(y) - a(y) sum_i w~_i lam_g'_i(y + e_i), then red-black sweeps with the
 // self term exact, from mu = 0: nodes with x + y even, then odd (a node's four
 // neighbours have the other colour, so each colour updates in place, in any
-// order), over-relaxed by MU_OMEGA for the first MU_SOR sweeps, until no node
-// changes by more than MU_RTOL of its value or after max_sweeps.  The result
-// does not depend on the list's order.
+// order; a periodic y axis of odd length has two more colours, band_colour),
+// over-relaxed by MU_OMEGA for the first MU_SOR sweeps, until no node changes by
+// more than MU_RTOL of its value or after max_sweeps.  The result does not depend
+// on the list's order.
 //
 // Every CTA takes a share of the band's nodes and gathers their coefficients
 // into arrays in the band's order; the last CTA to finish does the sweeps, from
@@ -118,11 +121,12 @@ __global__ void __launch_bounds__(BAND_THREADS, 1) adj_band_kernel(Dev d, AdjBuf
   // thread t of CTA k takes every BAND_CTAS-th node, so that a short band
   // spreads over all CTAs
   const int first = threadIdx.x * gridDim.x + blockIdx.x, step = gridDim.x * BAND_THREADS;
-  const int n0 = count[0], cnt = n0 + count[1];
-  const int o0 = old_count[0], ocnt = o0 + old_count[1];
-  for (int j = first; j < ocnt; j += step) b.nu[old_list[j < o0 ? j : n - 1 - (j - o0)]] = 0.f;
+  const int m = band_main(d.nx, d.ny, d.per_y);
+  const BandOrder now(count, n, m), old(old_count, n, m);
+  const int cnt = now.e4;
+  for (int j = first; j < old.e4; j += step) b.nu[old_list[old.entry(j)]] = 0.f;
   for (int j = first; j < cnt; j += step) {
-    const int s = list[j < n0 ? j : n - 1 - (j - n0)];
+    const int s = list[now.entry(j)];
     const int y = s / d.nx, x = s - y * d.nx;
     float lg[5], f4[4], a4[4];
     int p4[4];
@@ -146,7 +150,7 @@ __global__ void __launch_bounds__(BAND_THREADS, 1) adj_band_kernel(Dev d, AdjBuf
     for (int i = 0; i < 4; ++i) {
       const bool on = adj_mushy(f4[i]);
       c4[i] = on ? 1.f / (d.dTt + a4[i]) : 0.f;
-      p4[i] = !on ? j : p4[i] < n0 ? p4[i] : n0 + (n - 1 - p4[i]);
+      p4[i] = !on ? j : now.order(p4[i]);
     }
     float L = 0.f;
 #pragma unroll
@@ -162,6 +166,7 @@ __global__ void __launch_bounds__(BAND_THREADS, 1) adj_band_kernel(Dev d, AdjBuf
   __syncthreads();
   if (!last) return;
   __threadfence();
+  const int colours = now.e4 > now.e2 ? 4 : 2;
   if (cnt <= BAND_CAP) {
     float4* ct = band_smem;
     ushort4* ix = reinterpret_cast<ushort4*>(ct + BAND_CAP);
@@ -182,8 +187,8 @@ __global__ void __launch_bounds__(BAND_THREADS, 1) adj_band_kernel(Dev d, AdjBuf
     for (int k = 0; k < max_sweeps && more; ++k) {
       const float om = k < MU_SOR ? MU_OMEGA : 1.f;
       int moved = 0;
-      for (int c0 = 0; c0 < 2; ++c0) {
-        for (int j = (c0 ? n0 : 0) + threadIdx.x; j < (c0 ? cnt : n0); j += BAND_THREADS) {
+      for (int c0 = 0, lo = 0, hi = now.e1; c0 < colours; ++c0) {
+        for (int j = lo + threadIdx.x; j < hi; j += BAND_THREADS) {
           const float4 c = ct[j];
           const ushort4 q = ix[j];
           const float nb = c.x * mu[q.x] + c.y * mu[q.y] + c.z * mu[q.z] + c.w * mu[q.w];
@@ -193,12 +198,14 @@ __global__ void __launch_bounds__(BAND_THREADS, 1) adj_band_kernel(Dev d, AdjBuf
           moved |= fabsf(v - o) > MU_RTOL * fabsf(v);
           mu[j] = v;
         }
-        if (c0 == 0) __syncthreads();
+        lo = hi;
+        hi = c0 == 0 ? now.e2 : c0 == 1 ? now.e3 : now.e4;
+        if (c0 + 1 < colours) __syncthreads();
       }
       more = __syncthreads_or(moved);
     }
     for (int j = threadIdx.x; j < cnt; j += BAND_THREADS)
-      b.nu[list[j < n0 ? j : n - 1 - (j - n0)]] = mu[j] / __ldcg(b.bk + j).z;
+      b.nu[list[now.entry(j)]] = mu[j] / __ldcg(b.bk + j).z;
   } else {
     float* mu = b.mu;
     for (int j = threadIdx.x; j < cnt; j += BAND_THREADS) mu[j] = 0.f;
@@ -207,8 +214,8 @@ __global__ void __launch_bounds__(BAND_THREADS, 1) adj_band_kernel(Dev d, AdjBuf
     for (int k = 0; k < max_sweeps && more; ++k) {
       const float om = k < MU_SOR ? MU_OMEGA : 1.f;
       int moved = 0;
-      for (int c0 = 0; c0 < 2; ++c0) {
-        for (int j = (c0 ? n0 : 0) + threadIdx.x; j < (c0 ? cnt : n0); j += BAND_THREADS) {
+      for (int c0 = 0, lo = 0, hi = now.e1; c0 < colours; ++c0) {
+        for (int j = lo + threadIdx.x; j < hi; j += BAND_THREADS) {
           const float4 c = __ldcg(b.bc + j), kj = __ldcg(b.bk + j);
           const int4 q = __ldcg(b.bi + j);
           const float nb = c.x * mu[q.x] + c.y * mu[q.y] + c.z * mu[q.z] + c.w * mu[q.w];
@@ -218,15 +225,17 @@ __global__ void __launch_bounds__(BAND_THREADS, 1) adj_band_kernel(Dev d, AdjBuf
           moved |= fabsf(v - o) > MU_RTOL * fabsf(v);
           mu[j] = v;
         }
-        if (c0 == 0) __syncthreads();
+        lo = hi;
+        hi = c0 == 0 ? now.e2 : c0 == 1 ? now.e3 : now.e4;
+        if (c0 + 1 < colours) __syncthreads();
       }
       more = __syncthreads_or(moved);
     }
     for (int j = threadIdx.x; j < cnt; j += BAND_THREADS)
-      b.nu[list[j < n0 ? j : n - 1 - (j - n0)]] = mu[j] / __ldcg(b.bk + j).z;
+      b.nu[list[now.entry(j)]] = mu[j] / __ldcg(b.bk + j).z;
   }
   if (threadIdx.x == 0) {
-    old_count[0] = old_count[1] = 0;
+    old_count[0] = old_count[1] = old_count[2] = old_count[3] = 0;
     *b.done = 0;
   }
 }
@@ -295,7 +304,9 @@ __global__ void __launch_bounds__(AB) adj_full_kernel(Dev d, AdjBuffers b, Mat5 
     const float fa = f0[s], fb = f1[s];
     b.lamf[s] = __ldg(b.a + s) * S;
     if (fb != fa) b.lama[s] += -(fb - fa) * S;   // (adds 0 elsewhere)
-    if (adj_mushy(fa)) band_append(next_list, next_count, b.pos, n, s, (x + y) & 1);
+    if (adj_mushy(fa))
+      band_append(next_list, next_count, b.pos, n, band_main(d.nx, d.ny, d.per_y), s,
+                  band_colour(x, y, d.ny, d.per_y));
   }
 }
 

@@ -10,7 +10,7 @@ struct AdjBuffers {
   float* a;          // a = phi dT / (sigma St)
   float* lamg;       // 5 n: adjoint of the populations after the step being reversed
   float* lamf;       // adjoint of f_l after the step (in), before it (out)
-  // band nodes, by place in the band's order (colour 0, then colour 1):
+  // band nodes, by place in the band's order (BandOrder):
   float4* bc;        // c of the four neighbours, 0 off the band
   int4* bi;          // their places
   float4* bk;        // right-hand side, a w~_1 (both divided by the self term), T_l - T_s + a
@@ -49,7 +49,8 @@ void adj_scale(long long n, float* v, float k, cudaStream_t s);
 void adj_mul(long long n, float* v, const float* w, cudaStream_t s);
 // J into out[0]; out holds 129 doubles (the rest: partial sums)
 void adj_objective(const Dev& d, const float* fl, double* out, cudaStream_t s);
-// the band (non-wall nodes with 0 < f < 1) on a list of n entries (band_append)
+// the band (non-wall nodes with 0 < f < 1) on a list of n entries, four counts
+// (band_append)
 void adj_list(const Dev& d, const float* f, int* list, int* count, int* pos, cudaStream_t s);
 // d.fl to base + k n, k = ctr[0], which then advances (ctr[1]: scratch, 0)
 void adj_save(const Dev& d, float* base, unsigned* ctr, cudaStream_t s);

@@ -1444,7 +1444,7 @@ int lbm_adjoint(lbm_ctx* c, int objective, int64_t nsteps, int32_t checkpoint_ev
   b.lamtw = mem.get((size_t)c->d.ny);
   b.pos = reinterpret_cast<int*>(mem.get(n));
   int* lists[2] = {reinterpret_cast<int*>(mem.get(n)), reinterpret_cast<int*>(mem.get(n))};
-  int* counts = reinterpret_cast<int*>(mem.get(4));   // two a list
+  int* counts = reinterpret_cast<int*>(mem.get(8));   // four a list
   unsigned* ctr = reinterpret_cast<unsigned*>(mem.get(2));
   double* nu_acc = reinterpret_cast<double*>(mem.get(2));
   double* nu_rows = reinterpret_cast<double*>(mem.get(2 * (size_t)c->d.ny));
@@ -1525,7 +1525,7 @@ int lbm_adjoint(lbm_ctx* c, int objective, int64_t nsteps, int32_t checkpoint_ev
   // reverse sweep
   LBM_CUDA(cudaMemsetAsync(b.lama, 0, n * sizeof(float), c->stream));
   LBM_CUDA(cudaMemsetAsync(b.lamtw, 0, c->d.ny * sizeof(float), c->stream));
-  LBM_CUDA(cudaMemsetAsync(counts, 0, 4 * sizeof(int), c->stream));
+  LBM_CUDA(cudaMemsetAsync(counts, 0, 8 * sizeof(int), c->stream));
   LBM_CUDA(cudaMemsetAsync(b.nu, 0, n * sizeof(float), c->stream));
   LBM_CUDA(cudaMemsetAsync(b.done, 0, sizeof(unsigned), c->stream));
   lbm::adj_list(c->d, fl_end, lists[0], counts, b.pos, c->stream);
@@ -1534,8 +1534,8 @@ int lbm_adjoint(lbm_ctx* c, int objective, int64_t nsteps, int32_t checkpoint_ev
   auto reverse = [&](cudaStream_t sm, const float* F, int64_t lo, int64_t hi) {
     for (int64_t m = hi - 1; m >= lo; --m) {
       const float* f0 = F + (size_t)(m - lo) * n;
-      lbm::adj_step(c->d, b, f0, f0 + n, lists[cur], counts + 2 * cur, lists[1 - cur],
-                    counts + 2 * (1 - cur), sweeps, nu, sm);
+      lbm::adj_step(c->d, b, f0, f0 + n, lists[cur], counts + 4 * cur, lists[1 - cur],
+                    counts + 4 * (1 - cur), sweeps, nu, sm);
       std::swap(b.lamg, b.lamgpre);
       cur ^= 1;
     }
@@ -1677,7 +1677,7 @@ int lbm_adjoint_coupled(lbm_ctx* c, int objective, int64_t nsteps, int32_t check
   b.pos = reinterpret_cast<int*>(mem.get(n));
   float* lK = mem.get(n);
   int* lists[2] = {reinterpret_cast<int*>(mem.get(n)), reinterpret_cast<int*>(mem.get(n))};
-  int* counts = reinterpret_cast<int*>(mem.get(4));   // two a list
+  int* counts = reinterpret_cast<int*>(mem.get(8));   // four a list
   double* nu_acc = reinterpret_cast<double*>(mem.get(2));
   double* nu_rows = reinterpret_cast<double*>(mem.get(2 * (size_t)d.ny));
   unsigned* ctr = reinterpret_cast<unsigned*>(mem.get(4));   // two counter pairs
@@ -1731,7 +1731,7 @@ int lbm_adjoint_coupled(lbm_ctx* c, int objective, int64_t nsteps, int32_t check
   LBM_CUDA(cudaMemsetAsync(b.lama, 0, n * sizeof(float), c->stream));
   LBM_CUDA(cudaMemsetAsync(lK, 0, n * sizeof(float), c->stream));
   LBM_CUDA(cudaMemsetAsync(b.lamtw, 0, d.ny * sizeof(float), c->stream));
-  LBM_CUDA(cudaMemsetAsync(counts, 0, 4 * sizeof(int), c->stream));
+  LBM_CUDA(cudaMemsetAsync(counts, 0, 8 * sizeof(int), c->stream));
   LBM_CUDA(cudaMemsetAsync(b.nu, 0, n * sizeof(float), c->stream));
   LBM_CUDA(cudaMemsetAsync(b.done, 0, sizeof(unsigned), c->stream));
   lbm::adj_list(c->d, last + 14 * n, lists[0], counts, b.pos, c->stream);
@@ -1792,9 +1792,9 @@ int lbm_adjoint_coupled(lbm_ctx* c, int objective, int64_t nsteps, int32_t check
       A.lf0 = lf[1 - cur];
       A.lg0 = lg[1 - cur];
       A.next_list = lists[1 - cur];
-      A.next_count = counts + 2 * (1 - cur);
+      A.next_count = counts + 4 * (1 - cur);
       b.lamg = lg[cur];
-      lbm::adj_coupled_step(c->d, b, A, lists[cur], counts + 2 * cur, sweeps, sm);
+      lbm::adj_coupled_step(c->d, b, A, lists[cur], counts + 4 * cur, sweeps, sm);
       cur ^= 1;
     }
   };

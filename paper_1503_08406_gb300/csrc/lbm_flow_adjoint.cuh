@@ -437,14 +437,42 @@ struct CoupledStep {
   int* next_pos = nullptr;
 };
 
-// Put node s of colour c = (x + y) & 1 on a band list of n entries: colour 0 from
-// the front (count[0] of them), colour 1 from the back (count[1]).
-LBM_HD void band_append(int* list, int* count, int* pos, int n, int s, int c) {
+// The band by colour: no two neighbours share one, so that a colour's nodes update
+// in place in any order.  Colours 0 and 1 are those of a chessboard.  On a periodic
+// y axis of odd length row ny - 1 meets row 0 in its own colour: that row's nodes
+// take colours 2 and 3 in turn (x is never periodic here).
+LBM_HD int band_colour(int x, int y, int ny, int per_y) {
+  return per_y && (ny & 1) && y == ny - 1 ? 2 + (x & 1) : (x + y) & 1;
+}
+// A band list has n entries, as many as nodes, the last n - m of them for the
+// nodes of colours 2 and 3.
+LBM_HD int band_main(int nx, int ny, int per_y) {
+  return nx * ny - (per_y && (ny & 1) ? nx : 0);
+}
+// put node s of colour c on it: colours 0 and 2 from the front of their part (count[c]
+// of them), 1 and 3 from the back
+LBM_HD void band_append(int* list, int* count, int* pos, int n, int m, int s, int c) {
   const int i = hd_fetch_add(count + c, 1);
-  const int at = c ? n - 1 - i : i;
+  const int at = c == 0 ? i : c == 1 ? m - 1 - i : c == 2 ? m + i : n - 1 - i;
   list[at] = s;
   pos[s] = at;
 }
+// The band in order, colour by colour: those of colour 0 first, at 0 .. e1, then
+// colour 1 up to e2, and so on; e4 in all.
+struct BandOrder {
+  int n, m, e1, e2, e3, e4;
+  LBM_HD BandOrder(const int* count, int n_, int m_)
+      : n(n_), m(m_), e1(count[0]), e2(e1 + count[1]), e3(e2 + count[2]), e4(e3 + count[3]) {}
+  // the list entry of the j-th
+  LBM_HD int entry(int j) const {
+    return j < e1 ? j : j < e2 ? m - 1 - (j - e1) : j < e3 ? m + (j - e2) : n - 1 - (j - e3);
+  }
+  // which is at this entry (one in use)
+  LBM_HD int order(int at) const {
+    return at < e1 ? at : at < m ? e1 + (m - 1 - at) : at < m + (e3 - e2) ? e2 + (at - m)
+                                                                        : e3 + (n - 1 - at);
+  }
+};
 
 // the flux moments' rate at liquid fraction fl, and its derivative
 template <typename R>
@@ -606,7 +634,10 @@ LBM_HD void coupled_reverse_node(const CoupledStep<R>& A, int x, int y) {
   A.lfl[s] = lfl;
   const R fa = A.fl0[s];
   if (!wall && adj_mushy(fa)) {
-    if (A.next_pos) band_append(A.next_list, A.next_count, A.next_pos, (int)n, s, (x + y) & 1);
+    if (A.next_pos)
+      band_append(A.next_list, A.next_count, A.next_pos, (int)n,
+                  band_main(A.geo.nx, A.geo.ny, A.geo.per_y), s,
+                  band_colour(x, y, A.geo.ny, A.geo.per_y));
     else A.next_list[hd_fetch_add(A.next_count, 1)] = s;
   }
 }
