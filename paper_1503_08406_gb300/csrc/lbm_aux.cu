@@ -298,14 +298,18 @@ __global__ void __launch_bounds__(RB) reduce_kernel(Dev d, int layout, double* p
 }
 
 // Does this part of a split read-out (mode 0 all, 1 tiles away from the front,
-// 2 tiles near it, by the step of parity par just taken) take tile t?
+// 2 tiles near it, by the step of parity par just taken) take tile t?  (SEAM: on a
+// lattice with one)
+template <bool SEAM>
 __device__ __forceinline__ bool takes_part(const Dev& d, int mode, int par, int t) {
-  return mode == 0 || (mode == 2) == near_listed(d, t, par, d.ctr[par]);
+  return mode == 0 || (mode == 2) == (SEAM ? near_listed(d, t, par, d.ctr[par])
+                                           : near_beside(d, t, par, d.ctr[par]));
 }
 
 // The left-wall Nusselt number of the current state (the rows and the
 // formula of reduce_kernel), added to acc[0]; one block, fixed summation order.
 // Mode 1 leaves its rows' terms in rows[], where mode 2 finds them.
+template <bool SEAM>
 __global__ void __launch_bounds__(RB) wall_nusselt_kernel(Dev d, int layout, int mode, int par,
                                                           double* rows, double* acc) {
   __shared__ double sh[RB];
@@ -315,7 +319,7 @@ __global__ void __launch_bounds__(RB) wall_nusselt_kernel(Dev d, int layout, int
   if (d.wall_l && d.nx >= 3)
     for (int y = y0 + tid; y < y1; y += RB) {
       double r;
-      if (takes_part(d, mode, par, (y / TE) * d.etx)) {
+      if (takes_part<SEAM>(d, mode, par, (y / TE) * d.etx)) {
         const double T0 = node_T(d, 0, y, layout), T1 = node_T(d, 1, y, layout),
                      T2 = node_T(d, 2, y, layout);
         r = -(-3.0 * T0 + 4.0 * T1 - T2) * 0.5 * (double)d.H_over_dT;
@@ -410,6 +414,7 @@ __global__ void validate_kernel(Dev d, const float* phi, const float* K, const f
 // so one captured launch serves every replay of a graph.  mode and par as in
 // takes_part: the next step's stream-collide pass over the far tiles may start
 // once mode 1 is done with them.
+template <bool SEAM>
 __global__ void __launch_bounds__(256) keep_state_kernel(Dev d, int layout, int mode, int par,
                                                          float* base, unsigned* ctr) {
   const int n = (int)d.n, nx = d.nx;
@@ -418,7 +423,7 @@ __global__ void __launch_bounds__(256) keep_state_kernel(Dev d, int layout, int 
   float* dst = base + (ctr ? (long long)ctr[0] * 15 * n : 0LL);
   const int x = blockIdx.x * 32 + threadIdx.x;
   for (int yb = blockIdx.y * 8; yb < d.ny; yb += gridDim.y * 8) {
-    if (mode != 0 && !takes_part(d, mode, par, (yb / TE) * d.etx + (int)blockIdx.x)) continue;
+    if (mode != 0 && !takes_part<SEAM>(d, mode, par, (yb / TE) * d.etx + (int)blockIdx.x)) continue;
     const int y = yb + threadIdx.y;
     if (x >= nx || y >= d.ny) continue;
     const int s = y * nx + x;
@@ -530,7 +535,8 @@ void launch_reduce(const Dev& d, int layout, double* partials, double* out, int 
 }
 void launch_wall_nusselt(const Dev& d, int layout, int mode, int par, double* rows, double* acc,
                          cudaStream_t s) {
-  wall_nusselt_kernel<<<1, RB, 0, s>>>(d, layout, mode, par, rows, acc);
+  const auto kernel = d.seam ? wall_nusselt_kernel<true> : wall_nusselt_kernel<false>;
+  kernel<<<1, RB, 0, s>>>(d, layout, mode, par, rows, acc);
 }
 void launch_get_state(const Dev& d, int layout, float* f, float* g, cudaStream_t s) {
   get_state_kernel<<<grid1(d.n, 256), 256, 0, s>>>(d, layout, f, g);
@@ -542,7 +548,8 @@ void launch_keep_state(const Dev& d, int layout, float* base, unsigned* ctr, cud
                        int mode, int par) {
   const int nby = (d.ny + 7) / 8, most = 2432 / d.etx;   // about two waves of blocks
   const dim3 grid(d.etx, nby < most ? nby : most > 1 ? most : 1);
-  keep_state_kernel<<<grid, dim3(32, 8), 0, s>>>(d, layout, mode, par, base, ctr);
+  const auto kernel = d.seam ? keep_state_kernel<true> : keep_state_kernel<false>;
+  kernel<<<grid, dim3(32, 8), 0, s>>>(d, layout, mode, par, base, ctr);
 }
 void launch_nonfinite(const Dev& d, int nblocks, cudaStream_t s) {
   nonfinite_kernel<<<nblocks, 256, 0, s>>>(d);

@@ -71,15 +71,23 @@ __device__ __forceinline__ void fstore(S* p, float v, unsigned& rnd) {
 // COUNT_TILES tiles that is one store that nothing waits for: the solve kernel
 // counts the stamped tiles itself (an append to a list, a chain of three
 // memory round trips, ends a small lattice's pass 2 us later).  A larger one
-// appends to the step's list, and stamps the tiles around it in the near map, which costs its long pass nothing and spares every CTA of the solve
-// a walk over all the flags.
+// appends to the step's list, and stamps the tiles beside it in the near map, which
+// costs its long pass nothing and spares every CTA of the solve a walk over all the
+// flags.
 __device__ __forceinline__ void mark_tile(const Dev& d, int t, int par, int stamp) {
   int* fl = d.flags + par * d.ntiles + t;
   if (d.ntiles <= COUNT_TILES) {
     *fl = stamp;
   } else if (*fl != stamp && atomicExch(fl, stamp) != stamp) {
     d.list[par * d.ntiles + atomicAdd(&d.lcount[par], 1)] = t;
-    mark_near(d, t, par, stamp);
+    const int ty = t / d.etx, tx = t - ty * d.etx;
+    for (int k = 0; k < 9; ++k) {
+      int xx = tx + k % 3 - 1, yy = ty + k / 3 - 1;
+      if (d.per_x) xx = xx < 0 ? d.etx - 1 : xx >= d.etx ? 0 : xx;
+      if (d.per_y) yy = yy < 0 ? d.ety - 1 : yy >= d.ety ? 0 : yy;
+      if (xx >= 0 && xx < d.etx && yy >= 0 && yy < d.ety)
+        d.nearmap[par * d.ntiles + yy * d.etx + xx] = stamp;
+    }
   }
 }
 
@@ -538,12 +546,12 @@ __device__ __forceinline__ void step_prologue(const Dev& d) {
 }
 
 // Split steps: does this launch (MODE 1 far tiles, MODE 2 near tiles) take the
-// tile whose enthalpy tile is et?  Near: around a tile (near_place) that the
-// previous step (its stamp: prev) listed.
+// tile whose enthalpy tile is et?  Near: beside a tile that the previous step (its
+// stamp: prev) listed.
 template <int PAR, int MODE>
 __device__ __forceinline__ bool takes_tile(const Dev& d, int et, int prev) {
   if (MODE == 0) return true;
-  return (MODE == 2) == near_listed(d, et, 1 - PAR, prev);
+  return (MODE == 2) == near_beside(d, et, 1 - PAR, prev);
 }
 
 // ---- ordinary-load kernel ----------------------------------------------------
@@ -612,35 +620,37 @@ __device__ __forceinline__ void step_tile(const Dev& d, int x0, int y0, int prev
     mark_tile(d, (y / TE) * d.etx + x0 / TE, PAR, stamp);
 }
 
-// MODE as for launch_fused; 3: the near tiles, found from the previous step's list
+// MODE as for launch_fused; 3: the near tiles, found from the previous step's list;
+// 4 and 5: modes 1 and 2 of a lattice with a seam (instances of their own: asking
+// for it takes 0.3 of the far pass's 17 us at 1001 x 701)
 template <typename S, int PAR, int FLOW, int MODE>
 __global__ void __launch_bounds__(TX* TY, 4) fused_step_kernel(Dev d) {
   constexpr unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x;
+  constexpr bool SEAM = MODE >= 4, NEAR = MODE == 2 || MODE == 5;
   const int prev = d.ctr[1 - PAR], stamp = prev + 1;   // (no launch of this step changes it)
-  if (MODE != 1 && blockIdx.x == 0 && blockIdx.y == 0) {
-    if (MODE == 2) wait_for_previous();
+  if (MODE != 1 && MODE != 4 && blockIdx.x == 0 && blockIdx.y == 0) {
+    if (NEAR) wait_for_previous();
     if (lane == 0 && threadIdx.y == 0) step_prologue<PAR>(d);
   }
   if (MODE == 3) {
     const int cnt = d.lcount[2 + 1 - PAR];
-    const int places = near_places(d);
-    for (int u = blockIdx.x; u < 4 * places * cnt; u += gridDim.x) {
+    for (int u = blockIdx.x; u < 36 * cnt; u += gridDim.x) {
       int t, k, x0, y0;
-      if (!near_tile(d, u, cnt, places, 1 - PAR, t, k, x0, y0)) continue;
-      const unsigned at =
-          __ballot_sync(FULL, lane < places && listed_at(d, t, lane, 1 - PAR, prev));
-      if (__ffs(at) - 1 == near_inverse(k)) step_tile<S, PAR, FLOW>(d, x0, y0, prev, stamp);
+      if (!near_tile(d, u, cnt, 1 - PAR, t, k, x0, y0)) continue;
+      const unsigned at = __ballot_sync(FULL, lane < 9 && listed_beside(d, t, lane, 1 - PAR, prev));
+      if (__ffs(at) - 1 == 8 - k) step_tile<S, PAR, FLOW>(d, x0, y0, prev, stamp);
     }
     return;
   }
-  if (MODE != 0) {   // (one tile per CTA: a warp's first lanes look at its surroundings)
+  if (MODE != 0) {   // (one tile per CTA: a warp's first nine lanes look at its surroundings)
     const int et = ((blockIdx.y * TY) / TE) * d.etx + (blockIdx.x * TX) / TE;
-    const bool hit = d.ntiles > COUNT_TILES
-                         ? lane == 0 && d.nearmap[(1 - PAR) * d.ntiles + et] == prev
-                         : lane < near_places(d) && listed_at(d, et, lane, 1 - PAR, prev);
-    if ((MODE == 2) != __any_sync(FULL, hit)) return;
-    if (MODE == 2) wait_for_previous();
+    bool hit = d.ntiles > COUNT_TILES
+                   ? lane == 0 && d.nearmap[(1 - PAR) * d.ntiles + et] == prev
+                   : lane < 9 && listed_beside(d, et, lane, 1 - PAR, prev);
+    if (SEAM && lane >= 9 && lane < 16) hit = listed_at(d, et, lane, 1 - PAR, prev);
+    if (NEAR != __any_sync(FULL, hit)) return;
+    if (NEAR) wait_for_previous();
   }
   step_tile<S, PAR, FLOW>(d, blockIdx.x * TX, blockIdx.y * TY, prev, stamp);
 }
@@ -894,8 +904,7 @@ __device__ __forceinline__ void fused_tma_body(const Dev& d, const TmaMaps& m, i
   // runs of consecutive tiles per CTA).  The near-tile pass of a larger lattice
   // takes units of the previous step's list instead, 32 at a time.
   const bool listed = MODE == 2 && near_from_list(d);
-  constexpr int PLACES = 9;   // (walls on every side: no seam)
-  const int units = listed ? 4 * PLACES * d.lcount[2 + 1 - PAR] : ntile;
+  const int units = listed ? 36 * d.lcount[2 + 1 - PAR] : ntile;   // (walls around: no seam)
   // A far-tile pass takes nearly every tile: its first copies are issued before
   // it is known whether it takes them (a batch member first reads what to copy).
   // With the near pass from the list: 2048^2 103.3 -> 100.0 us a step, 4096 x
@@ -913,11 +922,11 @@ __device__ __forceinline__ void fused_tma_body(const Dev& d, const TmaMaps& m, i
       int et = 0, px = 0, py = 0;
       if (listed) {
         int k = 0;
-        take = near_tile(d, u, units / (4 * PLACES), PLACES, 1 - PAR, et, k, px, py);
+        take = near_tile(d, u, units / 36, 1 - PAR, et, k, px, py);
         if (take) {
           unsigned at = 0u;
 #pragma unroll
-          for (int j = 0; j < PLACES; ++j) at |= listed_at(d, et, j, 1 - PAR, prev) ? 1u << j : 0u;
+          for (int j = 0; j < 9; ++j) at |= listed_beside(d, et, j, 1 - PAR, prev) ? 1u << j : 0u;
           take = __ffs(at) - 1 == 8 - k;
         }
       } else if (take) {
@@ -1036,7 +1045,7 @@ static void launch_step_one(const Dev& d, cudaStream_t s) {
   const dim3 block(TX, TY);
   dim3 grid((d.nx + TX - 1) / TX, (d.ny + TY - 1) / TY);
   if (MODE == 3) grid = dim3(8 * d.egrid);
-  if (MODE == 2 && early_launches(d))
+  if ((MODE == 2 || MODE == 5) && early_launches(d))
     launch_early(fused_step_kernel<S, PAR, FLOW, MODE>, grid, block, 0, s, d);
   else fused_step_kernel<S, PAR, FLOW, MODE><<<grid, block, 0, s>>>(d);
 }
@@ -1089,7 +1098,9 @@ static void launch_fused_t(const Dev& d, const TmaMaps* m, int parity, int mode,
     return;
   }
   if (mode == 0) launch_mode<S, 0>(d, parity, s);
-  else if (mode == 1) launch_mode<S, 1>(d, parity, s);
+  else if (mode == 1 && !d.seam) launch_mode<S, 1>(d, parity, s);
+  else if (mode == 1) launch_mode<S, 4>(d, parity, s);
+  else if (d.seam) launch_mode<S, 5>(d, parity, s);
   else if (near_from_list_step(d)) launch_mode<S, 3>(d, parity, s);
   else launch_mode<S, 2>(d, parity, s);
 }

@@ -71,7 +71,6 @@ struct Dev {
   float H_over_dT;
   int etx, ety;              // enthalpy tiles
   int ntiles;                // etx * ety
-  int seam;                  // seam_axes: axes on which near tiles lie across a narrow last one
   int egrid, cgrid;          // CTAs of the enthalpy solve / commit kernels (they walk the tile list)
   int tgrid;                 // CTAs of the TMA-staged fused kernel
   int tslots;                // its CTAs resident at once (SMs x CTAs per SM)
@@ -92,7 +91,7 @@ struct Dev {
                              // next step's near-tile pass
   int* ctr;                  // [2]: step stamp per parity (the fused pass sets ctr[p] = ctr[1-p] + 1)
   int* nearmap;              // [2][ntiles], lattices of more than COUNT_TILES tiles: per parity,
-                             // the stamp of the step that listed a tile around this one (mark_near)
+                             // the stamp of the step that listed a tile beside this one (mark_tile)
   int* proc;                 // per enthalpy tile: (stamp << 3) | bits, bit 0 solved, bit 1
                              // some f_l changed, bit 2 some node's flow activity changed
   float2* scr;               // per node of solved tiles: (f_l(n), f_l(n+1))
@@ -110,6 +109,7 @@ struct Dev {
   long long* trace;
   unsigned* trace_n;
   unsigned trace_cap;
+  int seam;                  // seam_axes: axes on which near tiles lie across a narrow last one
   int* stats;                // [0] inner cap hit, [1] tiles solved, [2] max sweeps,
                              // [3] last tile that hit the cap, [4] a bounded wait gave up,
                              // [5] the sentinel found a non-finite value

@@ -42,104 +42,98 @@ LBM_HD int seam_axes(int nx, int ny, int per_x, int per_y) {
 // Places around a tile: 0..8 the 3 x 3 tiles row by row (4 the tile itself), and
 // with a seam 9..15 those across it: (across x, rows -1 0 1), (columns -1 0 1,
 // across y), (across both).
-template <typename D>
-LBM_HD int near_places(const D& d) {
-  return d.seam ? 16 : 9;
-}
-// the place of a seen from the tile at place k of a
-LBM_HD int near_inverse(int k) { return k < 9 ? 8 - k : k < 12 ? 20 - k : k < 15 ? 26 - k : k; }
-
 // tile a's counterpart across the narrow last one of `tiles` on an axis, or -1
 LBM_HD int tile_across(int a, int tiles) {
   return a == 0 ? tiles - 2 : a == tiles - 2 ? 0 : a == 1 ? tiles - 1 : a == tiles - 1 ? 1 : -1;
 }
 LBM_HD int tile_beside(int a, int o, int tiles, int per) {
   a += o;
-  if (a >= 0 && a < tiles) return a;
-  return !per ? -1 : a < 0 ? tiles - 1 : 0;
+  if (per) a = a < 0 ? tiles - 1 : a >= tiles ? 0 : a;
+  return a >= 0 && a < tiles ? a : -1;
 }
-// the tile at place k of tile t, or -1: places 0..8, and all places
-template <typename D>
-LBM_HD int beside_place(const D& d, int t, int k) {
-  const int ty = t / d.etx, tx = t - ty * d.etx;
-  const int xx = tile_beside(tx, k % 3 - 1, d.etx, d.per_x);
-  const int yy = tile_beside(ty, k / 3 - 1, d.ety, d.per_y);
-  return xx < 0 || yy < 0 ? -1 : yy * d.etx + xx;
-}
+// the tile at place k of tile t, or -1
 template <typename D>
 LBM_HD int near_place(const D& d, int t, int k) {
-  if (k < 9) return beside_place(d, t, k);
   const int ty = t / d.etx, tx = t - ty * d.etx;
-  const bool ax = k < 12 || k == 15, ay = k >= 12;
-  const int xx = !ax ? tile_beside(tx, k - 13, d.etx, d.per_x)
+  const bool ax = k >= 9 && (k < 12 || k == 15), ay = k >= 12;
+  const int ox = k < 9 ? k % 3 - 1 : k - 13, oy = k < 9 ? k / 3 - 1 : k - 10;
+  const int xx = !ax ? tile_beside(tx, ox, d.etx, d.per_x)
                      : d.seam & 1 ? tile_across(tx, d.etx) : -1;
-  const int yy = !ay ? tile_beside(ty, k - 10, d.ety, d.per_y)
+  const int yy = !ay ? tile_beside(ty, oy, d.ety, d.per_y)
                      : d.seam & 2 ? tile_across(ty, d.ety) : -1;
   return xx < 0 || yy < 0 ? -1 : yy * d.etx + xx;
 }
 
 // Was the tile at place k of tile t listed in the step of parity par with this
-// stamp?  (Any lattice.)
+// stamp?  (places 0..8; all)
+template <typename D>
+LBM_HD bool listed_beside(const D& d, int t, int k, int par, int stamp) {
+  const int ty = t / d.etx, tx = t - ty * d.etx;
+  int xx = tx + k % 3 - 1, yy = ty + k / 3 - 1;
+  if (d.per_x) xx = xx < 0 ? d.etx - 1 : xx >= d.etx ? 0 : xx;
+  if (d.per_y) yy = yy < 0 ? d.ety - 1 : yy >= d.ety ? 0 : yy;
+  if (xx < 0 || xx >= d.etx || yy < 0 || yy >= d.ety) return false;
+  return d.flags[par * d.ntiles + yy * d.etx + xx] == stamp;
+}
 template <typename D>
 LBM_HD bool listed_at(const D& d, int t, int k, int par, int stamp) {
   const int o = near_place(d, t, k);
   return o >= 0 && d.flags[par * d.ntiles + o] == stamp;
 }
-// Is tile t near, i.e. was a tile around it listed?  Nine independent loads on a
-// small lattice, where they wait once; one on a large one, whose CTAs are many
-// (2048^2: nine took 3% of the step) and whose marks keep a map of it.
+// Is tile t near, i.e. was a tile around it listed?  Places 0..8 are nine
+// independent loads on a small lattice, where they wait once, and one on a large
+// one, whose CTAs are many (2048^2: nine took 3% of the step) and whose marks keep a
+// map of it.  (A lattice with tensor maps is walled: no seam.)
 template <typename D>
-LBM_HD bool near_listed(const D& d, int t, int par, int stamp) {
+LBM_HD bool near_beside(const D& d, int t, int par, int stamp) {
   if (d.ntiles > COUNT_TILES) return d.nearmap[par * d.ntiles + t] == stamp;
   bool hit = false;
 #ifdef __CUDA_ARCH__
 #pragma unroll
 #endif
-  for (int k = 0; k < 9; ++k) hit |= listed_at(d, t, k, par, stamp);
+  for (int k = 0; k < 9; ++k) hit |= listed_beside(d, t, k, par, stamp);
+  return hit;
+}
+template <typename D>
+LBM_HD bool near_listed(const D& d, int t, int par, int stamp) {
+  bool hit = near_beside(d, t, par, stamp);
   if (d.seam)
     for (int k = 9; k < 16; ++k) hit |= listed_at(d, t, k, par, stamp);
   return hit;
 }
-// tile t was listed: stamp the tiles around it in the near map
-template <typename D>
-LBM_HD void mark_near(const D& d, int t, int par, int stamp) {
-  const int places = near_places(d);
-  for (int k = 0; k < places; ++k) {
-    const int o = near_place(d, t, k);
-    if (o >= 0) d.nearmap[par * d.ntiles + o] = stamp;
-  }
-}
 
 // Near-tile pass of a lattice whose step keeps a list (more tiles than CTAs in
 // the solve): its work is found from the list, not by asking every tile.  Unit u
-// of 4 x places a listed tile: one of the tiles around it and four 32x8 parts of
-// that, taken by the first listed tile, in the order of the places, around it.
+// of 36 a listed tile: one of the nine tiles around it and four 32x8 parts of
+// that, taken by the first listed tile (row by row) among the nine around it.
 // cnt: listed tiles of the step of parity par with this stamp.  (px, py): the
-// part's first node; k: the place it was reached by (taken if near_inverse(k) is
-// the first place of t that is listed).
+// part's first node; k: the place it was reached by (taken if 8 - k is the first
+// place of t that is listed).  Lattices without a seam only.
 template <typename D>
 LBM_HD bool near_from_list(const D& d) {
   return d.ntiles > d.egrid;
 }
 // The ordinary-load pass, one 32x8 tile per CTA, asks every tile as long as there
-// are few: at 768 x 640 (1920 of them) it ends 3 us sooner so.
+// are few: at 768 x 640 (1920 of them) it ends 3 us sooner so.  With a seam, too.
 template <typename D>
 LBM_HD bool near_from_list_step(const D& d) {
-  return near_from_list(d) &&
+  return near_from_list(d) && !d.seam &&
          (long long)((d.nx + TX - 1) / TX) * ((d.ny + TY - 1) / TY) > 8 * d.egrid;
 }
 template <typename D>
-LBM_HD bool near_tile(const D& d, int u, int cnt, int places, int par, int& t, int& k, int& px,
-                      int& py) {
-  if (u >= 4 * places * cnt) return false;
-  const int li = u / (4 * places), r = u - 4 * places * li;
+LBM_HD bool near_tile(const D& d, int u, int cnt, int par, int& t, int& k, int& px, int& py) {
+  if (u >= 36 * cnt) return false;
+  const int li = u / 36, r = u - 36 * li;
   k = r >> 2;
   const int l = d.list[par * d.ntiles + li];
-  t = places == 9 ? beside_place(d, l, k) : near_place(d, l, k);
-  if (t < 0) return false;
-  const int ty = t / d.etx;
-  px = (t - ty * d.etx) * TE;
-  py = ty * TE + TY * (r & 3);
+  const int ly = l / d.etx, lx = l - ly * d.etx;
+  int xx = lx + k % 3 - 1, yy = ly + k / 3 - 1;
+  if (d.per_x) xx = xx < 0 ? d.etx - 1 : xx >= d.etx ? 0 : xx;
+  if (d.per_y) yy = yy < 0 ? d.ety - 1 : yy >= d.ety ? 0 : yy;
+  if (xx < 0 || xx >= d.etx || yy < 0 || yy >= d.ety) return false;
+  t = yy * d.etx + xx;
+  px = xx * TE;
+  py = yy * TE + 8 * (r & 3);
   return py < d.ny;
 }
 

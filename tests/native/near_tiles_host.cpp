@@ -22,9 +22,9 @@ int wrap(int v, int n, int per) {
 
 // Lists `count` tiles (of the given seed; the whole row and column through one of
 // them too when `cross` is set) of an nx x ny lattice.  Returns 0 or what failed:
-// 1 a node of a listed tile's region in a tile not near, 2 near_listed and the near
-// map differ, 3 a part of a near tile not taken once, or one of a far tile taken,
-// 4 places not inverse to one another.
+// 1 a node of a listed tile's region in a tile not near, 2 near_listed
+// differs, 3 a part of a near tile not taken once, or one of a far tile taken, by
+// the near pass from the list (lattices without a seam).
 extern "C" int near_tiles_check(int nx, int ny, int per_x, int per_y, int count, int cross,
                                 int seed) {
   using namespace lbm;
@@ -49,22 +49,22 @@ extern "C" int near_tiles_check(int nx, int ny, int per_x, int per_y, int count,
   for (size_t i = order.size(); i > 1; --i) std::swap(order[i - 1], order[rand() % i]);
   for (int t : order) {
     flags[par * g.ntiles + t] = stamp;
-    mark_near(g, t, par, stamp);
+    for (int k = 0; k < 9; ++k)   // as mark_tile leaves it
+      if (near_place(g, t, k) >= 0) map[par * g.ntiles + near_place(g, t, k)] = stamp;
   }
   for (size_t i = 0; i < order.size(); ++i) list[par * g.ntiles + i] = order[i];
 
   // near by asking the flags (near_listed takes the map above COUNT_TILES)
-  const int places = near_places(g);
+  const int places = g.seam ? 16 : 9;
   std::vector<char> nr(g.ntiles, 0);
   for (int t = 0; t < g.ntiles; ++t)
     for (int k = 0; k < places; ++k) {
       nr[t] |= listed_at(g, t, k, par, stamp);
-      const int o = near_place(g, t, k);
-      if (o >= 0 && near_place(g, o, near_inverse(k)) != t) return 4;
+      if (k < 9 && listed_at(g, t, k, par, stamp) != listed_beside(g, t, k, par, stamp)) return 2;
     }
   for (int t = 0; t < g.ntiles; ++t)
     if (nr[t] != near_listed(g, t, par, stamp) ||
-        nr[t] != (map[par * g.ntiles + t] == stamp))
+        (!g.seam && nr[t] != near_beside(g, t, par, stamp)))
       return 2;
 
   for (int t : order) {
@@ -76,14 +76,16 @@ extern "C" int near_tiles_check(int nx, int ny, int per_x, int per_y, int count,
       }
   }
 
+  if (near_from_list_step(g) && g.seam) return 3;
+  if (g.seam) return 0;
   std::vector<int> taken(4 * g.ntiles, 0);
   const int cnt = (int)order.size();
-  for (int u = 0; u < 4 * places * cnt + 5; ++u) {
+  for (int u = 0; u < 36 * cnt + 5; ++u) {
     int t, k, px, py;
-    if (!near_tile(g, u, cnt, places, par, t, k, px, py)) continue;
+    if (!near_tile(g, u, cnt, par, t, k, px, py)) continue;
     unsigned at = 0u;
-    for (int j = 0; j < places; ++j) at |= listed_at(g, t, j, par, stamp) ? 1u << j : 0u;
-    if (ffs0(at) != near_inverse(k)) continue;
+    for (int j = 0; j < 9; ++j) at |= listed_beside(g, t, j, par, stamp) ? 1u << j : 0u;
+    if (ffs0(at) != 8 - k) continue;
     if (px != t % g.etx * TE || py / TE != t / g.etx || py >= ny || py % TY) return 3;
     ++taken[4 * t + py % TE / TY];
   }

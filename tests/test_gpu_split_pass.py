@@ -72,5 +72,5 @@ def test_narrow_last_tile_of_a_periodic_axis(P, nx, ny, cx, cy, flow):
 
 
 def test_narrow_last_tiles_of_a_mapped_lattice(P):
-    """1419 tiles: the near map, and the near-tile pass found from the list."""
+    """1419 tiles: the near map and the tiles across both edges."""
     _check_split(P, _strip_box(4099, 323, 2, 321))
