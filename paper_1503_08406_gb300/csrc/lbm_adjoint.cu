@@ -75,12 +75,11 @@ __device__ __forceinline__ bool band_node(const Dev& d, const float* f, int t) {
 }
 
 // the band of the state with liquid fraction f
-__global__ void adj_list_kernel(Dev d, const float* f, int* list, int* count, int* pos) {
+__global__ void adj_list_kernel(Dev d, const float* f, int* list, int* count, int* pos, int m) {
   const int s = blockIdx.x * AB + threadIdx.x;
   if (s >= (int)d.n) return;
   if (band_node(d, f, s))
-    band_append(list, count, pos, (int)d.n, band_main(d.nx, d.ny, d.per_y), s,
-                band_colour(s % d.nx, s / d.nx, d.ny, d.per_y));
+    band_append(list, count, pos, (int)d.n, m, s, band_colour(s % d.nx, s / d.nx, s, m));
 }
 
 // The fixed point's adjoint on the band: right-hand side
@@ -110,6 +109,26 @@ constexpr int BAND_THREADS = 1024;
 constexpr int BAND_CTAS = 64;
 constexpr int BAND_SMEM = BAND_CAP * (int)(sizeof(float4) + sizeof(ushort4) + 3 * sizeof(float));
 
+// sweep(lo, hi, omega) updates one colour's nodes and says whether one moved
+template <bool SEAM, typename F>
+__device__ __forceinline__ void band_sweeps(const BandOrder<SEAM>& o, int max_sweeps, F sweep) {
+  bool more = true;
+  for (int k = 0; k < max_sweeps && more; ++k) {
+    const float om = k < MU_SOR ? MU_OMEGA : 1.f;
+    int moved = sweep(0, o.e1, om);
+    __syncthreads();
+    moved |= sweep(o.e1, o.e2, om);
+    if (SEAM) {
+      __syncthreads();
+      moved |= sweep(o.e2, o.e3, om);
+      __syncthreads();
+      moved |= sweep(o.e3, o.e4, om);
+    }
+    more = __syncthreads_or(moved);
+  }
+}
+
+template <bool SEAM>
 __global__ void __launch_bounds__(BAND_THREADS, 1) adj_band_kernel(Dev d, AdjBuffers b,
                                                                 const float* f1, const int* list,
                                                                 const int* count,
@@ -121,8 +140,7 @@ __global__ void __launch_bounds__(BAND_THREADS, 1) adj_band_kernel(Dev d, AdjBuf
   // thread t of CTA k takes every BAND_CTAS-th node, so that a short band
   // spreads over all CTAs
   const int first = threadIdx.x * gridDim.x + blockIdx.x, step = gridDim.x * BAND_THREADS;
-  const int m = band_main(d.nx, d.ny, d.per_y);
-  const BandOrder now(count, n, m), old(old_count, n, m);
+  const BandOrder<SEAM> now(count, n, b.band_m), old(old_count, n, b.band_m);
   const int cnt = now.e4;
   for (int j = first; j < old.e4; j += step) b.nu[old_list[old.entry(j)]] = 0.f;
   for (int j = first; j < cnt; j += step) {
@@ -166,7 +184,6 @@ __global__ void __launch_bounds__(BAND_THREADS, 1) adj_band_kernel(Dev d, AdjBuf
   __syncthreads();
   if (!last) return;
   __threadfence();
-  const int colours = now.e4 > now.e2 ? 4 : 2;
   if (cnt <= BAND_CAP) {
     float4* ct = band_smem;
     ushort4* ix = reinterpret_cast<ushort4*>(ct + BAND_CAP);
@@ -183,59 +200,48 @@ __global__ void __launch_bounds__(BAND_THREADS, 1) adj_band_kernel(Dev d, AdjBuf
       mu[j] = 0.f;
     }
     __syncthreads();
-    bool more = true;
-    for (int k = 0; k < max_sweeps && more; ++k) {
-      const float om = k < MU_SOR ? MU_OMEGA : 1.f;
+    auto sweep = [&](int lo, int hi, float om) {
       int moved = 0;
-      for (int c0 = 0, lo = 0, hi = now.e1; c0 < colours; ++c0) {
-        for (int j = lo + threadIdx.x; j < hi; j += BAND_THREADS) {
-          const float4 c = ct[j];
-          const ushort4 q = ix[j];
-          const float nb = c.x * mu[q.x] + c.y * mu[q.y] + c.z * mu[q.z] + c.w * mu[q.w];
-          const float raw = rhs[j] - kk[j] * nb;
-          const float o = mu[j];
-          const float v = o + om * (raw - o);
-          moved |= fabsf(v - o) > MU_RTOL * fabsf(v);
-          mu[j] = v;
-        }
-        lo = hi;
-        hi = c0 == 0 ? now.e2 : c0 == 1 ? now.e3 : now.e4;
-        if (c0 + 1 < colours) __syncthreads();
+      for (int j = lo + threadIdx.x; j < hi; j += BAND_THREADS) {
+        const float4 c = ct[j];
+        const ushort4 q = ix[j];
+        const float nb = c.x * mu[q.x] + c.y * mu[q.y] + c.z * mu[q.z] + c.w * mu[q.w];
+        const float raw = rhs[j] - kk[j] * nb;
+        const float o = mu[j];
+        const float v = o + om * (raw - o);
+        moved |= fabsf(v - o) > MU_RTOL * fabsf(v);
+        mu[j] = v;
       }
-      more = __syncthreads_or(moved);
-    }
+      return moved;
+    };
+    band_sweeps(now, max_sweeps, sweep);
     for (int j = threadIdx.x; j < cnt; j += BAND_THREADS)
       b.nu[list[now.entry(j)]] = mu[j] / __ldcg(b.bk + j).z;
   } else {
     float* mu = b.mu;
     for (int j = threadIdx.x; j < cnt; j += BAND_THREADS) mu[j] = 0.f;
     __syncthreads();
-    bool more = true;
-    for (int k = 0; k < max_sweeps && more; ++k) {
-      const float om = k < MU_SOR ? MU_OMEGA : 1.f;
+    auto sweep = [&](int lo, int hi, float om) {
       int moved = 0;
-      for (int c0 = 0, lo = 0, hi = now.e1; c0 < colours; ++c0) {
-        for (int j = lo + threadIdx.x; j < hi; j += BAND_THREADS) {
-          const float4 c = __ldcg(b.bc + j), kj = __ldcg(b.bk + j);
-          const int4 q = __ldcg(b.bi + j);
-          const float nb = c.x * mu[q.x] + c.y * mu[q.y] + c.z * mu[q.z] + c.w * mu[q.w];
-          const float raw = kj.x - kj.y * nb;
-          const float o = mu[j];
-          const float v = o + om * (raw - o);
-          moved |= fabsf(v - o) > MU_RTOL * fabsf(v);
-          mu[j] = v;
-        }
-        lo = hi;
-        hi = c0 == 0 ? now.e2 : c0 == 1 ? now.e3 : now.e4;
-        if (c0 + 1 < colours) __syncthreads();
+      for (int j = lo + threadIdx.x; j < hi; j += BAND_THREADS) {
+        const float4 c = __ldcg(b.bc + j), kj = __ldcg(b.bk + j);
+        const int4 q = __ldcg(b.bi + j);
+        const float nb = c.x * mu[q.x] + c.y * mu[q.y] + c.z * mu[q.z] + c.w * mu[q.w];
+        const float raw = kj.x - kj.y * nb;
+        const float o = mu[j];
+        const float v = o + om * (raw - o);
+        moved |= fabsf(v - o) > MU_RTOL * fabsf(v);
+        mu[j] = v;
       }
-      more = __syncthreads_or(moved);
-    }
+      return moved;
+    };
+    band_sweeps(now, max_sweeps, sweep);
     for (int j = threadIdx.x; j < cnt; j += BAND_THREADS)
       b.nu[list[now.entry(j)]] = mu[j] / __ldcg(b.bk + j).z;
   }
   if (threadIdx.x == 0) {
-    old_count[0] = old_count[1] = old_count[2] = old_count[3] = 0;
+    old_count[0] = old_count[1] = 0;
+    if (SEAM) old_count[2] = old_count[3] = 0;
     *b.done = 0;
   }
 }
@@ -305,8 +311,7 @@ __global__ void __launch_bounds__(AB) adj_full_kernel(Dev d, AdjBuffers b, Mat5 
     b.lamf[s] = __ldg(b.a + s) * S;
     if (fb != fa) b.lama[s] += -(fb - fa) * S;   // (adds 0 elsewhere)
     if (adj_mushy(fa))
-      band_append(next_list, next_count, b.pos, n, band_main(d.nx, d.ny, d.per_y), s,
-                  band_colour(x, y, d.ny, d.per_y));
+      band_append(next_list, next_count, b.pos, n, b.band_m, s, band_colour(x, y, s, b.band_m));
   }
 }
 
@@ -410,21 +415,33 @@ __global__ void __launch_bounds__(128, 8) adj_coupled_kernel(CoupledStep<float> 
   for (int y = blockIdx.y; y < A.geo.ny; y += gridDim.y) coupled_reverse_node(A, x, y);
 }
 
+// (an odd periodic y axis, with its two further colours, has an instance of its own)
+static void launch_band(const Dev& d, const AdjBuffers& b, const float* f1, const int* list,
+                        const int* count, const int* old_list, int* old_count, int max_sweeps,
+                        cudaStream_t s) {
+  const auto kernel = b.band_m < (int)d.n ? adj_band_kernel<true> : adj_band_kernel<false>;
+  kernel<<<BAND_CTAS, BAND_THREADS, BAND_SMEM, s>>>(d, b, f1, list, count, old_list, old_count,
+                                                    max_sweeps);
+}
+
 void adj_coupled_step(const Dev& d, const AdjBuffers& b, const CoupledStep<float>& A, int* list,
                       int* count, int mu_sweeps, cudaStream_t s) {
-  adj_band_kernel<<<BAND_CTAS, BAND_THREADS, BAND_SMEM, s>>>(d, b, A.fl1, list, count, A.next_list,
-                                                             A.next_count, mu_sweeps);
+  launch_band(d, b, A.fl1, list, count, A.next_list, A.next_count, mu_sweeps, s);
   const dim3 grid((d.nx + 127) / 128, d.ny < 65535 ? d.ny : 65535);
   adj_coupled_kernel<<<grid, 128, 0, s>>>(A);
 }
 
 bool adj_init() {
-  return cudaFuncSetAttribute(adj_band_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              BAND_SMEM) == cudaSuccess;
+  for (auto kernel : {adj_band_kernel<false>, adj_band_kernel<true>})
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, BAND_SMEM) !=
+        cudaSuccess)
+      return false;
+  return true;
 }
 
-void adj_list(const Dev& d, const float* f, int* list, int* count, int* pos, cudaStream_t s) {
-  adj_list_kernel<<<blocks(d.n), AB, 0, s>>>(d, f, list, count, pos);
+void adj_list(const Dev& d, const AdjBuffers& b, const float* f, int* list, int* count,
+              cudaStream_t s) {
+  adj_list_kernel<<<blocks(d.n), AB, 0, s>>>(d, f, list, count, b.pos, b.band_m);
 }
 
 void adj_save(const Dev& d, float* base, unsigned* ctr, cudaStream_t s) {
@@ -436,8 +453,7 @@ void adj_save(const Dev& d, float* base, unsigned* ctr, cudaStream_t s) {
 void adj_step(const Dev& d, const AdjBuffers& b, const float* f0, const float* f1, int* list,
               int* count, int* old_list, int* old_count, int mu_sweeps, NuSrc nu,
               cudaStream_t s) {
-  adj_band_kernel<<<BAND_CTAS, BAND_THREADS, BAND_SMEM, s>>>(d, b, f1, list, count, old_list,
-                                                             old_count, mu_sweeps);
+  launch_band(d, b, f1, list, count, old_list, old_count, mu_sweeps, s);
   Mat5 At;
   for (int k = 0; k < 25; ++k) At.m[k] = b.At[k];
   const dim3 grid((d.nx + AB - 1) / AB, d.ny < 65535 ? d.ny : 65535);

@@ -21,6 +21,7 @@ struct AdjBuffers {
   float* lama;       // accumulated adjoint of a
   float* lamtw;      // ny: accumulated adjoint of the left wall profile
   int* pos;          // n: a band node's place in the band list (band_append)
+  int band_m;        // band_main of the lattice
   float At[25];      // transposed collision matrix (u = 0), passed to kernels by value
 };
 struct Mat5 {
@@ -51,7 +52,8 @@ void adj_mul(long long n, float* v, const float* w, cudaStream_t s);
 void adj_objective(const Dev& d, const float* fl, double* out, cudaStream_t s);
 // the band (non-wall nodes with 0 < f < 1) on a list of n entries, four counts
 // (band_append)
-void adj_list(const Dev& d, const float* f, int* list, int* count, int* pos, cudaStream_t s);
+void adj_list(const Dev& d, const AdjBuffers& b, const float* f, int* list, int* count,
+              cudaStream_t s);
 // d.fl to base + k n, k = ctr[0], which then advances (ctr[1]: scratch, 0)
 void adj_save(const Dev& d, float* base, unsigned* ctr, cudaStream_t s);
 // One step of the reverse sweep, given f_l before (f0) and after (f1) it and

@@ -1316,8 +1316,10 @@ struct DevMem {
 
 }  // namespace
 
-// the band solver's buffers (n nodes)
-static bool band_buffers(DevMem& mem, lbm::AdjBuffers& b, size_t n) {
+// the band solver's buffers
+static bool band_buffers(DevMem& mem, lbm::AdjBuffers& b, const lbm::Dev& d) {
+  const size_t n = (size_t)d.n;
+  b.band_m = lbm::band_main(d.nx, d.ny, d.per_y);
   b.bc = reinterpret_cast<float4*>(mem.get(4 * n));
   b.bi = reinterpret_cast<int4*>(mem.get(4 * n));
   b.bk = reinterpret_cast<float4*>(mem.get(4 * n));
@@ -1438,7 +1440,7 @@ int lbm_adjoint(lbm_ctx* c, int objective, int64_t nsteps, int32_t checkpoint_ev
   b.a = mem.get(n);
   b.lamg = mem.get(5 * n);
   b.lamf = mem.get(n);
-  const bool band = band_buffers(mem, b, n);
+  const bool band = band_buffers(mem, b, c->d);
   b.lamgpre = mem.get(5 * n);
   b.lama = mem.get(n);
   b.lamtw = mem.get((size_t)c->d.ny);
@@ -1528,7 +1530,7 @@ int lbm_adjoint(lbm_ctx* c, int objective, int64_t nsteps, int32_t checkpoint_ev
   LBM_CUDA(cudaMemsetAsync(counts, 0, 8 * sizeof(int), c->stream));
   LBM_CUDA(cudaMemsetAsync(b.nu, 0, n * sizeof(float), c->stream));
   LBM_CUDA(cudaMemsetAsync(b.done, 0, sizeof(unsigned), c->stream));
-  lbm::adj_list(c->d, fl_end, lists[0], counts, b.pos, c->stream);
+  lbm::adj_list(c->d, b, fl_end, lists[0], counts, c->stream);
   int cur = 0;
   // reversed steps m = hi - 1 .. lo, f_l of step m at F + (m - lo) n
   auto reverse = [&](cudaStream_t sm, const float* F, int64_t lo, int64_t hi) {
@@ -1671,7 +1673,7 @@ int lbm_adjoint_coupled(lbm_ctx* c, int objective, int64_t nsteps, int32_t check
   lbm::AdjBuffers b;
   b.a = mem.get(n);
   b.lamf = mem.get(n);
-  const bool band = band_buffers(mem, b, n);
+  const bool band = band_buffers(mem, b, c->d);
   b.lama = mem.get(n);   // adjoint of phi
   b.lamtw = mem.get((size_t)d.ny);
   b.pos = reinterpret_cast<int*>(mem.get(n));
@@ -1734,7 +1736,7 @@ int lbm_adjoint_coupled(lbm_ctx* c, int objective, int64_t nsteps, int32_t check
   LBM_CUDA(cudaMemsetAsync(counts, 0, 8 * sizeof(int), c->stream));
   LBM_CUDA(cudaMemsetAsync(b.nu, 0, n * sizeof(float), c->stream));
   LBM_CUDA(cudaMemsetAsync(b.done, 0, sizeof(unsigned), c->stream));
-  lbm::adj_list(c->d, last + 14 * n, lists[0], counts, b.pos, c->stream);
+  lbm::adj_list(c->d, b, last + 14 * n, lists[0], counts, c->stream);
   // the step's parameters
   lbm::CoupledStep<float> A;
   A.geo = lbm::CoupledGeo{d.nx, d.ny, d.per_x, d.per_y, {d.bc[0], d.bc[1], d.bc[2], d.bc[3]}};
@@ -1777,6 +1779,7 @@ int lbm_adjoint_coupled(lbm_ctx* c, int objective, int64_t nsteps, int32_t check
   A.lTw = b.lamtw;
   A.nu = b.nu;
   A.next_pos = b.pos;
+  A.band_m = b.band_m;
   // reverse sweep: step m of a stretch whose states sit at F (index m - lo)
   int cur = 0;
   auto reverse = [&](cudaStream_t sm, const float* F, int64_t lo, int64_t hi) {

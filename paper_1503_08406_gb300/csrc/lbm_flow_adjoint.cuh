@@ -432,23 +432,23 @@ struct CoupledStep {
   R *lphi, *lK, *lTw;                        // accumulated
   int *next_list, *next_count;               // band of the state before the step
   // optional: nu = c mu where lg1 does not hold it yet (0 off the band), and the
-  // band listed by colour (band_append): each node's place, and n list entries
+  // band listed by colour (band_append): each node's place, n list entries, and
+  // band_main of the lattice
   const R* nu = nullptr;
   int* next_pos = nullptr;
+  int band_m = 0;
 };
 
 // The band by colour: no two neighbours share one, so that a colour's nodes update
 // in place in any order.  Colours 0 and 1 are those of a chessboard.  On a periodic
-// y axis of odd length row ny - 1 meets row 0 in its own colour: that row's nodes
-// take colours 2 and 3 in turn (x is never periodic here).
-LBM_HD int band_colour(int x, int y, int ny, int per_y) {
-  return per_y && (ny & 1) && y == ny - 1 ? 2 + (x & 1) : (x + y) & 1;
-}
-// A band list has n entries, as many as nodes, the last n - m of them for the
-// nodes of colours 2 and 3.
+// y axis of odd length row ny - 1 meets row 0 in its own colour: that row's nodes,
+// those from m = band_main on, take colours 2 and 3 in turn (x is never periodic
+// here).  A band list has n entries, as many as nodes, the last n - m of them for
+// the nodes of colours 2 and 3.
 LBM_HD int band_main(int nx, int ny, int per_y) {
   return nx * ny - (per_y && (ny & 1) ? nx : 0);
 }
+LBM_HD int band_colour(int x, int y, int s, int m) { return s >= m ? 2 + (x & 1) : (x + y) & 1; }
 // put node s of colour c on it: colours 0 and 2 from the front of their part (count[c]
 // of them), 1 and 3 from the back
 LBM_HD void band_append(int* list, int* count, int* pos, int n, int m, int s, int c) {
@@ -458,17 +458,24 @@ LBM_HD void band_append(int* list, int* count, int* pos, int n, int m, int s, in
   pos[s] = at;
 }
 // The band in order, colour by colour: those of colour 0 first, at 0 .. e1, then
-// colour 1 up to e2, and so on; e4 in all.
+// colour 1 up to e2, and so on; e4 in all.  SEAM: with colours 2 and 3.
+template <bool SEAM>
 struct BandOrder {
   int n, m, e1, e2, e3, e4;
-  LBM_HD BandOrder(const int* count, int n_, int m_)
-      : n(n_), m(m_), e1(count[0]), e2(e1 + count[1]), e3(e2 + count[2]), e4(e3 + count[3]) {}
+  LBM_HD BandOrder(const int* count, int n_, int m_) : n(n_), m(m_) {
+    e1 = count[0];
+    e2 = e1 + count[1];
+    e3 = SEAM ? e2 + count[2] : e2;
+    e4 = SEAM ? e3 + count[3] : e2;
+  }
   // the list entry of the j-th
   LBM_HD int entry(int j) const {
+    if (!SEAM) return j < e1 ? j : n - 1 - (j - e1);
     return j < e1 ? j : j < e2 ? m - 1 - (j - e1) : j < e3 ? m + (j - e2) : n - 1 - (j - e3);
   }
   // which is at this entry (one in use)
   LBM_HD int order(int at) const {
+    if (!SEAM) return at < e1 ? at : e1 + (n - 1 - at);
     return at < e1 ? at : at < m ? e1 + (m - 1 - at) : at < m + (e3 - e2) ? e2 + (at - m)
                                                                         : e3 + (n - 1 - at);
   }
@@ -635,9 +642,8 @@ LBM_HD void coupled_reverse_node(const CoupledStep<R>& A, int x, int y) {
   const R fa = A.fl0[s];
   if (!wall && adj_mushy(fa)) {
     if (A.next_pos)
-      band_append(A.next_list, A.next_count, A.next_pos, (int)n,
-                  band_main(A.geo.nx, A.geo.ny, A.geo.per_y), s,
-                  band_colour(x, y, A.geo.ny, A.geo.per_y));
+      band_append(A.next_list, A.next_count, A.next_pos, (int)n, A.band_m, s,
+                  band_colour(x, y, s, A.band_m));
     else A.next_list[hd_fetch_add(A.next_count, 1)] = s;
   }
 }

@@ -6,15 +6,12 @@
 
 #include "lbm_flow_adjoint.cuh"
 
-// A random band (every node with probability percent / 100) of an nx x ny lattice,
-// listed in random order.  Returns 0, or what failed: 1 neighbours of one colour, 2
-// the list's places and the band's order not inverse, 3 a node missing or out of
-// its colour's range.
-extern "C" int band_order_check(int nx, int ny, int per_y, int percent, int seed) {
+template <bool SEAM>
+static int check(int nx, int ny, int per_y, int percent, int seed) {
   using namespace lbm;
   const int n = nx * ny, m = band_main(nx, ny, per_y);
   srand(seed);
-  auto colour = [&](int s) { return band_colour(s % nx, s / nx, ny, per_y); };
+  auto colour = [&](int s) { return band_colour(s % nx, s / nx, s, m); };
   for (int s = 0; s < n; ++s) {
     const int x = s % nx, y = s / nx;
     if (x + 1 < nx && colour(s) == colour(s + 1)) return 1;
@@ -28,7 +25,7 @@ extern "C" int band_order_check(int nx, int ny, int per_y, int percent, int seed
   std::vector<int> list(n, -1), pos(n, -1), seen(n, 0);
   int count[4] = {0, 0, 0, 0};
   for (int s : nodes) band_append(list.data(), count, pos.data(), n, m, s, colour(s));
-  const BandOrder o(count, n, m);
+  const BandOrder<SEAM> o(count, n, m);
   if (o.e4 != (int)nodes.size()) return 3;
   for (int j = 0; j < o.e4; ++j) {
     const int at = o.entry(j);
@@ -37,4 +34,13 @@ extern "C" int band_order_check(int nx, int ny, int per_y, int percent, int seed
     if (colour(list[at]) != c || seen[list[at]]++) return 3;
   }
   return 0;
+}
+
+// A random band (every node with probability percent / 100) of an nx x ny lattice,
+// listed in random order.  Returns 0, or what failed: 1 neighbours of one colour, 2
+// the list's places and the band's order not inverse, 3 a node missing or out of
+// its colour's range.
+extern "C" int band_order_check(int nx, int ny, int per_y, int percent, int seed) {
+  return lbm::band_main(nx, ny, per_y) < nx * ny ? check<true>(nx, ny, per_y, percent, seed)
+                                                 : check<false>(nx, ny, per_y, percent, seed);
 }
