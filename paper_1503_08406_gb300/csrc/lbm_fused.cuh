@@ -482,7 +482,8 @@ __device__ __forceinline__ bool node_update(const Dev& d, int x, int y, const Ge
 }
 
 // The update of a node of a warp that is liquid through and through (f_l = 1
-// exactly at every node and neighbour of the warp, none of them a wall node):
+// exactly at every node and neighbour of the warp, none of them a wall node, and
+// such nodes carry flow: f_act <= 1):
 // the same arithmetic on the same inputs, so the same bits, with f_l = 1 put in
 // and everything that asks about the neighbours left out.  Every store goes to
 // one plane's base (uniform over the warp) plus the node's offset.  For 16-bit
@@ -783,9 +784,9 @@ __device__ __forceinline__ bool tma_node(const Dev& d, const unsigned char* sb, 
       const int c = (ty + HY) * WX + (lane + HX);
       constexpr int PX = L::PX, PP = L::PX * L::PY;
       const int pc = PAR ? (ty + HY) * PX + (lane + L::HS) : ty * PX + lane;
-      if (FLOW && !EDGE && sizeof(S) == 2) {
-        // f_l = 1 in the warp's row and around it: each lane looks at its
-        // column, the outer lanes also at the one beyond
+      if (FLOW && !EDGE && sizeof(S) == 2 && (FLOW == 1 || d.f_act <= 1.f)) {
+        // f_l = 1 in the warp's row and around it (such nodes carry flow): each
+        // lane looks at its column, the outer lanes also at the one beyond
         const int e = c + (lane == 0 ? -1 : lane == TX - 1 ? 1 : 0);
         const bool liquid = sFL[c - WX] == 1.f && sFL[c] == 1.f && sFL[c + WX] == 1.f &&
                             sFL[e - WX] == 1.f && sFL[e] == 1.f && sFL[e + WX] == 1.f;
@@ -1038,8 +1039,12 @@ __global__ void __launch_bounds__(TX* TY, TMA_MIN_CTAS)
 
 // ---- launches ------------------------------------------------------------------
 
-// FLOW: 0 no flow lattice, 1 flow, 2 flow with extrapolated walls or front (a
-// variant of its own, which leaves the common one's registers alone)
+// FLOW: 0 no flow lattice, 1 flow, 2 flow with extrapolated walls or front, or
+// without flow at full melt (a variant of its own, which leaves the common one's
+// registers alone)
+static inline bool flow_extras(const Dev& d) {
+  return d.flow_front || d.flow_walls || !(d.f_act <= 1.f);
+}
 template <typename S, int PAR, int FLOW, int MODE>
 static void launch_step_one(const Dev& d, cudaStream_t s) {
   const dim3 block(TX, TY);
@@ -1052,7 +1057,7 @@ static void launch_step_one(const Dev& d, cudaStream_t s) {
 
 template <typename S, int MODE>
 static void launch_mode(const Dev& d, int parity, cudaStream_t s) {
-  if (d.flow && (d.flow_front || d.flow_walls)) {
+  if (d.flow && flow_extras(d)) {
     if (parity == 0) launch_step_one<S, 0, 2, MODE>(d, s);
     else launch_step_one<S, 1, 2, MODE>(d, s);
   } else if (d.flow) {
@@ -1076,7 +1081,7 @@ static void launch_tma_one(const Dev& d, const TmaMaps& m, cudaStream_t s) {
 
 template <typename S, int MODE>
 static void launch_tma_mode(const Dev& d, const TmaMaps& m, int parity, cudaStream_t s) {
-  if (d.flow && (d.flow_front || d.flow_walls)) {
+  if (d.flow && flow_extras(d)) {
     if (parity == 0) launch_tma_one<S, 0, 2, MODE>(d, m, s);
     else launch_tma_one<S, 1, 2, MODE>(d, m, s);
   } else if (d.flow) {
