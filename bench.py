@@ -49,7 +49,8 @@ BYTES_FLOW_NODE_16 = 68
 BYTES_SOLID_NODE_16 = 24
 KERNEL_SOURCES = ("paper_1503_08406_gb300/csrc/lbm_fused.cuh",
                   "paper_1503_08406_gb300/csrc/lbm_fused_f32.cu",
-                  "paper_1503_08406_gb300/csrc/lbm_internal.cuh")
+                  "paper_1503_08406_gb300/csrc/lbm_internal.cuh",
+                  "paper_1503_08406_gb300/csrc/lbm_tiles.cuh")
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "fused_tma_traffic_heterogeneous_cavity_2048.json")
 
 

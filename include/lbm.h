@@ -226,9 +226,10 @@ int lbm_autotune(lbm_ctx* c, int trial_steps, int32_t* variant, int32_t* tiles_p
  * for all steps (4 bytes per node and step) when that takes at most half the
  * free device memory, else as for sqrt(nsteps); checkpoint_every = K > 0: the
  * whole state kept every K steps and the steps between recomputed (a CUDA
- * graph per segment).  All choices give the same result.  Jacobi sweeps solve
- * the fixed point's adjoint per step until the largest change is within 4e-7
- * of the value, at most mu_sweeps (0: 64).  The context ends where the forward
+ * graph per segment).  All choices give the same result.  Gauss-Seidel sweeps
+ * (by colour, over-relaxed at first) solve the fixed point's adjoint per step
+ * until the largest change is within 4e-7 of the value, at most mu_sweeps (0:
+ * 64).  The context ends where the forward
  * run left it (nsteps further on).  Covers: no flow (flow = 0), periodic in y
  * with wall columns at x = 0 (Dirichlet, the profile) and x = nx - 1
  * (Dirichlet or adiabatic), FP32 storage, one thermal diffusivity;

@@ -19,9 +19,10 @@
 // nodes where 0 < z < 1 (elsewhere the clamp's derivative is 0): with
 // c = 1/(T_l - T_s + a) on those nodes and 0 elsewhere, the adjoint mu solves
 //   mu(y) = lam_f(y) + a(y) c(y) mu(y) - a(y) sum_i w~_i (c mu)(y + e_i),
-// solved here by Jacobi sweeps over those nodes only, with the self term exact
-// (a contraction: the row sums of the coupling are at most
-// 4 w~_1 a / (T_l - T_s + w~_0 a) <= 2/3).
+// solved here by over-relaxed red-black Gauss-Seidel sweeps over those nodes only,
+// with the self term exact (a contraction: the row sums of the coupling are at most
+// 4 w~_1 a / (T_l - T_s + w~_0 a) <= 2/3, so that any order of the nodes converges
+// for relaxation factors below 2 / (1 + 2/3) = 1.2).
 // At the fixed point z = f on those nodes, which removes the direct term of
 // d z / d a.
 #include "lbm_adjoint.cuh"
